@@ -1,0 +1,202 @@
+"""Workloads this library is measured on: what a serving or calibration program asks of it, through the public
+entry points of `paper_2607_04302_b200.binding`, from one 128-token head to 32768-token prefills.
+
+Three kinds of work:
+  attn       prefill attention.  entry "two": quantize_qkv, then attention_fwd (a program that also keeps the
+             packed 4-bit K/V); entry "raw": attention_fwd_raw, one call on raw Q/K/V.
+  quantize   quantize_qkv alone (filling a 4-bit cache; codes, metadata and operand images are kept).
+  calibrate  Smooth-QK factors from calibration activations; mode "auto" lets the applicability gate choose.
+
+With keep = True the program owns its buffers (quantized operands or workspace, output, status word) and passes
+them in, as a serving loop does; with keep = False it calls the plain form and takes what is returned."""
+import math
+
+import torch
+
+from paper_2607_04302_b200 import binding as hb
+
+_DTYPE = {"fp16": torch.float16, "bf16": torch.bfloat16}
+_CODE = {"fp16": hb.F16, "bf16": hb.BF16, "fp32": hb.F32}
+_MODE = {"strong": hb.MODE_STRONG, "mild": hb.MODE_MILD}
+_AGG = {"rms": hb.AGG_RMS, "mean": hb.AGG_MEAN, "p99": hb.AGG_P99}
+
+
+def _attn(B, Hq, Hkv, N, d, causal, dtype, out, smooth, gain, entry, keep, Bc=64, qmean=False):
+    return dict(kind="attn", B=B, Hq=Hq, Hkv=Hkv, N=N, d=d, causal=causal, dtype=dtype, out=out, smooth=smooth,
+                gain=gain, entry=entry, keep=keep, Bc=Bc, qmean=qmean)
+
+
+def _quantize(B, Hq, Hkv, N, d, dtype, smooth, gain):
+    return dict(kind="quantize", B=B, Hq=Hq, Hkv=Hkv, N=N, d=d, dtype=dtype, smooth=smooth, gain=gain)
+
+
+def _calibrate(S, Hq, Hkv, N, d, dtype, mode, agg, gain):
+    return dict(kind="calibrate", S=S, Hq=Hq, Hkv=Hkv, N=N, d=d, dtype=dtype, mode=mode, agg=agg, gain=gain)
+
+
+def listed():
+    cases = {
+        # the smallest call: one head, 128 tokens, FP16, plain call without buffers of one's own (latency, launches)
+        "tiny-1head-128": _attn(1, 1, 1, 128, 128, False, "fp16", "fp32", "strong", 20.0, "raw", False),
+        # a short ragged prompt (31 key tiles, the last query block half empty) of a small d = 64 model in FP16
+        "d64-ragged-1984": _attn(1, 12, 4, 1984, 64, True, "fp16", "fp16", "strong", 20.0, "raw", True),
+        # a batch of four ordinary 1K prompts of a GQA 32/8 model
+        "batch4-1k-causal": _attn(4, 32, 8, 1024, 128, True, "bf16", "bf16", "strong", 20.0, "raw", True),
+        # Qwen3-8B-shaped 4K prefill, quantized operands kept: the repository's headline step
+        "qwen3-4k-causal": _attn(1, 32, 8, 4096, 128, True, "bf16", "fp32", "strong", 20.0, "two", True),
+        # the same with the Q-Mean auxiliary
+        "qwen3-4k-qmean": _attn(1, 32, 8, 4096, 128, True, "bf16", "bf16", "strong", 20.0, "two", True, qmean=True),
+        # the same with 128-key tiles (the tile width is part of the result, so a program that pinned it stays there)
+        "qwen3-4k-bc128": _attn(1, 32, 8, 4096, 128, True, "bf16", "bf16", "strong", 20.0, "two", True, Bc=128),
+        # LLaMA3.1-8B-shaped 8K prefill, no outliers, smoothing bypassed, one call
+        "llama31-8k-causal": _attn(1, 32, 8, 8192, 128, True, "bf16", "fp16", "none", 1.0, "raw", True),
+        # Gemma2-9B-shaped 8K prefill, d = 256, mild smoothing
+        "gemma2-8k-d256": _attn(1, 16, 8, 8192, 256, True, "bf16", "bf16", "mild", 8.0, "two", True),
+        # non-causal (encoder-style) batch: every item equally heavy
+        "batch4-4k-full": _attn(4, 32, 8, 4096, 128, False, "bf16", "bf16", "strong", 20.0, "raw", True),
+        # the longest prompt of the sweep
+        "long-32k-causal": _attn(1, 32, 8, 32768, 128, True, "bf16", "bf16", "strong", 20.0, "raw", True),
+        # filling a 4-bit cache with an 8K prompt: bit-exact bytes
+        "quantize-8k": _quantize(1, 32, 8, 8192, 128, "bf16", "strong", 20.0),
+        # offline calibration of one layer: 32 sequences of 1024 tokens, the gate decides
+        "calibrate-32x1k": _calibrate(32, 32, 8, 1024, 128, "bf16", "auto", "rms", 20.0),
+    }
+    return [dict(c, name=n) for n, c in cases.items()]
+
+
+_HEADS = [(1, 1), (4, 1), (8, 8), (12, 4), (14, 2), (16, 8), (28, 4), (32, 8), (40, 8)]
+
+
+def _log_int(rng, lo, hi, step):
+    return max(lo, int(round(math.exp(rng.uniform(math.log(lo), math.log(hi))) / step)) * step)
+
+
+def _scores(c):
+    """Query-key pairs, weighted by what a pair costs next to the d = 128, 64-key-tile form."""
+    weight = 2.0 if c["d"] == 256 else 1.0
+    if c["Bc"] == 128:
+        weight *= 1.5 if c["d"] == 128 else 8.0
+    return c["B"] * c["Hq"] * c["N"] * c["N"] * (0.5 if c["causal"] else 1.0) * weight
+
+
+def draw(rng):
+    kind = rng.choice(["attn"] * 6 + ["quantize", "calibrate"])
+    Hq, Hkv = rng.choice(_HEADS)
+    dtype = rng.choice(["bf16", "bf16", "fp16"])
+    smooth = rng.choice(["strong", "strong", "mild", "none"])
+    gain = 1.0 if smooth == "none" else rng.choice([8.0, 20.0])
+    d = rng.choice([64, 128, 128, 128, 256])
+    if kind == "calibrate":
+        while True:
+            S, N = rng.randint(1, 48), _log_int(rng, 65, 2048, 1)
+            if S * Hq * N * d <= 1.4e8:
+                return _calibrate(S, Hq, Hkv, N, d, dtype, rng.choice(["auto", "strong", "mild"]),
+                                  rng.choice(["rms", "rms", "mean", "p99"]), gain)
+    B, N = rng.choice([1, 1, 2, 3, 4, 8]), _log_int(rng, 64, 32768, 64)
+    if kind == "quantize":
+        while B * Hq * N * d > 1.4e8:
+            N = _log_int(rng, 64, N, 64)
+        return _quantize(B, Hq, Hkv, N, d, dtype, smooth, gain)
+    option = rng.choice(["", "", "", "", "qmean", "bc128"])
+    c = _attn(B, Hq, Hkv, N, d, rng.random() < 0.7, dtype, rng.choice(["fp16", "bf16", "fp32"]), smooth, gain,
+              rng.choice(["two", "raw"]), rng.random() < 0.8, Bc=128 if option == "bc128" and d != 256 else 64,
+              qmean=option == "qmean")
+    while _scores(c) > 1.5e10:
+        c["N"] = _log_int(rng, 64, c["N"], 64)
+    return c
+
+
+def _normal(gen, shape, dtype):
+    return torch.randn(shape, generator=gen, dtype=torch.float32, device="cuda").to(dtype)
+
+
+def _add_outliers(k, gen, gain):
+    """Scale 1 in 32 channels of every KV head of k [.., Hkv, N, d]: the K outlier stripe of post-RoPE activations."""
+    if gain == 1.0:
+        return k
+    Hkv, d = k.shape[-3], k.shape[-1]
+    pick = torch.rand((Hkv, d), generator=gen, device="cuda").argsort(dim=1)[:, : max(1, d // 32)]
+    f = torch.ones((Hkv, d), dtype=torch.float32, device="cuda").scatter_(1, pick, gain)
+    return k.mul_(f[:, None, :].to(k.dtype))
+
+
+def prepare(case, seed):
+    gen = torch.Generator(device="cuda").manual_seed(int(seed))
+    c, dt = case, _DTYPE[case["dtype"]]
+    if c["kind"] == "calibrate":
+        q = _normal(gen, (c["S"], c["Hq"], c["N"], c["d"]), dt)
+        k = _add_outliers(_normal(gen, (c["S"], c["Hkv"], c["N"], c["d"]), dt), gen, c["gain"])
+        return dict(case=c, q=q, k=k)
+    B, Hq, Hkv, N, d = c["B"], c["Hq"], c["Hkv"], c["N"], c["d"]
+    state = dict(case=c, q=_normal(gen, (B, Hq, N, d), dt), k=_normal(gen, (B, Hkv, N, d), dt),
+                 v=_normal(gen, (B, Hkv, N, d), dt), s=None, inv_s=None, status=None, out=None, qkv=None, ws=None)
+    mark = gen.get_state()
+    _add_outliers(state["k"], gen, c["gain"])
+    if c["smooth"] != "none":                      # factors from a calibration set with the same outlier channels
+        cal = torch.Generator(device="cuda").manual_seed(int(seed) + 1)
+        q_cal, k_cal = _normal(cal, (2, Hq, 128, d), dt), _normal(cal, (2, Hkv, 128, d), dt)
+        gen.set_state(mark)
+        _add_outliers(k_cal, gen, c["gain"])
+        state["s"], state["inv_s"] = hb.smooth_calibrate(q_cal, k_cal, _MODE[c["smooth"]])
+    in_dt = _CODE[c["dtype"]]
+    if c["kind"] == "quantize":
+        state["qkv"] = hb.alloc_qkv(B, Hq, Hkv, N, d, in_dt, "cuda")
+    elif c["keep"]:
+        state["status"] = torch.zeros(1, dtype=torch.int32, device="cuda")
+        state["out"] = torch.empty((B, Hq, N, d), dtype={"fp32": torch.float32, **_DTYPE}[c["out"]], device="cuda")
+        if c["entry"] == "two":
+            state["qkv"] = hb.alloc_qkv(B, Hq, Hkv, N, d, in_dt, "cuda", qmean=c["qmean"])
+        else:
+            need = hb.attention_raw_workspace_bytes(B, Hq, Hkv, N, d, in_dt, c["causal"], c["Bc"], _CODE[c["out"]],
+                                                    qmean=c["qmean"])
+            state["ws"] = torch.empty(need, dtype=torch.uint8, device="cuda")
+    return state
+
+
+def run(state):
+    c = state["case"]
+    if c["kind"] == "calibrate":
+        if c["mode"] == "auto":
+            s, inv_s, stats = hb.smooth_calibrate_auto(state["q"], state["k"])
+            return dict(s=s, inv_s=inv_s, stats=stats)
+        s, inv_s = hb.smooth_calibrate(state["q"], state["k"], _MODE[c["mode"]], aggregator=_AGG[c["agg"]])
+        return dict(s=s, inv_s=inv_s)
+    q, k, v, s, inv_s = (state[n] for n in ("q", "k", "v", "s", "inv_s"))
+    if c["kind"] == "quantize":
+        x = hb.quantize_qkv(q, k, v, s, inv_s, out=state["qkv"])
+        return {n: getattr(x, n) for n in ("q_codes", "q_meta", "q_mma", "k_codes", "k_meta", "k_mma",
+                                           "v_codes", "v_meta", "v_mma")}
+    if c["entry"] == "raw":
+        out = hb.attention_fwd_raw(q, k, v, s, inv_s, c["causal"], Bc=c["Bc"], out_dtype=_CODE[c["out"]],
+                                   out=state["out"], workspace=state["ws"], d_status=state["status"], qmean=c["qmean"])
+        return dict(out=out)
+    x = hb.quantize_qkv(q, k, v, s, inv_s, out=state["qkv"], d_status=state["status"], qmean=c["qmean"])
+    out = hb.attention_fwd(x, c["causal"], Bc=c["Bc"], out_dtype=_CODE[c["out"]], out=state["out"],
+                           d_status=state["status"], qmean=c["qmean"])
+    return dict(out=out, k_codes=x.k_codes, k_meta=x.k_meta, v_codes=x.v_codes, v_meta=x.v_meta)
+
+
+def work(case):
+    c = case
+    if c["kind"] == "calibrate":                   # every activation read once; the factors written
+        n = c["S"] * (c["Hq"] + c["Hkv"]) * c["N"] * c["d"]
+        return dict(bytes=2 * n + 8 * c["Hkv"] * c["d"], flops=n)
+    n_in = c["B"] * (c["Hq"] + 2 * c["Hkv"]) * c["N"] * c["d"]
+    if c["kind"] == "quantize":                    # 16-bit in; 4.5-bit HIF4 and its 16-bit operand image out
+        return dict(bytes=n_in * (2 + 0.5625 + 2), flops=4 * n_in)
+    n_out = c["B"] * c["Hq"] * c["N"] * c["d"]
+    packed = c["B"] * 2 * c["Hkv"] * c["N"] * c["d"] * 0.5625 if c["entry"] == "two" else 0
+    pairs = c["B"] * c["Hq"] * (c["N"] * (c["N"] + 1) / 2 if c["causal"] else c["N"] * c["N"])
+    return dict(bytes=2 * n_in + packed + n_out * (4 if c["out"] == "fp32" else 2), flops=4 * pairs * c["d"])
+
+
+def tolerance(case):
+    if case["kind"] == "quantize":
+        return "exact"                             # codes, metadata and images are integers and exact values
+    if case["kind"] == "calibrate":
+        return dict(rel=1e-6, max=1e-5)            # pow in double, rounded once to FP32
+    # The sums are not what limits the agreement: tensor-core products in another order gave the same bits at every
+    # listed size.  Exponentials that differ in their last FP32 bit flip an element of P-hat in 1e5 to 1e6, which moves
+    # O by 2e-4 to 9e-4 in the 2-norm (keeping P in FP32 flips 100 times as many: 2.4e-3 to 9e-3) and single
+    # peaked rows by up to half the root mean square.
+    return dict(rel=1e-3, max=0.5)
