@@ -196,7 +196,7 @@ def tolerance(case):
     if case["kind"] == "calibrate":
         return dict(rel=1e-6, max=1e-5)            # pow in double, rounded once to FP32
     # The sums are not what limits the agreement: tensor-core products in another order gave the same bits at every
-    # listed size.  Exponentials that differ in their last FP32 bit flip an element of P-hat in 1e5 to 1e6, which moves
-    # O by 2e-4 to 9e-4 in the 2-norm (keeping P in FP32 flips 100 times as many: 2.4e-3 to 9e-3) and single
-    # peaked rows by up to half the root mean square.
+    # listed size.  What moves is P-hat: keeping P in FP32 instead of FP16 flips a few of 1e4 elements and moves O by
+    # 2.4e-3 to 9e-3 in the 2-norm (measured).  Exponentials that differ in their last FP32 bit flip about a hundredth
+    # of that, so a tenth of the distance; a single peaked row can move by up to half the root mean square.
     return dict(rel=1e-3, max=0.5)
