@@ -2,6 +2,7 @@
 // of P and the host-side TMA descriptor helper.
 #pragma once
 #include <cuda.h>
+#include <type_traits>
 
 #include "hifa4_internal.h"
 #include "hifa4_device.cuh"
@@ -67,19 +68,6 @@ struct Cfg {
 };
 
 __device__ __forceinline__ float f16_round(float x) { return __half2float(__float2half_rn(x)); }
-
-// exp2 of two values, each result rounded to FP16 (one packed conversion) and widened back.
-__device__ __forceinline__ void exp2_f16_pair(float t0, float t1, float& e0, float& e1)
-{
-    const float a = ex2_approx(t0), b = ex2_approx(t1);
-    uint32_t h2;
-    asm("cvt.rn.f16x2.f32 %0, %1, %2;" : "=r"(h2) : "f"(b), "f"(a));     // a -> low half, b -> high half
-    asm("{\n\t.reg .b16 lo, hi;\n\t"
-        "mov.b32 {lo, hi}, %2;\n\t"
-        "cvt.f32.f16 %0, lo;\n\t"
-        "cvt.f32.f16 %1, hi;\n\t}"
-        : "=f"(e0), "=f"(e1) : "r"(h2));
-}
 
 // Quantize NU*8 consecutive softmax weights of one 64-key HIF4 group (already rounded to FP16,
 // held as floats, all >= 0) and return the BF16 image of P-hat as NU*4 packed words (element 2i
@@ -160,109 +148,190 @@ __device__ __forceinline__ float p_of_score(float acc, float c1, float mL)
     return PF32 ? e : f16_round(e);                    // PF32: the variant that keeps P in FP32
 }
 
-// Arithmetic of the fused form (all exact except the exponential itself):
-//   q = RZ(p * (4/S))            group-constant multiplier; exactly j + 1/2 (in units of the finest
-//                                step S/4) on every rounding tie (see e6m2_inv4)
-//   y = q + 1.5 * 2^(23+k)       rounds q to the nearest multiple of 2^k, ties to the even multiple:
-//                                y - magic = m * 2^k with m the element code under shift k
-//   v = fma(y, S/4, -magic*S/4)  = m * 2^k * S/4, the dequantized value, no rounding
-// The shift k of a 4-key subgroup with maximum At is read off float bit patterns:
-//   need = max(bits(At) - bits(1.75 S) - 1 + 2^23, 0) >> 23   (0, 1 or 2)
-// (the shifts of the two subgroups of a level-2 unit are then combined by exp_quantize_units).
-// Multiplications, additions and FMAs run two elements at a time (f32x2).
-struct PQuantConst {              // per (row, 64-key group, tile) constants of the fused quantizer
+// Arithmetic of the fused form.  P is FP16, so the quantizer runs on packed FP16 pairs from the conversion on and
+// hands over a packed BF16 image: no widening back to FP32, no repacking.  The softmax warps are bound by instruction
+// issue: 13.9 executed warp instructions per score (polls included) instead of the 15.8 of the FP32 form, and the
+// attention of 32 / 8 heads at d = 128, causal, takes 178 instead of 187 us at N = 4096, 2.04 instead of 2.16 ms at
+// N = 16384 (B200, CUDA events).  In units of S/2:
+//   q = RN(p * (2/S) 2^-s)          2/S = hi + lo in two FP16 constants (the mantissas 4/(4+M) repeat with a period
+//                                   that divides 12, so one FP16 constant errs by 2^-12, which is not enough):
+//                                   q = fma(p, hi, RN(p * lo)).  Exactly on every rounding tie and on the right side
+//                                   of it everywhere else
+//   y = q + 1.5 * 2^(9+k) 2^-s      rounds q to the nearest multiple of the subgroup's step, ties to even;
+//                                   the low bits of y are the element code m
+//   v = fma_bf16(y, c, -n)          the bit pattern of y read as BF16 is 2^E (1 + m/128) with E known from k and s, so
+//                                   one BF16 FMA with c = step * 128 * 2^-E, n = step * 128 gives m * step exactly
+// s is 0 or 12: it keeps 2/S finite in FP16 for groups whose maximum is below 2^-12.  The shift k of a 4-key subgroup
+// is read off the bit pattern of its largest q: need = number of thresholds 3.5, 7 (1.75 S, 3.5 S) exceeded, then
+// k_t = max(need_t, need_other - 1) (that is the pair rule: the level-2 bit is set iff max(need) = 2 or min(need) >= 1,
+// and a subgroup that needs no shift of its own still gets one when its partner needs two); the two subgroups of a unit
+// share packed 16-bit integer operations.  tests/test_p_quantizer_arithmetic.py checks the scheme on every FP16 P, every
+// scale code and every shift.
+// The FP32-P variant keeps the FP32 form of the same scheme: q = RZ(p * (4/S)) (exactly on ties, see e6m2_inv4),
+// y = q + 1.5 * 2^(23+k), v = fma(y, S/4, -magic*S/4), two elements per f32x2 operation.
+template <bool PF32> struct PQuantConst;        // per (row, 64-key group, tile) constants of the fused quantizer
+template <> struct PQuantConst<true> {
     uint64_t c1c1, nml, inv44, s44;
     uint32_t c0_bits, s4_bits;
     int tadd;
 };
+template <> struct PQuantConst<false> {
+    uint64_t c1c1, nml;
+    uint32_t hi, lo, tadd, magic, c, n;          // packed pairs of equal halves
+    uint32_t s4_bits;                            // P-hat dump only
+};
 
-// Constants from the group maximum A of P.  A = 0 (every key masked) needs no branch: the scale
-// code clamps to 0, every p is 0 and every product below is an exact zero.
-__device__ __forceinline__ PQuantConst p_quant_const(float c1, float mL, float A)
+// Constants from the group maximum A of P.  A = 0 (every key masked) needs no branch: the scale stays finite, every p
+// is 0 and every product below is an exact zero.
+template <bool PF32>
+__device__ __forceinline__ PQuantConst<PF32> p_quant_const(float c1, float mL, float A)
 {
-    PQuantConst k;
-    const int code = e6m2_code_for_max(A);
-    const float S = e6m2_value(code);
-    const float inv4 = e6m2_inv4(code);
-    const float S4 = __uint_as_float(__float_as_uint(S) - (2u << 23));     // S / 4
-    k.tadd = (1 << 23) - ((int)__float_as_uint(1.75f * S) + 1);
-    k.c0_bits = __float_as_uint(-12582912.f * S4);                         // -1.5 * 2^23 * S/4
-    k.s4_bits = __float_as_uint(S4);
+    PQuantConst<PF32> k;
     k.c1c1 = pack2(c1, c1);
     k.nml = pack2(-mL, -mL);
-    k.inv44 = pack2(inv4, inv4);
-    k.s44 = pack2(S4, S4);
+    if constexpr (PF32) {
+        const int code = e6m2_code_for_max(A);
+        const float S = e6m2_value(code);
+        const float inv4 = e6m2_inv4(code);
+        const float S4 = __uint_as_float(__float_as_uint(S) - (2u << 23)); // S / 4
+        k.tadd = (1 << 23) - ((int)__float_as_uint(1.75f * S) + 1);
+        k.c0_bits = __float_as_uint(-12582912.f * S4);                     // -1.5 * 2^23 * S/4
+        k.s4_bits = __float_as_uint(S4);
+        k.inv44 = pack2(inv4, inv4);
+        k.s44 = pack2(S4, S4);
+    } else {
+        const bool small = A < 0x1p-12f;
+        const int code = e6m2_code_for_max(fmaxf(A, 0x1p-24f));
+        const int e = code >> 2, M = code & 3;
+        const uint32_t sel = 0x1010u + 0x2222u * (uint32_t)M;              // both halves = entry M of a table of four
+        const uint32_t sh = (uint32_t)((small ? 37 : 49) - e) * 0x04000400u;
+        const uint32_t top = (small ? 12u : 0u) * 0x04000400u;
+        k.hi = __byte_perm(0x3A663C00u, 0x38923955u, sel) + sh;            // RN16(4/(4+M)) * 2^(49-e-s)
+        k.lo = M ? k.hi - 0x30003000u : 0u;                                // hi * 2^-12
+        k.tadd = 0xC0FFC0FFu + top;                                        // 1023 - bits(3.5 * 2^-s), per half
+        k.magic = 0x62006200u - top;                                       // 768 * 2^-s
+        const uint32_t m5 = (uint32_t)M << 5;
+        k.c = (((uint32_t)(e + (small ? 111 : 15)) << 7) | m5) * 0x00010001u;
+        k.n = (0x8000u | ((uint32_t)(e + 84) << 7) | m5) * 0x00010001u;
+        k.s4_bits = ((uint32_t)((code >> 2) + 77) << 23) | ((uint32_t)M << 21);
+    }
     return k;
 }
 
-// P = exp2(acc * c1 - mL) rounded to FP16 (PF32: left in FP32) for the 8 keys of unit u.
-template <int NU, bool PF32 = false>
-__device__ __forceinline__ void exp_unit(const float (&acc)[NU * 8], int u, const PQuantConst& k, float (&p)[8])
+// P = exp2(acc * c1 - mL) for the 8 keys of unit u: FP16 pairs in natural order, or FP32 values (PF32).
+template <int NU>
+__device__ __forceinline__ void exp_unit(const float (&acc)[NU * 8], int u, const PQuantConst<false>& k, uint32_t (&p)[4])
+{
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        float t0, t1;
+        unpack2(fma2(pack2(acc[8 * u + 2 * i], acc[8 * u + 2 * i + 1]), k.c1c1, k.nml), t0, t1);
+        asm("cvt.rn.f16x2.f32 %0, %1, %2;" : "=r"(p[i]) : "f"(ex2_approx(t1)), "f"(ex2_approx(t0)));
+    }
+}
+template <int NU>
+__device__ __forceinline__ void exp_unit(const float (&acc)[NU * 8], int u, const PQuantConst<true>& k, float (&p)[8])
 {
 #pragma unroll
     for (int i = 0; i < 8; i += 2) {
         float t0, t1;
         unpack2(fma2(pack2(acc[8 * u + i], acc[8 * u + i + 1]), k.c1c1, k.nml), t0, t1);
-        if (PF32) { p[i] = ex2_approx(t0); p[i + 1] = ex2_approx(t1); }
-        else exp2_f16_pair(t0, t1, p[i], p[i + 1]);
+        p[i] = ex2_approx(t0);
+        p[i + 1] = ex2_approx(t1);
     }
 }
 
-// Units U0..U1-1 of a thread's NU units: acc -> P (FP16) -> P-hat image words w[4u..4u+3].
-// The exponentials of unit u+1 are issued before unit u is quantized, so that the MUFU latency of
-// one unit hides behind the ALU/FMA work of the previous one.
-// A unit is two 4-key subgroups t = 0, 1 with shifts k_t = max(need_t, need_other - 1) (that is the
-// pair rule: the level-2 bit is set iff max(need) = 2 or min(need) >= 1, and a subgroup that needs no
-// shift of its own still gets one when its partner needs two).  On bit patterns, with
-// x_t = max(bits(At_t) + tadd, 0) = need_t * 2^23 + fraction: k_t * 2^23 = max(x_t, x_other - 2^23)
-// with the fraction masked off.  The packed operations pair key i of subgroup 0 with key i of
-// subgroup 1, so that one pair of per-subgroup constants (magic, c) serves four packed operations.
-template <int NU, int U0, int U1, bool DBG, bool PF32 = false>
-__device__ __forceinline__ void exp_quantize_units(const float (&acc)[NU * 8], const PQuantConst& k, bool zero_group,
-                                                   uint32_t (&w)[NU * 4], uint8_t* dump_codes, float* dump_step)
+// One level-2 unit: P -> P-hat image words w[0..3]; codes / ks0, ks1: the element codes and k << 23 for the dump.
+__device__ __forceinline__ void quantize_unit(const uint32_t (&p)[4], const PQuantConst<false>& k, uint32_t (&w)[4],
+                                              uint32_t (&codes)[2], int& ks0, int& ks1)
+{
+    uint32_t q[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) q[i] = h2_fma(p[i], k.hi, h2_mul(p[i], k.lo));
+    const uint32_t a = h2_max(q[0], q[1]), b = h2_max(q[2], q[3]);
+    const uint32_t At = h2_max(__byte_perm(a, b, 0x5410), __byte_perm(a, b, 0x7632));     // {subgroup 0, subgroup 1}
+    const uint32_t x = __viaddmax_s16x2(At, k.tadd, 0u);
+    const uint32_t ks = __viaddmax_s16x2(__byte_perm(x, x, 0x1032), 0xFC00FC00u, x);      // max(x_t, x_other - 1024)
+    const uint32_t kk = ks & 0x0C000C00u;                                                  // k_t << 10
+    const uint32_t magic = kk | k.magic;
+    const uint32_t t = kk >> 3;                                                            // k_t << 7
+    const uint32_t n = k.n + t, c = k.c + t - kk;
+    const uint32_t magic0 = dup_lo(magic), magic1 = dup_hi(magic);
+    uint32_t y[4];
+    y[0] = h2_add(q[0], magic0);
+    y[1] = h2_add(q[1], magic0);
+    y[2] = h2_add(q[2], magic1);
+    y[3] = h2_add(q[3], magic1);
+    w[0] = bf2_fma(y[0], dup_lo(c), dup_lo(n));
+    w[1] = bf2_fma(y[1], dup_lo(c), dup_lo(n));
+    w[2] = bf2_fma(y[2], dup_hi(c), dup_hi(n));
+    w[3] = bf2_fma(y[3], dup_hi(c), dup_hi(n));
+    codes[0] = __byte_perm(y[0], y[1], 0x6420) & 0x0F0F0F0Fu;
+    codes[1] = __byte_perm(y[2], y[3], 0x6420) & 0x0F0F0F0Fu;
+    ks0 = (int)((kk & 0xFFFFu) << 13);
+    ks1 = (int)((kk >> 16) << 13);
+}
+// The packed operations pair key i of subgroup 0 with key i of subgroup 1, so that one pair of per-subgroup constants
+// (magic, c) serves four packed operations.  On bit patterns, with x_t = max(bits(At_t) + tadd, 0) = need_t * 2^23 +
+// fraction: k_t * 2^23 = max(x_t, x_other - 2^23) with the fraction masked off.
+__device__ __forceinline__ void quantize_unit(const float (&p)[8], const PQuantConst<true>& k, uint32_t (&w)[4],
+                                              uint32_t (&codes)[2], int& ks0, int& ks1)
 {
     const int MAGIC_BITS = 0x4B400000;                                    // 1.5 * 2^23
-    float pn[8];
-    exp_unit<NU, PF32>(acc, U0, k, pn);
+    const float At0 = fmaxf(max3(p[0], p[1], p[2]), p[3]);
+    const float At1 = fmaxf(max3(p[4], p[5], p[6]), p[7]);
+    const int x0 = max((int)__float_as_uint(At0) + k.tadd, 0);
+    const int x1 = max((int)__float_as_uint(At1) + k.tadd, 0);
+    ks0 = max(x0, x1 - (1 << 23)) & (int)0xFF800000;
+    ks1 = max(x1, x0 - (1 << 23)) & (int)0xFF800000;
+    const uint64_t mm = pack2(__int_as_float(MAGIC_BITS + ks0), __int_as_float(MAGIC_BITS + ks1));
+    const uint64_t cc = pack2(__int_as_float((int)k.c0_bits + ks0), __int_as_float((int)k.c0_bits + ks1));
+    float v[8], c[8];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const uint64_t y = add2(mul2_rz(pack2(p[i], p[4 + i]), k.inv44), mm);
+        unpack2(fma2(y, k.s44, cc), v[i], v[4 + i]);
+        unpack2(y, c[i], c[4 + i]);
+    }
+    // BF16 image: every value has at most 8 significant bits, so the upper halves of the FP32 patterns
+    // are the BF16 values (a byte permute instead of a conversion)
+#pragma unroll
+    for (int i = 0; i < 4; ++i) w[i] = __byte_perm(__float_as_uint(v[2 * i]), __float_as_uint(v[2 * i + 1]), 0x7632);
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+        codes[h] = (__float_as_uint(c[4 * h]) & 15u) | ((__float_as_uint(c[4 * h + 1]) & 15u) << 8) |
+                   ((__float_as_uint(c[4 * h + 2]) & 15u) << 16) | ((__float_as_uint(c[4 * h + 3]) & 15u) << 24);
+}
+
+// Units U0..U1-1 of a thread's NU units: acc -> P -> P-hat image words w[4u..4u+3].
+// The exponentials of unit u+1 are issued before unit u is quantized, so that the MUFU latency of
+// one unit hides behind the ALU/FMA work of the previous one.
+template <int NU, int U0, int U1, bool DBG, bool PF32 = false>
+__device__ __forceinline__ void exp_quantize_units(const float (&acc)[NU * 8], const PQuantConst<PF32>& k, bool zero_group,
+                                                   uint32_t (&w)[NU * 4], uint8_t* dump_codes, float* dump_step)
+{
+    using P8 = std::conditional_t<PF32, float[8], uint32_t[4]>;
+    P8 pn;
+    exp_unit<NU>(acc, U0, k, pn);
 #pragma unroll
     for (int u = U0; u < U1; ++u) {
-        float p[8];
+        P8 p;
 #pragma unroll
-        for (int i = 0; i < 8; ++i) p[i] = pn[i];
-        if (u + 1 < U1) exp_unit<NU, PF32>(acc, u + 1, k, pn);
-        const float At0 = fmaxf(max3(p[0], p[1], p[2]), p[3]);
-        const float At1 = fmaxf(max3(p[4], p[5], p[6]), p[7]);
-        const int x0 = max((int)__float_as_uint(At0) + k.tadd, 0);
-        const int x1 = max((int)__float_as_uint(At1) + k.tadd, 0);
-        const int ks0 = max(x0, x1 - (1 << 23)) & (int)0xFF800000;
-        const int ks1 = max(x1, x0 - (1 << 23)) & (int)0xFF800000;
-        const uint64_t mm = pack2(__int_as_float(MAGIC_BITS + ks0), __int_as_float(MAGIC_BITS + ks1));
-        const uint64_t cc = pack2(__int_as_float((int)k.c0_bits + ks0), __int_as_float((int)k.c0_bits + ks1));
-        float v[8];
-        uint64_t y[4];
+        for (int i = 0; i < (PF32 ? 8 : 4); ++i) p[i] = pn[i];
+        if (u + 1 < U1) exp_unit<NU>(acc, u + 1, k, pn);
+        uint32_t wu[4], codes[2];
+        int ks0, ks1;
+        quantize_unit(p, k, wu, codes, ks0, ks1);
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            y[i] = add2(mul2_rz(pack2(p[i], p[4 + i]), k.inv44), mm);
-            unpack2(fma2(y[i], k.s44, cc), v[i], v[4 + i]);
-        }
-        // BF16 image: every value has at most 8 significant bits, so the upper halves of the FP32 patterns
-        // are the BF16 values (a byte permute instead of a conversion)
-#pragma unroll
-        for (int i = 0; i < 4; ++i) w[4 * u + i] = __byte_perm(__float_as_uint(v[2 * i]), __float_as_uint(v[2 * i + 1]), 0x7632);
+        for (int i = 0; i < 4; ++i) w[4 * u + i] = wu[i];
         if (DBG) {
-            float c[8];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) unpack2(y[i], c[i], c[4 + i]);
             if (dump_step) {
                 dump_step[2 * u] = zero_group ? 0.f : __int_as_float((int)k.s4_bits + ks0);
                 dump_step[2 * u + 1] = zero_group ? 0.f : __int_as_float((int)k.s4_bits + ks1);
             }
             if (dump_codes) {
-#pragma unroll
-                for (int h = 0; h < 2; ++h)
-                    reinterpret_cast<uint32_t*>(dump_codes)[2 * u + h] =
-                        (__float_as_uint(c[4 * h]) & 15u) | ((__float_as_uint(c[4 * h + 1]) & 15u) << 8) |
-                        ((__float_as_uint(c[4 * h + 2]) & 15u) << 16) | ((__float_as_uint(c[4 * h + 3]) & 15u) << 24);
+                reinterpret_cast<uint32_t*>(dump_codes)[2 * u] = codes[0];
+                reinterpret_cast<uint32_t*>(dump_codes)[2 * u + 1] = codes[1];
             }
         }
     }

@@ -408,7 +408,7 @@ attention_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid
                 }
                 {
                     uint32_t w[NU * 4];
-                    const PQuantConst qc = p_quant_const(args.c1, mL, A);
+                    const auto qc = p_quant_const<false>(args.c1, mL, A);
                     constexpr int U_SPLIT = (3 * NU) / 4;
                     exp_quantize_units<NU, 0, U_SPLIT, DBG>(p, qc, A == 0.f, w, dc, ds);
                     // next tile (of this item, or the first of the next item): scores and partial maximum
