@@ -340,8 +340,9 @@ int hifa4_attention_fwd_raw(const hifa4_shape* shape, const void* q, const void*
     size_t used = qkv_layout(shape, prm->qmean, (char*)workspace, &bufs);
     if ((s == nullptr) != (inv_s == nullptr)) return HIFA4_ERR_INVALID_ARG;
     // K and V here, Q inside the attention kernel: pays once the Q-hat image (written, then read) is large; measured
-    // on B200 at d = 128: -1 to -3 % of the two launches from 64k query rows up, slower below
-    if (attention_qraw_supported(*shape, *prm) && (long long)shape->B * shape->Hq * shape->N >= 65536) {
+    // on B200 at d = 128: -1 to -3 % of the two launches from 64k query rows up, slower below.  The kernel with two query
+    // blocks per CTA gains more than that (5 to 10 %) and takes Q-hat, so its sizes go through the quantizer.
+    if (attention_qraw_supported(*shape, *prm) && !attention_pair_pays(*shape, *prm) && (long long)shape->B * shape->Hq * shape->N >= 65536) {
         if ((rc = hifa4_quantize_qkv(shape, nullptr, k, v, s, inv_s, &bufs, d_status, stream))) return rc;
         return hifa4_attention_fwd_qraw(shape, q, s, &bufs, prm, out, (char*)workspace + used, d_status, stream);
     }

@@ -414,11 +414,15 @@ int launch_attention(const hifa4_shape& sh, const HeadMap& map, const hifa4_qkv&
             for (int c = 1; c <= sh.B && c * sh.Hkv <= want; ++c)
                 if (sh.B % c == 0) g_b = c;
             a.group_heads = g_b * sh.Hq;
+            a.unit_heads = 1;
+            a.group_units = g_b * sh.Hq;
         } else {
             int g_kv = 1;
             for (int c = 1; c <= n_kv && c <= want; ++c)
                 if (n_kv % c == 0) g_kv = c;
             a.group_heads = g_kv * (sh.Hq / sh.Hkv);
+            a.unit_heads = sh.Hq / sh.Hkv;
+            a.group_units = g_kv;
         }
     }
     a.normalizer = prm.normalizer ? 1 : 0;
@@ -445,6 +449,8 @@ int launch_attention(const hifa4_shape& sh, const HeadMap& map, const hifa4_qkv&
         if (sh.d == 256 && prm.Bc == 64) return launch_cfg<256, 64, true>(sh, qkv, a, st);
         return HIFA4_ERR_UNSUPPORTED;
     }
+    if (!q_raw && !f8 && a.dbg.n_blocks == 0 && attention_pair_pays(sh, prm))
+        return launch_attention_pair(sh, qkv, a, st);
     if (sh.d == 64 && prm.Bc == 64) return launch_attention_ws64(sh, qkv, a, st);
     if (sh.d == 64 && prm.Bc == 128) return launch_cfg<64, 128, false>(sh, qkv, a, st);
     if (sh.d == 128 && prm.Bc == 64) return launch_attention_ws64(sh, qkv, a, st);

@@ -25,6 +25,7 @@ struct AttnArgs {
     int B, Hq, Hkv, N;
     int causal, out_dtype;
     int group_heads;              // CTA order: groups of this many (batch, query head) pairs, one group after the other
+    int unit_heads, group_units;  // two-block kernel: query heads per unit (G, or 1 under a custom head map), units per group
     float c0, c1;                 // sigma, sigma * log2(e)
     int normalizer;               // 1: l accumulates the unquantized P (mismatched), not P-hat
     unsigned long long* hist;     // mass-error histogram [n_bins + 2] or null
@@ -337,6 +338,79 @@ __device__ __forceinline__ void exp_quantize_units(const float (&acc)[NU * 8], c
     }
 }
 
+// Maximum of 64 values: eight chains of eight (three-input maxima), then one chain over the eight.
+__device__ __forceinline__ float max64(const float (&p)[64])
+{
+    float t8[8];
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+        float t = max3(p[8 * c], p[8 * c + 1], p[8 * c + 2]);
+        t = max3(t, p[8 * c + 3], p[8 * c + 4]);
+        t = max3(t, p[8 * c + 5], p[8 * c + 6]);
+        t8[c] = fmaxf(t, p[8 * c + 7]);
+    }
+    float mx = max3(t8[0], t8[1], t8[2]);
+    mx = max3(mx, t8[3], t8[4]);
+    mx = max3(mx, t8[5], t8[6]);
+    return fmaxf(mx, t8[7]);
+}
+
+// Rescale of a row's history: the D channels and the normaliser column of [O | l] at tensor-memory address t_o times
+// rsc, 64 columns per round trip (the other columns of the ones block are never read).  The caller waits for the stores.
+// The loop is not unrolled: unrolled, ptxas overlaps two round trips and spills (120 bytes of reloads per tile at d = 128).
+template <int D>
+__device__ __forceinline__ void rescale_columns(uint32_t t_o, float rsc)
+{
+    const uint64_t rr = pack2(rsc, rsc);
+    auto scale32 = [&](uint32_t (&r)[32]) {
+#pragma unroll
+        for (int i = 0; i < 32; i += 2) {
+            float x0, x1;
+            unpack2(mul2(pack2(__uint_as_float(r[i]), __uint_as_float(r[i + 1])), rr), x0, x1);
+            r[i] = __float_as_uint(x0);
+            r[i + 1] = __float_as_uint(x1);
+        }
+    };
+    uint32_t rl[1];
+    tmem_ld1(t_o + D, rl);
+#pragma unroll 1
+    for (int cc = 0; cc < D / 64; ++cc) {
+        uint32_t r0[32], r1[32];
+        tmem_ld32(t_o + cc * 64, r0);
+        tmem_ld32(t_o + cc * 64 + 32, r1);
+        tmem_wait_ld();
+        scale32(r0);
+        tmem_st32(t_o + cc * 64, r0);
+        scale32(r1);
+        tmem_st32(t_o + cc * 64 + 32, r1);
+    }
+    rl[0] = __float_as_uint(__uint_as_float(rl[0]) * rsc);
+    tmem_st1(t_o + D, rl);
+}
+
+// A warp stores 64 bytes of each of its 32 rows (lane = row, 16 words each): through a swizzled 2 KB tile of shared
+// memory, so that a store instruction covers whole 64-byte pieces of 8 rows.  Rows at or past `rows` are not written.
+__device__ __forceinline__ void store_rows64(uint32_t stage, const uint32_t (&w)[16], uint8_t* dst, size_t row_bytes,
+                                             int rows, int lane)
+{
+#pragma unroll
+    for (int c = 0; c < 4; ++c)
+        asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};"
+                     ::"r"(stage + lane * 64 + ((c ^ ((lane >> 1) & 3)) << 4)), "r"(w[4 * c]), "r"(w[4 * c + 1]), "r"(w[4 * c + 2]),
+                       "r"(w[4 * c + 3]) : "memory");
+    __syncwarp();
+    const int c = lane & 3;
+#pragma unroll
+    for (int it = 0; it < 4; ++it) {
+        const int r = it * 8 + (lane >> 2);
+        uint4 v;
+        asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];"
+                     : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(stage + r * 64 + ((c ^ ((r >> 1) & 3)) << 4)));
+        if (r < rows) *reinterpret_cast<uint4*>(dst + (size_t)r * row_bytes + c * 16) = v;
+    }
+    __syncwarp();
+}
+
 // Whole 64-key group held by one thread; the image goes to row `row` of a 128-byte-swizzled
 // shared-memory tile (the layout a K-major tcgen05 operand descriptor with SWIZZLE_128B reads).
 __device__ __forceinline__ void quantize_p64(const float (&p)[64], uint32_t p_sub_base, int row,
@@ -369,6 +443,8 @@ int launch_attention_ws(const hifa4_shape& sh, const hifa4_qkv& qkv, const AttnA
 
 // Warp-specialised kernels for Bc = 64, d = 64, 128 or 256 (hifa4_attention_ws64.cu).
 int launch_attention_ws64(const hifa4_shape& sh, const hifa4_qkv& qkv, const AttnArgs& args, cudaStream_t st);
+// The same with two query blocks per CTA that share the K / V tiles, d = 128 (hifa4_attention_pair.cu).
+int launch_attention_pair(const hifa4_shape& sh, const hifa4_qkv& qkv, const AttnArgs& args, cudaStream_t st);
 // Self-test instantiation (d = 128): one bounded wait is made to run out (see hifa4_selftest_wait_timeout).
 int launch_attention_ws64_selftest(const hifa4_shape& sh, const hifa4_qkv& qkv, const AttnArgs& args, cudaStream_t st);
 
