@@ -98,15 +98,8 @@ int hifa4_smooth_calibrate(const void* q_cal, const void* k_cal, int S, int Hq, 
     if ((rc = check_arch())) return rc;
     cudaStream_t st = (cudaStream_t)stream;
     double a = mode == 1 ? 0.5 : mode == 2 ? 0.25 : mode == 4 ? (double)alpha : 0.0;
-    size_t n = (size_t)S * Hkv * d;
-    float* kmax = absmax_ws;
-    float* qmax = absmax_ws + n;
-    if (cudaMemsetAsync(absmax_ws, 0, 2 * n * sizeof(float), st) != cudaSuccess) return HIFA4_ERR_CUDA;
-    if (mode != 0) {
-        if (launch_absmax(dt, k_cal, kmap, S, Hkv, Hkv, Ncal, d, kmax, st) != cudaSuccess) return HIFA4_ERR_CUDA;
-        if (launch_absmax(dt, q_cal, qmap, S, Hq, Hkv, Ncal, d, qmax, st) != cudaSuccess) return HIFA4_ERR_CUDA;
-    }
-    if (launch_smooth_finalize(kmax, qmax, S, Hkv * d, a, mode == 0, aggregator, nullptr, s, inv_s, st) != cudaSuccess)
+    if (launch_calibrate(dt, q_cal, k_cal, qmap, S, Hq, Hkv, Ncal, d, a, mode == 0, aggregator, absmax_ws, nullptr, nullptr, s,
+                         inv_s, st) != cudaSuccess)
         return HIFA4_ERR_CUDA;
     if (host_stats) {
         host_stats->rho_K = NAN;
@@ -134,14 +127,8 @@ int hifa4_smooth_calibrate_auto(const void* q_cal, const void* k_cal, int S, int
     if (nk >= (1ll << 32)) return HIFA4_ERR_UNSUPPORTED;          // 32-bit histogram counters
     if ((rc = check_arch())) return rc;
     cudaStream_t st = (cudaStream_t)stream;
-    const size_t n = (size_t)S * Hkv * d;
-    float* kmax = absmax_ws;
-    float* qmax = absmax_ws + n;
-    if (cudaMemsetAsync(absmax_ws, 0, 2 * n * sizeof(float), st) != cudaSuccess) return HIFA4_ERR_CUDA;
-    if (launch_absmax(dt, k_cal, kmap, S, Hkv, Hkv, Ncal, d, kmax, st) != cudaSuccess) return HIFA4_ERR_CUDA;
-    if (launch_absmax(dt, q_cal, qmap, S, Hq, Hkv, Ncal, d, qmax, st) != cudaSuccess) return HIFA4_ERR_CUDA;
-    if (launch_gate(dt, k_cal, nk, kmax, qmax, (int)n, gate_ws, d_stats, st) != cudaSuccess) return HIFA4_ERR_CUDA;
-    if (launch_smooth_finalize(kmax, qmax, S, Hkv * d, 0.0, 0, 0, gate_result(gate_ws), s, inv_s, st) != cudaSuccess)
+    if (launch_calibrate(dt, q_cal, k_cal, qmap, S, Hq, Hkv, Ncal, d, 0.0, false, 0, absmax_ws, gate_ws, d_stats, s, inv_s, st) !=
+        cudaSuccess)
         return HIFA4_ERR_CUDA;
     return HIFA4_OK;
 }

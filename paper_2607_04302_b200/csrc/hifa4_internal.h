@@ -36,17 +36,12 @@ struct SmemOptIn {
 cudaError_t launch_quantize_qkv(int dtype, const hifa4_shape& sh, const HeadMap& qmap, const void* q,
                                 const void* k, const void* v, const float* s, const float* inv_s,
                                 const hifa4_qkv& out, cudaStream_t st);
-cudaError_t launch_absmax(int dtype, const void* x, const HeadMap& map, int S, int H, int Hkv,
-                          int Ncal, int d, float* ws, cudaStream_t st);
-// gate: null, or the device {alpha, bypass} pair written by launch_gate (overrides alpha / bypass).
+// Smooth-QK factors from calibration activations (hifa4_calibrate.cu).  absmax_ws: 2 * S * Hkv * d floats.  gate_ws: null, or
+// HIFA4_GATE_WS_BYTES bytes: the gate then chooses alpha and bypass and fills d_stats (4 floats or null).
 // aggregator: 0 root-mean-square, 1 mean, 2 nearest-rank 99th percentile of the per-sample maxima.
-cudaError_t launch_smooth_finalize(const float* kmax, const float* qmax, int S, int n, double alpha,
-                                   int bypass, int aggregator, const double* gate, float* s, float* inv_s,
-                                   cudaStream_t st);
-// Gate statistics and decision on the device.  gate_ws: HIFA4_GATE_WS_BYTES bytes; d_stats: 4 floats or null.
-cudaError_t launch_gate(int dtype, const void* k_cal, long long nk, const float* kmax, const float* qmax,
-                        int n_max, void* gate_ws, float* d_stats, cudaStream_t st);
-const double* gate_result(void* gate_ws);
+cudaError_t launch_calibrate(int dtype, const void* q_cal, const void* k_cal, const HeadMap& qmap, int S, int Hq, int Hkv,
+                             int Ncal, int d, double alpha, bool bypass, int aggregator, float* absmax_ws, void* gate_ws,
+                             float* d_stats, float* s, float* inv_s, cudaStream_t st);
 
 // Attention forward on the BF16 operand images; returns a hifa4_status.
 // q_raw non-null: Q is the raw 16-bit tensor (qkv.q_mma is not read) and is smoothed with q_scale (or not, if null)

@@ -1,5 +1,4 @@
-// Smooth-QK scaling fused with HIF4 quantization (Algorithm 1 lines 1 and 3) and the
-// calibration reduction behind the Smooth-QK factors (Eq. "sqk").  Q, K and V are quantized by one
+// Smooth-QK scaling fused with HIF4 quantization (Algorithm 1 lines 1 and 3).  Q, K and V are quantized by one
 // launch: 128-bit coalesced loads, one 8-lane team per 64-element group, shuffle reductions,
 // packed f32x2 arithmetic.
 #include "hifa4_internal.h"
@@ -192,77 +191,6 @@ quantize_qkv_kernel(const __grid_constant__ QuantJob job)
     }
 }
 
-// Calibration: per (sample, kv head, channel) maximum magnitude over tokens (and over the query
-// heads of the group).  Non-negative floats order like their bit patterns, so atomicMax on the
-// uint view is exact.  ws [S, Hkv, d] is cleared by the caller.
-template <typename T>
-__global__ void __launch_bounds__(256)
-absmax_kernel(const uint16_t* __restrict__ x, HeadMap map, int H, int Hkv, int Ncal, int d,
-              int tokens_per_block, uint32_t* __restrict__ ws)
-{
-    const int sh = blockIdx.x;                       // sample * H + head
-    const int smp = sh / H, h = sh % H;
-    const int g = map.kv_of[h];
-    const int chunks = d / 8;
-    const int c8 = threadIdx.x % chunks, tl = threadIdx.x / chunks, tstep = blockDim.x / chunks;
-    const int t0 = blockIdx.y * tokens_per_block;
-    const int t1 = min(t0 + tokens_per_block, Ncal);
-    float mx[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    if (tl < tstep) {
-        for (int t = t0 + tl; t < t1; t += tstep) {
-            uint4 raw = __ldg(reinterpret_cast<const uint4*>(x + ((long long)sh * Ncal + t) * d) + c8);
-            const uint16_t* r16 = reinterpret_cast<const uint16_t*>(&raw);
-#pragma unroll
-            for (int i = 0; i < 8; ++i) mx[i] = fmaxf(mx[i], fabsf(In16<T>::to_f(r16[i])));
-        }
-#pragma unroll
-        for (int i = 0; i < 8; ++i)
-            atomicMax(ws + ((long long)smp * Hkv + g) * d + c8 * 8 + i, __float_as_uint(mx[i]));
-    }
-}
-
-// s = Kagg^alpha / Qagg^(1-alpha); 1 where degenerate.  The per-sample maxima are combined over the S samples
-// by root-mean-square (aggregator 0, the paper's choice), mean (1) or nearest-rank 99th percentile (2).
-// gate (optional, device): {alpha, bypass flag} chosen by the applicability gate; overrides the arguments.
-__device__ __forceinline__ double percentile99(const float* __restrict__ v, int S, long long stride)
-{
-    const long long rank = (long long)ceil(0.99 * (double)S) < 1 ? 1 : (long long)ceil(0.99 * (double)S);
-    for (int a = 0; a < S; ++a) {                            // selection by counting: S is small
-        const float va = v[a * stride];
-        long long below = 0, not_above = 0;
-        for (int b = 0; b < S; ++b) { const float vb = v[b * stride]; below += vb < va; not_above += vb <= va; }
-        if (below < rank && rank <= not_above) return (double)va;
-    }
-    return 0.0;
-}
-__global__ void smooth_finalize_kernel(const float* __restrict__ kmax, const float* __restrict__ qmax,
-                                       int S, int n, double alpha, int bypass, int aggregator,
-                                       const double* __restrict__ gate, float* __restrict__ s, float* __restrict__ inv_s)
-{
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    if (gate) { alpha = gate[0]; bypass = gate[1] != 0.0; }
-    double kagg, qagg;
-    if (aggregator == 2) {
-        kagg = percentile99(kmax + i, S, n);
-        qagg = percentile99(qmax + i, S, n);
-    } else {
-        double ks = 0, qs = 0;
-        for (int m = 0; m < S; ++m) {
-            double a = kmax[(long long)m * n + i], b = qmax[(long long)m * n + i];
-            ks += aggregator == 1 ? a : a * a;
-            qs += aggregator == 1 ? b : b * b;
-        }
-        kagg = aggregator == 1 ? ks / S : sqrt(ks / S);
-        qagg = aggregator == 1 ? qs / S : sqrt(qs / S);
-    }
-    double sv = 1.0;
-    if (!bypass && kagg > 0 && qagg > 0) sv = pow(kagg, alpha) / pow(qagg, 1.0 - alpha);
-    float sf = (float)sv;
-    s[i] = sf;
-    inv_s[i] = __frcp_rn(sf);
-}
-
 // ------------------------------------------------------------------------------- launchers
 cudaError_t launch_quantize_qkv(int dtype, const hifa4_shape& sh, const HeadMap& qmap, const void* q,
                                 const void* k, const void* v, const float* s, const float* inv_s,
@@ -293,28 +221,6 @@ cudaError_t launch_quantize_qkv(int dtype, const hifa4_shape& sh, const HeadMap&
         if (upt == 4) quantize_qkv_kernel<__nv_bfloat16, 4><<<(unsigned)total, QUANT_THREADS, 0, st>>>(job);
         else quantize_qkv_kernel<__nv_bfloat16, 2><<<(unsigned)total, QUANT_THREADS, 0, st>>>(job);
     }
-    count_launch();
-    return cudaGetLastError();
-}
-
-cudaError_t launch_absmax(int dtype, const void* x, const HeadMap& map, int S, int H, int Hkv,
-                          int Ncal, int d, float* ws, cudaStream_t st)
-{
-    const int tpb = 256;
-    dim3 grid(S * H, (Ncal + tpb - 1) / tpb);
-    if (dtype == HIFA4_F16)
-        absmax_kernel<__half><<<grid, 256, 0, st>>>((const uint16_t*)x, map, H, Hkv, Ncal, d, tpb, (uint32_t*)ws);
-    else
-        absmax_kernel<__nv_bfloat16><<<grid, 256, 0, st>>>((const uint16_t*)x, map, H, Hkv, Ncal, d, tpb, (uint32_t*)ws);
-    count_launch();
-    return cudaGetLastError();
-}
-
-cudaError_t launch_smooth_finalize(const float* kmax, const float* qmax, int S, int n, double alpha,
-                                   int bypass, int aggregator, const double* gate, float* s, float* inv_s,
-                                   cudaStream_t st)
-{
-    smooth_finalize_kernel<<<(n + 127) / 128, 128, 0, st>>>(kmax, qmax, S, n, alpha, bypass, aggregator, gate, s, inv_s);
     count_launch();
     return cudaGetLastError();
 }
