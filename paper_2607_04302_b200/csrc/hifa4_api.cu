@@ -147,11 +147,9 @@ size_t hifa4_quant_bytes(const hifa4_shape* shape, int which, int part)
     }
 }
 
-int hifa4_quantize_qkv(const hifa4_shape* shape, const void* q, const void* k, const void* v,
-                       const float* s, const float* inv_s, const hifa4_qkv* out, int* d_status,
-                       void* stream)
+static int quantize_common(const hifa4_shape* shape, const void* q, const void* k, const void* v, const float* s,
+                           const float* inv_s, const hifa4_qkv* out, bool with_codes, void* stream)
 {
-    (void)d_status;
     g_calls[1].fetch_add(1, std::memory_order_relaxed);
     int rc = check_shape(shape);
     if (rc) return rc;
@@ -164,9 +162,17 @@ int hifa4_quantize_qkv(const hifa4_shape* shape, const void* q, const void* k, c
     if ((rc = build_map(shape->Hq, shape->Hkv, shape->q_to_kv, qmap, kmap))) return rc;
     if ((rc = check_arch())) return rc;
     cudaStream_t st = (cudaStream_t)stream;
-    if (launch_quantize_qkv(shape->in_dtype, *shape, qmap, q, k, v, s, inv_s, *out, st) != cudaSuccess)
+    if (launch_quantize_qkv(shape->in_dtype, *shape, qmap, q, k, v, s, inv_s, *out, with_codes, st) != cudaSuccess)
         return HIFA4_ERR_CUDA;
     return HIFA4_OK;
+}
+
+int hifa4_quantize_qkv(const hifa4_shape* shape, const void* q, const void* k, const void* v,
+                       const float* s, const float* inv_s, const hifa4_qkv* out, int* d_status,
+                       void* stream)
+{
+    (void)d_status;
+    return quantize_common(shape, q, k, v, s, inv_s, out, true, stream);
 }
 
 static int check_attn(const hifa4_shape* shape, const hifa4_attn_params* prm)
@@ -330,10 +336,11 @@ int hifa4_attention_fwd_raw(const hifa4_shape* shape, const void* q, const void*
     // on B200 at d = 128: -1 to -3 % of the two launches from 64k query rows up, slower below.  The kernel with two query
     // blocks per CTA gains more than that (5 to 10 %) and takes Q-hat, so its sizes go through the quantizer.
     if (attention_qraw_supported(*shape, *prm) && !attention_pair_pays(*shape, *prm) && (long long)shape->B * shape->Hq * shape->N >= 65536) {
-        if ((rc = hifa4_quantize_qkv(shape, nullptr, k, v, s, inv_s, &bufs, d_status, stream))) return rc;
+        if ((rc = quantize_common(shape, nullptr, k, v, s, inv_s, &bufs, false, stream))) return rc;
         return hifa4_attention_fwd_qraw(shape, q, s, &bufs, prm, out, (char*)workspace + used, d_status, stream);
     }
-    if ((rc = hifa4_quantize_qkv(shape, q, k, v, s, inv_s, &bufs, d_status, stream))) return rc;
+    // the attention kernels read the operand images only: codes and metadata are not formed
+    if ((rc = quantize_common(shape, q, k, v, s, inv_s, &bufs, false, stream))) return rc;
     return hifa4_attention_fwd(shape, &bufs, prm, out, (char*)workspace + used, nullptr, d_status, stream);
 }
 

@@ -28,18 +28,6 @@ struct ScanJob {
     HeadMap qmap;
 };
 
-template <typename T> __device__ __forceinline__ uint32_t max16(uint32_t a, uint32_t b);   // two 16-bit floats; a NaN loses
-template <> __device__ __forceinline__ uint32_t max16<__half>(uint32_t a, uint32_t b)
-{
-    return h2_max(a, b);
-}
-template <> __device__ __forceinline__ uint32_t max16<__nv_bfloat16>(uint32_t a, uint32_t b)
-{
-    uint32_t r;
-    asm("max.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
-    return r;
-}
-
 // One group of 512 threads takes rows r0..r1-1 of x [S, H, Ncal, d]: maxima in registers (thread t always holds vector
 // t % C of a row) while the rows belong to one (sample, KV head), then one reduction through shared memory and d atomics.
 template <typename T, bool HIST>

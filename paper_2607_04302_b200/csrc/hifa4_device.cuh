@@ -90,6 +90,37 @@ template <> struct Pair16<__half> {
     }
 };
 
+// Larger of two packed pairs, half by half (a NaN loses).
+template <typename T> __device__ __forceinline__ uint32_t max16(uint32_t a, uint32_t b);
+template <> __device__ __forceinline__ uint32_t max16<__half>(uint32_t a, uint32_t b) { return h2_max(a, b); }
+template <> __device__ __forceinline__ uint32_t max16<__nv_bfloat16>(uint32_t a, uint32_t b)
+{
+    uint32_t r;
+    asm("max.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
+    return r;
+}
+
+// Magnitudes of a packed pair; smaller of two packed BF16 pairs.
+template <typename T> __device__ __forceinline__ uint32_t abs16(uint32_t a);
+template <> __device__ __forceinline__ uint32_t abs16<__half>(uint32_t a)
+{
+    uint32_t r;
+    asm("abs.f16x2 %0, %1;" : "=r"(r) : "r"(a));
+    return r;
+}
+template <> __device__ __forceinline__ uint32_t abs16<__nv_bfloat16>(uint32_t a)
+{
+    uint32_t r;
+    asm("abs.bf16x2 %0, %1;" : "=r"(r) : "r"(a));
+    return r;
+}
+__device__ __forceinline__ uint32_t min16_bf16(uint32_t a, uint32_t b)
+{
+    uint32_t r;
+    asm("min.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
+    return r;
+}
+
 // ---------------------------------------------------------------------------
 // HIF4 quantization of values that are exact in a 16-bit input type, one level-2 unit (8 elements =
 // two level-3 subgroups) at a time.  All arithmetic is exact:
@@ -121,9 +152,30 @@ __device__ __forceinline__ Hif4Group hif4_group(float A)
     g.tadd = (1 << 23) - ((int)__float_as_uint(1.75f * S) + 1);
     return g;
 }
-// x: the unit's values (already clamped to +-top), a0 / a1: the maxima of its two subgroups.  w: BF16 image of
-// the dequantized values (element 2i in the low half of word i); y: the biased quotients (the low byte of
-// bits(y[i]) is the signed element code); a, k0, k1: level-2 shift and the subgroups' total shifts.
+// x: the unit's values (already clamped to +-top); ks0, ks1: the subgroups' total shifts, k << 23.  w: BF16 image of the
+// dequantized values (element 2i in the low half of word i); y: the biased quotients (the low byte of bits(y[i]) is the
+// signed element code).
+__device__ __forceinline__ void hif4_unit_values(const float (&x)[8], uint32_t ks0, uint32_t ks1, const Hif4Group& g,
+                                                 uint32_t (&w)[4], float (&y)[8])
+{
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const uint32_t ks = h ? ks1 : ks0;
+        const float magic = __uint_as_float(0x4B400000u + ks), ck = __uint_as_float(g.c0_bits + ks);
+        const uint64_t mm = pack2(magic, magic), cc = pack2(ck, ck);
+        const uint64_t y01 = add2(mul2_rz(pack2(x[4 * h], x[4 * h + 1]), g.inv44), mm);
+        const uint64_t y23 = add2(mul2_rz(pack2(x[4 * h + 2], x[4 * h + 3]), g.inv44), mm);
+        float v0, v1, v2, v3;
+        unpack2(fma2(y01, g.s44, cc), v0, v1);
+        unpack2(fma2(y23, g.s44, cc), v2, v3);
+        // at most 6 significant bits: the upper halves of the FP32 patterns are the BF16 values
+        w[2 * h] = __byte_perm(__float_as_uint(v0), __float_as_uint(v1), 0x7632);
+        w[2 * h + 1] = __byte_perm(__float_as_uint(v2), __float_as_uint(v3), 0x7632);
+        unpack2(y01, y[4 * h], y[4 * h + 1]);
+        unpack2(y23, y[4 * h + 2], y[4 * h + 3]);
+    }
+}
+// The same from the maxima a0, a1 of the two subgroups; a, k0, k1: level-2 shift and the subgroups' total shifts.
 __device__ __forceinline__ void hif4_unit(const float (&x)[8], float a0, float a1, const Hif4Group& g,
                                           uint32_t (&w)[4], float (&y)[8], int& a, int& k0, int& k1)
 {
@@ -132,22 +184,7 @@ __device__ __forceinline__ void hif4_unit(const float (&x)[8], float a0, float a
     a = (n0 + n1 + 2) >> 2;
     k0 = max(n0, a);
     k1 = max(n1, a);
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        const uint32_t ks = (uint32_t)(h ? k1 : k0) << 23;
-        const uint32_t magic_bits = 0x4B400000u + ks;
-        const float magic = __uint_as_float(magic_bits), ck = __uint_as_float(g.c0_bits + ks);
-        const uint64_t mm = pack2(magic, magic), cc = pack2(ck, ck);
-        const uint64_t y01 = add2(mul2_rz(pack2(x[4 * h], x[4 * h + 1]), g.inv44), mm);
-        const uint64_t y23 = add2(mul2_rz(pack2(x[4 * h + 2], x[4 * h + 3]), g.inv44), mm);
-        float v0, v1, v2, v3;
-        unpack2(fma2(y01, g.s44, cc), v0, v1);
-        unpack2(fma2(y23, g.s44, cc), v2, v3);
-        asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(w[2 * h]) : "f"(v1), "f"(v0));
-        asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(w[2 * h + 1]) : "f"(v3), "f"(v2));
-        unpack2(y01, y[4 * h], y[4 * h + 1]);
-        unpack2(y23, y[4 * h + 2], y[4 * h + 3]);
-    }
+    hif4_unit_values(x, (uint32_t)k0 << 23, (uint32_t)k1 << 23, g, w, y);
 }
 
 // Packed sign-magnitude nibbles of one level-2 unit from the biased quotients y of hif4_unit: element i in nibble i.

@@ -32,10 +32,11 @@ struct SmemOptIn {
 };
 
 // One launch for Q, K and V (null inputs are skipped).  out.q_mu / out.k_sum non-null: Q-Mean
-// (subtract the per-row mean of Q and write it; write the per-row channel sum of K).
+// (subtract the per-row mean of Q and write it; write the per-row channel sum of K).  with_codes = false: only the operand
+// images (and the Q-Mean vectors) are formed.
 cudaError_t launch_quantize_qkv(int dtype, const hifa4_shape& sh, const HeadMap& qmap, const void* q,
                                 const void* k, const void* v, const float* s, const float* inv_s,
-                                const hifa4_qkv& out, cudaStream_t st);
+                                const hifa4_qkv& out, bool with_codes, cudaStream_t st);
 // Smooth-QK factors from calibration activations (hifa4_calibrate.cu).  absmax_ws: 2 * S * Hkv * d floats.  gate_ws: null, or
 // HIFA4_GATE_WS_BYTES bytes: the gate then chooses alpha and bypass and fills d_stats (4 floats or null).
 // aggregator: 0 root-mean-square, 1 mean, 2 nearest-rank 99th percentile of the per-sample maxima.

@@ -1,6 +1,8 @@
 // Smooth-QK scaling fused with HIF4 quantization (Algorithm 1 lines 1 and 3).  Q, K and V are quantized by one
 // launch: 128-bit coalesced loads, one 8-lane team per 64-element group, shuffle reductions,
 // packed f32x2 arithmetic.
+#include <type_traits>
+
 #include "hifa4_internal.h"
 #include "hifa4_device.cuh"
 #include "hifa4_ptx.cuh"
@@ -9,38 +11,135 @@ namespace hifa4 {
 
 using namespace ptx;
 
-// One lane owns 8 consecutive elements of a 64-element group = one level-2 unit = two
-// level-3 subgroups; the 8 lanes of a team (aligned inside a warp) own the group.
-// x[8]: values already smoothed and rounded to the input dtype.  Returns the packed nibbles; w gets
-// the BF16 image of the dequantized values (element 2i in the low half of word i); meta_word the
-// group's metadata (every lane of the team gets the same word).
-// The arithmetic is hif4_group / hif4_unit (exact; the same scheme as the in-register quantizer of P).
-__device__ __forceinline__ uint32_t quantize8(float (&x)[8], int j, uint32_t (&w)[4], uint32_t& meta_word)
+// A team of four lanes owns a 64-element group; lane j owns its level-2 units j and j + 4 (8 elements each), so that the
+// team's 16-byte loads and image stores cover 64 contiguous bytes each.
+// The kernel is bound by instruction issue, the ALU pipe (logic, permutes, shifts, 16-bit maxima, conversions; half rate)
+// first, before it is bound by memory; hence four lanes instead of eight (what a lane does once per group was a third of
+// the instructions), maxima, shift selection and metadata on packed 16-bit patterns, and multiplications where they
+// replace logic: 17 executed warp instructions per element of a lane instead of 25.  Q, K and V of 32 / 8 heads, d = 128,
+// bf16: N = 8192 49.7 -> 41.5 us (230 MB, 5.5 TB/s), N = 4096 27.4 -> 24.7 us; persistent CTAs that load the next piece
+// under the current one were slower (64 us: fewer independent chains per scheduler), and so were one share per thread
+// (48 us) and three or five CTAs per SM.
+struct Group {                        // constants of a 64-element group whose maximum magnitude is A
+    uint32_t s_bits;                  // the scale S = smallest E6M2 value with 7 S >= A (clamped to the code range)
+    uint64_t inv44, s44;              // {4/S, 4/S}, {S/4, S/4}
+    uint32_t c0_bits;                 // bits(-magic * S/4)
+};
+// Biased quotient y = RZ(x * RN(4/S)) + magic * 2^k, magic = 1.5 * 2^23 + 8: rounds to the nearest multiple of 2^k, ties to
+// even (see e6m2_inv4 on the ties); the low bits of y are m + 8 >= 1, m the signed code; fma(y, S/4, -magic * 2^k * S/4) =
+// m * 2^k * S/4 without rounding (magic * (4 + M) has at most 24 significant bits).
+constexpr uint32_t Q_MAGIC_BITS = 0x4B400008u;
+__device__ __forceinline__ Group group_of(float A)
 {
-    float a0 = fmaxf(max3(fabsf(x[0]), fabsf(x[1]), fabsf(x[2])), fabsf(x[3]));
-    float a1 = fmaxf(max3(fabsf(x[4]), fabsf(x[5]), fabsf(x[6])), fabsf(x[7]));
-    float A = fmaxf(a0, a1);
-    A = fmaxf(A, __shfl_xor_sync(0xffffffffu, A, 1));
-    A = fmaxf(A, __shfl_xor_sync(0xffffffffu, A, 2));
-    A = fmaxf(A, __shfl_xor_sync(0xffffffffu, A, 4));
-    const Hif4Group g = hif4_group(A);                            // A = 0 gives code 0 and an all-zero group
-    if (A > g.top) {                                              // only above the E6M2 range: saturate
+    Group g;
+    // S = A / 7 rounded up to two mantissa bits.  1/7 is rounded down, so A = 7 S gives at most S; any other A with at most
+    // 11 significant bits exceeds 7 S by 2^-11 of itself or more, which the two roundings cannot hide.
+    const uint32_t t = (__float_as_uint(__fmul_rn(A, __uint_as_float(0x3E124924u))) + 0x1FFFFFu) & 0xFFE00000u;
+    g.s_bits = min(max(t, 0x27800000u), 0x47600000u);              // codes 0 and 255
+    const float s4 = __uint_as_float(g.s_bits - (2u << 23));
+    float r;                                                       // 4/S correctly rounded: S has three significant bits, so the
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(s4));         // residual is exact and one step decides the rounding
+    r = fmaf(fmaf(-s4, r, 1.f), r, r);
+    g.inv44 = pack2(r, r);
+    g.s44 = pack2(s4, s4);
+    g.c0_bits = __float_as_uint(__fmul_rn(-12582920.f, s4));
+    return g;
+}
+
+// Shifts of the two subgroups of a unit from their maxima At (packed), k_t * 2^7 in the two halves:
+// k_t = max(need_t, need_other - 1), need = number of 1.75 S, 3.5 S exceeded (the pair rule of the level-2 bit).
+template <typename T> __device__ __forceinline__ uint32_t unit_shifts(uint32_t At, float S);
+// BF16 patterns: x_t = max(bits(At_t) - bits(1.75 S) - 1 + 2^7, 0) = need_t * 2^7 + fraction; 1.75 S is a BF16 value, and
+// -bits(1.75 S) - 1 + 2^7 is the complement of bits(0.875 S).
+template <> __device__ __forceinline__ uint32_t unit_shifts<__nv_bfloat16>(uint32_t At, float S)
+{
+    const uint32_t b = __float_as_uint(0.875f * S);
+    const uint32_t x = __viaddmax_s16x2(At, ~__byte_perm(b, b, 0x3232), 0u);
+    return __viaddmax_s16x2(__byte_perm(x, x, 0x1032), 0xFF80FF80u, x) & 0x01800180u;
+}
+// FP16 subnormals have no binades, so FP16 maxima are widened first.
+template <> __device__ __forceinline__ uint32_t unit_shifts<__half>(uint32_t At, float S)
+{
+    float a0, a1;
+    Pair16<__half>::unpack(At, a0, a1);
+    const int b = (int)__float_as_uint(0.875f * S) + 1;
+    const int x0 = max((int)__float_as_uint(a0) - b, 0), x1 = max((int)__float_as_uint(a1) - b, 0);
+    const int k0 = max(x0, x1 - (1 << 23)) >> 23, k1 = max(x1, x0 - (1 << 23)) >> 23;
+    return (uint32_t)(k0 << 7 | k1 << 23);
+}
+
+// xw: the 16 values as packed pairs (words 0-3 unit j, 4-7 unit j + 4), already smoothed and rounded to T.  Returns the
+// BF16 image in xw; CODES: also the packed nibbles of the two units and the group's metadata word (same on every lane).
+template <typename T, bool CODES>
+__device__ __forceinline__ void quantize16(uint32_t (&xw)[8], int j, uint32_t (&nib)[2], uint32_t& meta_word)
+{
+    uint32_t At[2];                                               // {subgroup 0, subgroup 1} of each unit
 #pragma unroll
-        for (int i = 0; i < 8; ++i) x[i] = fminf(fmaxf(x[i], -g.top), g.top);
-        a0 = fminf(a0, g.top);
-        a1 = fminf(a1, g.top);
+    for (int u = 0; u < 2; ++u) {
+        const uint32_t m0 = max16<T>(abs16<T>(xw[4 * u]), abs16<T>(xw[4 * u + 1]));
+        const uint32_t m1 = max16<T>(abs16<T>(xw[4 * u + 2]), abs16<T>(xw[4 * u + 3]));
+        At[u] = max16<T>(__byte_perm(m0, m1, 0x5410), __byte_perm(m0, m1, 0x7632));
     }
-    float y[8];
-    int a, k0, k1;
-    hif4_unit(x, a0, a1, g, w, y, a, k0, k1);
-    uint32_t part = hif4_unit_meta(j, a, k0, k1);
-    if (j == 0) part |= (uint32_t)g.code;
-    const uint32_t nib = hif4_unit_nibbles(y);
-    part |= __shfl_xor_sync(0xffffffffu, part, 1);
-    part |= __shfl_xor_sync(0xffffffffu, part, 2);
-    part |= __shfl_xor_sync(0xffffffffu, part, 4);
-    meta_word = part;
-    return nib;
+    uint32_t A2 = max16<T>(At[0], At[1]);
+    A2 = max16<T>(A2, __byte_perm(A2, A2, 0x1032));
+    A2 = max16<T>(A2, __shfl_xor_sync(0xffffffffu, A2, 1));
+    A2 = max16<T>(A2, __shfl_xor_sync(0xffffffffu, A2, 2));
+    float A, Ah;
+    Pair16<T>::unpack(A2, Ah, A);
+    const Group g = group_of(A);                                  // A = 0 gives code 0 and an all-zero group
+    if (std::is_same<T, __nv_bfloat16>::value && A > 401408.f) {  // above 7 S of the largest scale: saturate
+#pragma unroll
+        for (int i = 0; i < 8; ++i) xw[i] = max16<T>(min16_bf16(xw[i], 0x48C448C4u), 0xC8C4C8C4u);
+        At[0] = min16_bf16(At[0], 0x48C448C4u);
+        At[1] = min16_bf16(At[1], 0x48C448C4u);
+    }
+    uint32_t ks[2];
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+        ks[u] = unit_shifts<T>(At[u], __uint_as_float(g.s_bits));
+        const uint32_t ks0 = ks[u] << 16, ks1 = ks[u] & 0xFFFF0000u;          // k << 23
+        const uint64_t mm = pack2(__uint_as_float(Q_MAGIC_BITS + ks0), __uint_as_float(Q_MAGIC_BITS + ks1));
+        const uint64_t cc = pack2(__uint_as_float(g.c0_bits + ks0), __uint_as_float(g.c0_bits + ks1));
+        // element i of subgroup 0 is paired with element i of subgroup 1: one pair of constants serves four operations
+        float x[8], v[8], y[8];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) Pair16<T>::unpack(xw[4 * u + i], x[2 * i], x[2 * i + 1]);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const uint64_t yy = add2(mul2_rz(pack2(x[i], x[4 + i]), g.inv44), mm);
+            unpack2(fma2(yy, g.s44, cc), v[i], v[4 + i]);
+            unpack2(yy, y[i], y[4 + i]);
+        }
+        // at most 6 significant bits: the upper halves of the FP32 patterns are the BF16 values
+#pragma unroll
+        for (int i = 0; i < 4; ++i) xw[4 * u + i] = __byte_perm(__float_as_uint(v[2 * i]), __float_as_uint(v[2 * i + 1]), 0x7632);
+        if (CODES) {
+            // nibbles m + 8 of a subgroup add up in the low 16 bits (magic * 16^i is zero there except for its 8), then all
+            // eight are turned from offset to sign-magnitude form: negative where bit 3 is clear, |m| = 8 - (m + 8)
+            uint32_t h[2];
+#pragma unroll
+            for (int t = 0; t < 2; ++t) {
+                h[t] = __float_as_uint(y[4 * t + 3]) * 16u + __float_as_uint(y[4 * t + 2]);
+                h[t] = h[t] * 16u + __float_as_uint(y[4 * t + 1]);
+                h[t] = h[t] * 16u + __float_as_uint(y[4 * t]);
+            }
+            const uint32_t b = __byte_perm(h[0], h[1], 0x5410);
+            const uint32_t neg = ~b & 0x88888888u, one = neg >> 3;
+            nib[u] = (((b & 0x77777777u) ^ (one * 7u)) + one) | neg;
+        }
+    }
+    if (CODES) {
+        // level-2 bit of a unit: both subgroups shifted; level-3 bit: k = 2, or k = 1 without the level-2 bit.  Both units
+        // at once: k of (unit, subgroup) at bits 0, 16 (unit j) and 8, 24 (unit j + 4)
+        const uint32_t w = (ks[0] >> 7) | (ks[1] << 1);
+        const uint32_t nz = w | (w >> 1), aa = nz & (nz >> 16) & 0x00000101u;
+        const uint32_t l3 = ((w >> 1) | (w & ~(aa * 0x00010001u))) & 0x01010101u;
+        uint32_t part = ((aa | (aa >> 4)) & 0x11u) << (8 + j);
+        part |= ((l3 | (l3 >> 15)) & 0x0303u) << (16 + 2 * j);
+        part |= __shfl_xor_sync(0xffffffffu, part, 1);
+        part |= __shfl_xor_sync(0xffffffffu, part, 2);
+        meta_word = part | ((g.s_bits >> 21) - 316u);             // + scale code 4 (exponent - 79) + mantissa
+    }
 }
 
 struct QuantJob {                     // one launch quantizes Q, K and V (any of them may be absent)
@@ -52,119 +151,158 @@ struct QuantJob {                     // one launch quantizes Q, K and V (any of
     float *q_mu, *k_sum;              // Q-Mean auxiliary outputs or null
     int Hq, Hkv, N, d;
     unsigned q_blocks, k_blocks;      // CTAs [0, q_blocks) take Q, the next k_blocks K, the rest V
-    unsigned row_blocks_per_head;     // N * d / 8 / (256 * UPT)
+    unsigned row_blocks_per_head;     // N * d / 16 / (256 * UPT)
+    unsigned v_tiles;                 // 64 x 64 tiles of V, two per CTA
     HeadMap qmap;
 };
 
 constexpr int QUANT_THREADS = 256;
-// Row units per thread (template parameter UPT): 4 where a head holds a multiple of 1024 units, which
-// keeps 64 bytes of loads in flight per thread (the kernel is latency-bound below that), else 2.
+// Lane shares (16 elements) per thread, template parameter UPT: 2 where a head holds a multiple of 512 of them (64 bytes of
+// loads in flight per thread), else 1.
 
-// Q and K: groups along d.  One head is N*d/8 units of 8 channels; a CTA takes 256 * UPT consecutive
-// units, thread t the units t, t + 256, ... (all loads are issued before any arithmetic).  The two
-// units share their channel offset, hence their Smooth-QK factors.
-template <typename T, int UPT>
+// Q and K: groups along d.  One head is N*d/16 lane shares; a CTA takes 256 * UPT consecutive ones, thread t the shares t,
+// t + 256 (all loads are issued before any arithmetic).  The shares of a thread have their channels, hence their Smooth-QK
+// factors, in common.
+template <typename T, int UPT, bool CODES, bool QM>
 __device__ __forceinline__ void quantize_rows_cta(const uint16_t* __restrict__ x, const float* __restrict__ scale,
                                                   int kv_row, long long head, unsigned blk_in_head, int N, int d,
                                                   uint8_t* __restrict__ codes, uint32_t* __restrict__ meta,
                                                   uint16_t* __restrict__ img, float* __restrict__ mu_out,
                                                   float* __restrict__ ksum_out)
 {
-    const int upr = d >> 3;                                                   // units per row
-    const unsigned u0 = blk_in_head * (QUANT_THREADS * UPT) + threadIdx.x;    // unit inside the head
-    const long long base = head * (long long)N * upr;                         // first unit of the head
-    const int c0 = (int)(u0 & (unsigned)(upr - 1)) << 3;
-    uint4 raw[UPT];
+    const int spr = d >> 4;                                                   // lane shares per row
+    const int j = threadIdx.x & 3;
+    const unsigned s0 = blk_in_head * (QUANT_THREADS * UPT) + threadIdx.x;    // share inside the head
+    const long long g0 = head * (long long)N * (d >> 6) + (s0 >> 2);          // 64-element group
+    const uint4* src = reinterpret_cast<const uint4*>(x) + g0 * 8 + j;
+    uint4 raw[UPT][2];
 #pragma unroll
-    for (int r = 0; r < UPT; ++r)
-        raw[r] = __ldg(reinterpret_cast<const uint4*>(x) + base + u0 + r * QUANT_THREADS);
-    float sv[8];
+    for (int r = 0; r < UPT; ++r) {
+        raw[r][0] = __ldg(src + r * (QUANT_THREADS * 2));
+        raw[r][1] = __ldg(src + r * (QUANT_THREADS * 2) + 4);
+    }
+    const int c0 = (int)((s0 >> 2) & (unsigned)((d >> 6) - 1)) * 64 + j * 8;  // first channel; the other unit is 32 further
+    float4 sv[4];
     if (scale) {
         const float4* sp = reinterpret_cast<const float4*>(scale + (long long)kv_row * d + c0);
-        const float4 s0 = __ldg(sp), s1 = __ldg(sp + 1);
-        sv[0] = s0.x; sv[1] = s0.y; sv[2] = s0.z; sv[3] = s0.w;
-        sv[4] = s1.x; sv[5] = s1.y; sv[6] = s1.z; sv[7] = s1.w;
+        sv[0] = __ldg(sp); sv[1] = __ldg(sp + 1); sv[2] = __ldg(sp + 8); sv[3] = __ldg(sp + 9);
     }
 #pragma unroll
     for (int r = 0; r < UPT; ++r) {
-        const unsigned u = u0 + r * QUANT_THREADS;
-        const long long t = base + u;
-        const uint32_t rw[4] = {raw[r].x, raw[r].y, raw[r].z, raw[r].w};
-        float v[8];
+        const long long grp = g0 + r * (QUANT_THREADS / 4);
+        uint32_t xw[8] = {raw[r][0].x, raw[r][0].y, raw[r][0].z, raw[r][0].w, raw[r][1].x, raw[r][1].y, raw[r][1].z, raw[r][1].w};
+        if (scale) {                                       // FP32 product, rounded once to the activation dtype
 #pragma unroll
-        for (int i = 0; i < 4; ++i) Pair16<T>::unpack(rw[i], v[2 * i], v[2 * i + 1]);
-        if (scale) {
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                float a, b;
-                unpack2(mul2(pack2(v[2 * i], v[2 * i + 1]), pack2(sv[2 * i], sv[2 * i + 1])), a, b);
-                Pair16<T>::unpack(Pair16<T>::round_pack(a, b), v[2 * i], v[2 * i + 1]);
+            for (int i = 0; i < 8; ++i) {
+                float lo, hi, a, b;
+                Pair16<T>::unpack(xw[i], lo, hi);
+                const float4 f = sv[i >> 1];
+                unpack2(mul2(pack2(lo, hi), (i & 1) ? pack2(f.z, f.w) : pack2(f.x, f.y)), a, b);
+                xw[i] = Pair16<T>::round_pack(a, b);
             }
         }
-        if (mu_out || ksum_out) {
-            // Q-Mean auxiliary (Algorithm 1 lines 2 and 6).  A row of d channels sits in d/8 consecutive,
+        if (QM) {
+            // Q-Mean auxiliary (Algorithm 1 lines 2 and 6).  A row of d channels sits in d/16 consecutive,
             // aligned lanes; the sum runs in double, where it is exact for any row whose values span fewer
             // than ~40 binades, so its order does not matter.
-            const long long row = head * N + (u >> (31 - __clz(upr)));
+            const long long row = head * N + (s0 + r * QUANT_THREADS) / (unsigned)spr;
+            const bool first = ((threadIdx.x & (unsigned)(spr - 1)) == 0);
             double sum = 0.0;
 #pragma unroll
-            for (int i = 0; i < 8; ++i) sum += (double)v[i];
-            for (int off = 1; off < upr; off <<= 1) sum += __shfl_xor_sync(0xffffffffu, sum, off);
-            if (mu_out) {                                // q_z = round_in(q~ - mu), mu = FP16(mean)
+            for (int i = 0; i < 8; ++i) {
+                float lo, hi;
+                Pair16<T>::unpack(xw[i], lo, hi);
+                sum += (double)lo + (double)hi;
+            }
+            for (int off = 1; off < spr; off <<= 1) sum += __shfl_xor_sync(0xffffffffu, sum, off);
+            if (mu_out) {                                  // q_z = round_in(q~ - mu), mu = FP16(mean)
                 const float mu = __half2float(__double2half(sum / (double)d));
 #pragma unroll
-                for (int i = 0; i < 8; ++i) v[i] = In16<T>::round_d((double)v[i] - (double)mu);
-                if (c0 == 0) mu_out[row] = mu;
-            } else if (c0 == 0) {
+                for (int i = 0; i < 8; ++i) {
+                    float lo, hi;
+                    Pair16<T>::unpack(xw[i], lo, hi);
+                    xw[i] = Pair16<T>::round_pack(In16<T>::round_d((double)lo - (double)mu), In16<T>::round_d((double)hi - (double)mu));
+                }
+                if (first) mu_out[row] = mu;
+            } else if (first) {
                 ksum_out[row] = __half2float(__double2half(sum));
             }
         }
-        uint32_t w[4], mw;
-        const uint32_t nib = quantize8(v, threadIdx.x & 7, w, mw);
-        reinterpret_cast<uint32_t*>(codes)[t] = nib;
-        reinterpret_cast<uint4*>(img)[t] = make_uint4(w[0], w[1], w[2], w[3]);
-        if ((threadIdx.x & 7) == 0) meta[t >> 3] = mw;
+        uint32_t nib[2], mw;
+        quantize16<T, CODES>(xw, j, nib, mw);
+        uint4* dst = reinterpret_cast<uint4*>(img) + grp * 8 + j;
+        dst[0] = make_uint4(xw[0], xw[1], xw[2], xw[3]);
+        dst[4] = make_uint4(xw[4], xw[5], xw[6], xw[7]);
+        if (CODES) {
+            uint32_t* cw = reinterpret_cast<uint32_t*>(codes) + grp * 8 + j;
+            cw[0] = nib[0];
+            cw[4] = nib[1];
+            if (j == 0) meta[grp] = mw;
+        }
     }
 }
 
-// V: groups of 64 tokens per channel; outputs are stored transposed ([.., d, N]).  One CTA
-// transposes a 64-token x 64-channel tile through shared memory.  The tile is kept as 64 rows of
-// 8 16-byte chunks, chunk c of row r stored at position c ^ (r >> 3), so that both the row-wise
-// 16-byte stores and the column-wise 4-byte reads (a thread reads two adjacent channels of 8
-// consecutive tokens) are free of bank conflicts.  256 threads = 32 channel pairs x 8 lanes.
-template <typename T>
-__device__ __forceinline__ void quantize_tokens_cta(const uint16_t* __restrict__ x, long long bh, int tok0, int ch0,
-                                                    int N, int d, uint8_t* __restrict__ codes,
-                                                    uint32_t* __restrict__ meta, uint16_t* __restrict__ img)
+// V: groups of 64 tokens per channel; outputs are stored transposed ([.., d, N]).  Half a CTA (128 threads) transposes a
+// 64-token x 64-channel tile through shared memory.  The tile is kept as 64 rows of 8 16-byte chunks, chunk c of row r
+// stored at position c ^ f(r) with f(r) = 2 (r / 8) mod 8 + r / 32, so that both the row-wise 16-byte stores and the
+// column-wise 4-byte reads (a thread reads two adjacent channels of 8 consecutive tokens, a warp 8 channel pairs x 4
+// lanes) are free of bank conflicts.
+template <typename T, bool CODES>
+__device__ __forceinline__ void quantize_tokens_half(uint4* tile, bool valid, const uint16_t* __restrict__ x, long long bh, int tok0,
+                                                     int ch0, int N, int d, uint8_t* __restrict__ codes,
+                                                     uint32_t* __restrict__ meta, uint16_t* __restrict__ img)
 {
-    __shared__ uint4 tile[64 * 8];
-    const uint16_t* src = x + (bh * N + tok0) * (long long)d + ch0;
+    const int tid = threadIdx.x & 127;
+    auto swz = [](int r) { return ((r >> 3) * 2 & 7) + (r >> 5); };
+    if (valid) {
+        const uint16_t* src = x + (bh * N + tok0) * (long long)d + ch0;
+        uint4 v[4];
 #pragma unroll
-    for (int it = 0; it < 2; ++it) {
-        const int idx = threadIdx.x + it * QUANT_THREADS;
-        const int r = idx >> 3, c8 = idx & 7;
-        tile[r * 8 + (c8 ^ (r >> 3))] = __ldg(reinterpret_cast<const uint4*>(src + (long long)r * d) + c8);
+        for (int it = 0; it < 4; ++it) {
+            const int idx = tid + it * 128;
+            v[it] = __ldg(reinterpret_cast<const uint4*>(src + (long long)(idx >> 3) * d) + (idx & 7));
+        }
+#pragma unroll
+        for (int it = 0; it < 4; ++it) {
+            const int idx = tid + it * 128, r = idx >> 3;
+            tile[r * 8 + ((idx & 7) ^ swz(r))] = v[it];
+        }
     }
     __syncthreads();
-    const int cp = threadIdx.x >> 3, j = threadIdx.x & 7;          // channel pair, level-2 unit
+    if (!valid) return;
+    const int cp = tid >> 2, j = tid & 3;                          // channel pair, lane of the team
     const uint32_t* tw = reinterpret_cast<const uint32_t*>(tile);
-    float va[8], vb[8];
+    uint32_t wa[8], wb[8];                                         // channels 2 cp and 2 cp + 1, token pairs
 #pragma unroll
-    for (int i = 0; i < 8; ++i)
-        Pair16<T>::unpack(tw[(8 * j + i) * 32 + ((((cp >> 2) ^ j) << 2) | (cp & 3))], va[i], vb[i]);
+    for (int u = 0; u < 2; ++u)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int r = 8 * (j + 4 * u) + 2 * i;
+            const int pos = (((cp >> 2) ^ swz(r)) << 2) | (cp & 3);
+            const uint32_t t0 = tw[r * 32 + pos], t1 = tw[(r + 1) * 32 + pos];
+            wa[4 * u + i] = __byte_perm(t0, t1, 0x5410);
+            wb[4 * u + i] = __byte_perm(t0, t1, 0x7632);
+        }
 #pragma unroll
     for (int c = 0; c < 2; ++c) {
-        uint32_t w[4], mw;
-        const uint32_t nib = quantize8(c ? vb : va, j, w, mw);
+        uint32_t (&xw)[8] = c ? wb : wa;
+        uint32_t nib[2], mw;
+        quantize16<T, CODES>(xw, j, nib, mw);
         const long long orow = bh * d + ch0 + 2 * cp + c;             // row of the transposed outputs
-        reinterpret_cast<uint32_t*>(codes + orow * (N / 2) + tok0 / 2)[j] = nib;
-        reinterpret_cast<uint4*>(img + orow * (long long)N + tok0)[j] = make_uint4(w[0], w[1], w[2], w[3]);
-        if (j == 0) meta[orow * (N / 64) + tok0 / 64] = mw;
+        uint4* dst = reinterpret_cast<uint4*>(img + orow * (long long)N + tok0) + j;
+        dst[0] = make_uint4(xw[0], xw[1], xw[2], xw[3]);
+        dst[4] = make_uint4(xw[4], xw[5], xw[6], xw[7]);
+        if (CODES) {
+            uint32_t* cw = reinterpret_cast<uint32_t*>(codes + orow * (N / 2) + tok0 / 2) + j;
+            cw[0] = nib[0];
+            cw[4] = nib[1];
+            if (j == 0) meta[orow * (N / 64) + tok0 / 64] = mw;
+        }
     }
 }
 
-template <typename T, int UPT>
-__global__ void __launch_bounds__(QUANT_THREADS)
+template <typename T, int UPT, bool CODES, bool QM>
+__global__ void __launch_bounds__(QUANT_THREADS, 4)
 quantize_qkv_kernel(const __grid_constant__ QuantJob job)
 {
     // a dependent grid launched with programmatic stream serialization (the attention kernel) may start
@@ -177,24 +315,26 @@ quantize_qkv_kernel(const __grid_constant__ QuantJob job)
         const unsigned head = blk / job.row_blocks_per_head;             // b * H + h
         const unsigned in_head = blk - head * job.row_blocks_per_head;
         if (is_q)
-            quantize_rows_cta<T, UPT>(job.q, job.s, job.qmap.kv_of[head % (unsigned)job.Hq], head, in_head, job.N, job.d,
+            quantize_rows_cta<T, UPT, CODES, QM>(job.q, job.s, job.qmap.kv_of[head % (unsigned)job.Hq], head, in_head, job.N, job.d,
                                  job.q_codes, job.q_meta, job.q_img, job.q_mu, nullptr);
         else
-            quantize_rows_cta<T, UPT>(job.k, job.inv_s, (int)(head % (unsigned)job.Hkv), head, in_head, job.N, job.d,
+            quantize_rows_cta<T, UPT, CODES, QM>(job.k, job.inv_s, (int)(head % (unsigned)job.Hkv), head, in_head, job.N, job.d,
                                  job.k_codes, job.k_meta, job.k_img, nullptr, job.k_sum);
     } else {
         blk -= job.q_blocks + job.k_blocks;
+        __shared__ uint4 tiles[2][64 * 8];
+        const unsigned half = threadIdx.x >> 7, t = 2 * blk + half;
         const unsigned tok_blocks = job.N / 64, ch_blocks = job.d / 64;
-        const unsigned tb = blk % tok_blocks, rest = blk / tok_blocks;
+        const unsigned tb = t % tok_blocks, rest = t / tok_blocks;
         const unsigned cb = rest % ch_blocks, bh = rest / ch_blocks;
-        quantize_tokens_cta<T>(job.v, bh, tb * 64, cb * 64, job.N, job.d, job.v_codes, job.v_meta, job.v_img);
+        quantize_tokens_half<T, CODES>(tiles[half], t < job.v_tiles, job.v, bh, tb * 64, cb * 64, job.N, job.d, job.v_codes, job.v_meta, job.v_img);
     }
 }
 
 // ------------------------------------------------------------------------------- launchers
 cudaError_t launch_quantize_qkv(int dtype, const hifa4_shape& sh, const HeadMap& qmap, const void* q,
                                 const void* k, const void* v, const float* s, const float* inv_s,
-                                const hifa4_qkv& out, cudaStream_t st)
+                                const hifa4_qkv& out, bool with_codes, cudaStream_t st)
 {
     QuantJob job{};
     job.q = (const uint16_t*)q; job.k = (const uint16_t*)k; job.v = (const uint16_t*)v;
@@ -204,23 +344,30 @@ cudaError_t launch_quantize_qkv(int dtype, const hifa4_shape& sh, const HeadMap&
     job.q_img = (uint16_t*)out.q_mma; job.k_img = (uint16_t*)out.k_mma; job.v_img = (uint16_t*)out.v_mma;
     job.q_mu = out.q_mu; job.k_sum = out.k_sum;
     job.Hq = sh.Hq; job.Hkv = sh.Hkv; job.N = sh.N; job.d = sh.d;
-    const long long head_units = (long long)sh.N * sh.d / 8;
-    const int upt = head_units % (QUANT_THREADS * 4) == 0 ? 4 : 2;
-    job.row_blocks_per_head = (unsigned)(head_units / (QUANT_THREADS * upt));
+    const long long head_shares = (long long)sh.N * sh.d / 16;
+    const int upt = head_shares % (QUANT_THREADS * 2) == 0 ? 2 : 1;
+    job.row_blocks_per_head = (unsigned)(head_shares / (QUANT_THREADS * upt));
     job.q_blocks = q ? (unsigned)sh.B * sh.Hq * job.row_blocks_per_head : 0u;
     job.k_blocks = k ? (unsigned)sh.B * sh.Hkv * job.row_blocks_per_head : 0u;
-    const unsigned v_blocks = v ? (unsigned)sh.B * sh.Hkv * (sh.N / 64) * (sh.d / 64) : 0u;
+    job.v_tiles = v ? (unsigned)sh.B * sh.Hkv * (sh.N / 64) * (sh.d / 64) : 0u;
+    const unsigned v_blocks = (job.v_tiles + 1) / 2;
     job.qmap = qmap;
     const unsigned long long total = (unsigned long long)job.q_blocks + job.k_blocks + v_blocks;
     if (total == 0) return cudaSuccess;
     if (total > 0x7FFFFFFFull) return cudaErrorInvalidConfiguration;
-    if (dtype == HIFA4_F16) {
-        if (upt == 4) quantize_qkv_kernel<__half, 4><<<(unsigned)total, QUANT_THREADS, 0, st>>>(job);
-        else quantize_qkv_kernel<__half, 2><<<(unsigned)total, QUANT_THREADS, 0, st>>>(job);
-    } else {
-        if (upt == 4) quantize_qkv_kernel<__nv_bfloat16, 4><<<(unsigned)total, QUANT_THREADS, 0, st>>>(job);
-        else quantize_qkv_kernel<__nv_bfloat16, 2><<<(unsigned)total, QUANT_THREADS, 0, st>>>(job);
-    }
+    const bool qm = out.q_mu != nullptr;
+    auto pick = [&](auto t) {
+        using T = decltype(t);
+        auto by_upt = [&](auto codes, auto q_mean) {
+            constexpr bool C = decltype(codes)::value, M = decltype(q_mean)::value;
+            return upt == 2 ? quantize_qkv_kernel<T, 2, C, M> : quantize_qkv_kernel<T, 1, C, M>;
+        };
+        using Yes = std::true_type;
+        using No = std::false_type;
+        return with_codes ? (qm ? by_upt(Yes(), Yes()) : by_upt(Yes(), No())) : (qm ? by_upt(No(), Yes()) : by_upt(No(), No()));
+    };
+    auto kern = dtype == HIFA4_F16 ? pick(__half()) : pick(__nv_bfloat16());
+    kern<<<(unsigned)total, QUANT_THREADS, 0, st>>>(job);
     count_launch();
     return cudaGetLastError();
 }

@@ -1,0 +1,40 @@
+"""The quantizer at the edges of its splits (one or two lane shares per thread, an odd number of V tiles, rows of 4, 8 and
+16 lanes) and of its arithmetic (every scale code, saturation above the E6M2 range, FP16 subnormals, ties, empty groups),
+bit for bit against the oracle."""
+import pytest
+import torch
+
+from paper_2607_04302_b200 import synth
+from tests import parity
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+
+
+@pytest.mark.parametrize("Hq,Hkv,N,d,dtype,qmean", [
+    (1, 1, 64, 64, "bf16", False), (3, 1, 192, 64, "fp16", True), (1, 1, 64, 128, "bf16", True),
+    (2, 1, 320, 128, "fp16", False), (1, 1, 64, 256, "bf16", True), (5, 5, 448, 64, "bf16", False)])
+def test_sizes_match_the_oracle(Hq, Hkv, N, d, dtype, qmean):
+    from paper_2607_04302_b200 import binding as hb
+    cfg = synth.config("C2", N=N, Hq=Hq, Hkv=Hkv, d=d, dtype=dtype, cal_samples=2, cal_tokens=64)
+    q, k, v = synth.make_qkv(cfg)
+    s, inv_s = parity.calibrate(cfg, DEV)
+    qkv = hb.quantize_qkv(q.to(DEV), k.to(DEV), v.to(DEV), s, inv_s, qmean=qmean)
+    parity.check_quantized(cfg, q, k, v, s, inv_s, qkv, qmean=qmean)
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "fp16"])
+def test_extreme_magnitudes_match_the_oracle(dtype):
+    from paper_2607_04302_b200 import binding as hb
+    gen = torch.Generator().manual_seed(7)
+    cfg = synth.config("C3", N=512, Hq=1, Hkv=1, dtype=dtype)
+    lo, hi = (-26.0, 15.9) if dtype == "fp16" else (-60.0, 30.0)       # past both ends of the E6M2 range in bf16
+    e = torch.linspace(lo, hi, 512)[:, None]
+    x = torch.randn((512, 128), generator=gen) * torch.exp2(e)
+    ties = torch.exp2(torch.floor(e)) * torch.randint(-15, 16, (512, 128), generator=gen) / 2
+    x = torch.where(torch.rand((512, 128), generator=gen) < 0.5, ties, x)
+    x[17] = 0
+    x[:, 5] = 0
+    x = (x.clamp(-65504, 65504) if dtype == "fp16" else x).to(synth.torch_dtype(cfg))[None, None]
+    qkv = hb.quantize_qkv(x.to(DEV), x.to(DEV), x.to(DEV))
+    parity.check_quantized(cfg, x, x, x, None, None, qkv)
