@@ -153,12 +153,20 @@ def _check(rc: int, where: str):
         raise Hifa4Error(rc, where)
 
 
+# Host time per call matters for short prompts (two launches of 4 and 8 us): pointers travel as plain integers (argtypes
+# turn them into void*), the stream is read as a handle (0.2 us; building a torch.cuda.Stream object takes 3.3 us), and
+# outputs come from empty_like (1.4 us against 2.4 us for torch.empty with a shape).
 def _ptr(t):
-    return None if t is None else C.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
 def _stream():
-    return C.c_void_p(torch.cuda.current_stream().cuda_stream)
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+
+
+def _empty_out(like, out_dtype):
+    """Contiguous uninitialised tensor of `like`'s shape and device."""
+    return torch.empty_like(like, dtype=_TORCH_DT[out_dtype], memory_format=torch.contiguous_format)
 
 
 def _map_arr(q_to_kv):
@@ -202,10 +210,10 @@ class QuantizedQKV:
     k_sum: torch.Tensor | None = None       # Q-Mean auxiliary: channel sum of the smoothed key
 
     def struct(self) -> _QKV:
-        ptrs = [getattr(self, n).data_ptr() for n in ("q_codes", "q_meta", "q_mma", "k_codes",
-                                                      "k_meta", "k_mma", "v_codes", "v_meta", "v_mma")]
-        ptrs += [None if t is None else t.data_ptr() for t in (self.q_mu, self.k_sum)]
-        return _QKV(*ptrs)
+        return _QKV(self.q_codes.data_ptr(), self.q_meta.data_ptr(), self.q_mma.data_ptr(),
+                    self.k_codes.data_ptr(), self.k_meta.data_ptr(), self.k_mma.data_ptr(),
+                    self.v_codes.data_ptr(), self.v_meta.data_ptr(), self.v_mma.data_ptr(),
+                    _ptr(self.q_mu), _ptr(self.k_sum))
 
 
 def quant_bytes(B, Hq, Hkv, N, d, in_dtype, which, part) -> int:
@@ -216,8 +224,10 @@ def quant_bytes(B, Hq, Hkv, N, d, in_dtype, which, part) -> int:
 def alloc_qkv(B, Hq, Hkv, N, d, in_dtype, device, q_to_kv=None, qmean=False) -> QuantizedQKV:
     """Allocate the buffers with the sizes the library reports (qmean: also the two Q-Mean vectors)."""
     bufs = {}
+    size = lib().hifa4_quant_bytes
+    sh = C.byref(_shape(B, Hq, Hkv, N, d, in_dtype))
     for w, name, H in ((Q, "q", Hq), (K, "k", Hkv), (V, "v", Hkv)):
-        nb = [quant_bytes(B, Hq, Hkv, N, d, in_dtype, w, p) for p in (CODES, META, MMA)]
+        nb = [size(sh, w, p) for p in (CODES, META, MMA)]
         if 0 in nb:
             raise Hifa4Error(2, "hifa4_quant_bytes")
         tok_axis = (w == V)
@@ -268,7 +278,7 @@ def smooth_calibrate_auto(q_cal, k_cal, q_to_kv=None):
     inv_s = torch.empty_like(s)
     ws = torch.empty((2, S, Hkv, d), dtype=torch.float32, device=dev)
     gate_ws = torch.empty(GATE_WS_BYTES // 8, dtype=torch.int64, device=dev)
-    stats = torch.zeros(4, dtype=torch.float32, device=dev)
+    stats = torch.empty(4, dtype=torch.float32, device=dev)
     keep, mp = _map_arr(q_to_kv)
     rc = lib().hifa4_smooth_calibrate_auto(_ptr(q_cal), _ptr(k_cal), S, Hq, Hkv, Ncal, d, mp, _DT[q_cal.dtype],
                                            _ptr(s), _ptr(inv_s), _ptr(ws), _ptr(gate_ws), _ptr(stats), _stream())
@@ -330,7 +340,7 @@ def attention_fwd(qkv: QuantizedQKV, causal: bool, Bc: int = 64, out_dtype=F32, 
     prm = _params(causal, Bc, out_dtype, Br=Br, softmax_scale=softmax_scale, qmean=int(qmean),
                   normalizer=int(normalizer), p_dtype=p_dtype)
     if out is None:
-        out = torch.empty((qkv.B, qkv.Hq, qkv.N, qkv.d), dtype=_TORCH_DT[out_dtype], device=dev)
+        out = _empty_out(qkv.q_mma, out_dtype)
     st = qkv.struct()
     dbg_p, dump = None, None
     if debug_blocks:
@@ -360,7 +370,7 @@ def attention_fwd_qraw(q, s, kv: QuantizedQKV, causal: bool, out_dtype=F32, out=
     assert tuple(q.shape) == (kv.B, kv.Hq, kv.N, kv.d)
     prm = _params(causal, 64, out_dtype, softmax_scale=softmax_scale, p_dtype=p_dtype)
     if out is None:
-        out = torch.empty((kv.B, kv.Hq, kv.N, kv.d), dtype=_TORCH_DT[out_dtype], device=q.device)
+        out = _empty_out(q, out_dtype)
     st = kv.struct()
     rc = lib().hifa4_attention_fwd_qraw(C.byref(sh), _ptr(q), _ptr(s), C.byref(st), C.byref(prm), _ptr(out), None,
                                         _ptr(d_status), _stream())
@@ -383,7 +393,7 @@ def attention_fwd_f8qk(qkv: QuantizedQKV, causal: bool, out_dtype=F32, out=None,
         out = torch.empty((qkv.B, qkv.Hq, qkv.N, qkv.d), dtype=_TORCH_DT[out_dtype], device=dev)
     st = qkv.struct()
     rc = lib().hifa4_attention_fwd_f8qk(C.byref(sh), C.byref(st), C.byref(prm), _ptr(out), _ptr(workspace),
-                                        C.c_size_t(workspace.numel()), _ptr(d_status), _stream())
+                                        workspace.numel(), _ptr(d_status), _stream())
     _check(rc, "hifa4_attention_fwd_f8qk")
     return out
 
@@ -437,11 +447,11 @@ def attention_fwd_raw(q, k, v, s, inv_s, causal: bool, Bc: int = 64, out_dtype=F
     if need == 0:
         raise Hifa4Error(2, "hifa4_attention_raw_workspace_bytes")
     if workspace is None:
-        workspace = torch.empty(need, dtype=torch.uint8, device=q.device)
+        workspace = q.new_empty(need, dtype=torch.uint8)
     if out is None:
-        out = torch.empty((B, Hq, N, d), dtype=_TORCH_DT[out_dtype], device=q.device)
+        out = _empty_out(q, out_dtype)
     rc = lib().hifa4_attention_fwd_raw(C.byref(sh), _ptr(q), _ptr(k), _ptr(v), _ptr(s), _ptr(inv_s),
                                        C.byref(prm), _ptr(out), _ptr(workspace),
-                                       C.c_size_t(workspace.numel()), _ptr(d_status), _stream())
+                                       workspace.numel(), _ptr(d_status), _stream())
     _check(rc, "hifa4_attention_fwd_raw")
     return out
