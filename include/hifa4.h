@@ -258,7 +258,7 @@ size_t hifa4_attention_workspace_bytes(const hifa4_shape* shape, const hifa4_att
  *   *_mma images are read).  out: [B,Hq,N,d] of prm->out_dtype.
  *   workspace: at least hifa4_attention_workspace_bytes() bytes (NULL if 0).
  *   dbg: NULL, or a P-hat dump request.
- * Scheduling note: for Bc = 64 the grid is launched with programmatic stream
+ * Scheduling note (calibration and quantization alike): for Bc = 64 the grid is launched with programmatic stream
  * serialization, i.e. its CTAs may become resident while the preceding kernel
  * of the stream is still draining; they read and write no global memory before
  * that kernel has completed, so the usual stream order of results holds. */

@@ -521,19 +521,8 @@ static int launch_pair(const hifa4_shape& sh, const hifa4_qkv& qkv, const AttnAr
     static SmemOptIn opt_in;
     if (!opt_in.ensure(kern, C::SMEM_BYTES)) return HIFA4_ERR_CUDA;
     const int blocks = (sh.N + 127) / 128 * args.unit_heads;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(((blocks + 1) / 2) * (sh.Hq / args.unit_heads) * sh.B));
-    cfg.blockDim = dim3(C::THREADS);
-    cfg.dynamicSmemBytes = C::SMEM_BYTES;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;   // see griddepcontrol.wait in the kernel
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, mq, mk, mv, args);
-    count_launch();
-    return e == cudaSuccess && cudaGetLastError() == cudaSuccess ? HIFA4_OK : HIFA4_ERR_CUDA;
+    const unsigned grid = (unsigned)(((blocks + 1) / 2) * (sh.Hq / args.unit_heads) * sh.B);
+    return launch_dependent(kern, grid, C::THREADS, C::SMEM_BYTES, st, mq, mk, mv, args) == cudaSuccess ? HIFA4_OK : HIFA4_ERR_CUDA;
 }
 
 // Whether this kernel is the faster one: a pair per SM and wave here, against up to two blocks per SM in the 64-key kernel,

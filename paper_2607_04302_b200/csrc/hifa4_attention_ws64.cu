@@ -613,20 +613,8 @@ static int launch_ws64(const hifa4_shape& sh, const hifa4_qkv& qkv, const AttnAr
     auto kern = attention_fwd_ws64_kernel<DH, DBG, PF32, QM, SELFTEST, QRAW, F8QK>;
     static SmemOptIn opt_in;
     if (!opt_in.ensure(kern, C::SMEM_BYTES)) return HIFA4_ERR_CUDA;
-    dim3 grid((unsigned)(((sh.N + 127) / 128) * sh.Hq * sh.B));
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grid;
-    cfg.blockDim = dim3(C::THREADS);
-    cfg.dynamicSmemBytes = C::SMEM_BYTES;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;   // see griddepcontrol.wait in the kernel
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, mq, mk, mv, args);
-    count_launch();
-    return e == cudaSuccess && cudaGetLastError() == cudaSuccess ? HIFA4_OK : HIFA4_ERR_CUDA;
+    const unsigned grid = (unsigned)(((sh.N + 127) / 128) * sh.Hq * sh.B);
+    return launch_dependent(kern, grid, C::THREADS, C::SMEM_BYTES, st, mq, mk, mv, args) == cudaSuccess ? HIFA4_OK : HIFA4_ERR_CUDA;
 }
 
 template <int DH>

@@ -133,6 +133,7 @@ __global__ void __launch_bounds__(256)
 clear_kernel(uint32_t* __restrict__ a, long long na, uint32_t* __restrict__ b, int nb)
 {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     const long long step = (long long)gridDim.x * 256, i0 = (long long)blockIdx.x * 256 + threadIdx.x;
     for (long long i = i0; i < na; i += step) a[i] = 0;
     for (long long i = i0; i < nb; i += step) b[i] = 0;
@@ -247,25 +248,6 @@ smooth_finalize_kernel(const float* __restrict__ kmax, const float* __restrict__
 }
 
 // ------------------------------------------------------------------------------- launchers
-// Launch that may become resident while its predecessor in the stream drains (it waits before it touches memory).
-template <typename... KArgs, typename... Args>
-static cudaError_t launch_dependent(void (*kern)(KArgs...), unsigned grid, unsigned block, size_t smem, cudaStream_t st, Args... args)
-{
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(block);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...);
-    count_launch();
-    return e != cudaSuccess ? e : cudaGetLastError();
-}
-
 template <typename T, bool HIST>
 static cudaError_t launch_scan(const ScanJob& job, cudaStream_t st)
 {
@@ -289,9 +271,8 @@ cudaError_t launch_calibrate(int dtype, const void* q_cal, const void* k_cal, co
     uint32_t* gmax = hist ? hist + HIST_BINS : nullptr;
     cudaError_t e;
     if (hist) {
-        clear_kernel<<<64, 256, 0, st>>>(reinterpret_cast<uint32_t*>(absmax_ws), 2 * n, hist, HIST_BINS + 2);
-        count_launch();
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        if ((e = launch_dependent(clear_kernel, 64, 256, 0, st, reinterpret_cast<uint32_t*>(absmax_ws), 2 * n, hist, HIST_BINS + 2)) != cudaSuccess)
+            return e;
     } else if ((e = cudaMemsetAsync(absmax_ws, 0, 2 * n * sizeof(float), st)) != cudaSuccess) {
         return e;
     }

@@ -31,6 +31,26 @@ struct SmemOptIn {
     }
 };
 
+// Launch that may become resident while its predecessor in the stream drains (programmatic stream serialization): the
+// kernel executes griddepcontrol.wait before it touches memory.
+template <typename... KArgs, typename... Args>
+cudaError_t launch_dependent(void (*kern)(KArgs...), unsigned grid, unsigned block, size_t smem, cudaStream_t st, Args... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...);
+    count_launch();
+    return e != cudaSuccess ? e : cudaGetLastError();
+}
+
 // One launch for Q, K and V (null inputs are skipped).  out.q_mu / out.k_sum non-null: Q-Mean
 // (subtract the per-row mean of Q and write it; write the per-row channel sum of K).  with_codes = false: only the operand
 // images (and the Q-Mean vectors) are formed.
