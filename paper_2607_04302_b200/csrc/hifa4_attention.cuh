@@ -357,7 +357,9 @@ __device__ __forceinline__ float max64(const float (&p)[64])
 
 // Rescale of a row's history: the D channels and the normaliser column of [O | l] at tensor-memory address t_o times
 // rsc, 64 columns per round trip (the other columns of the ones block are never read).  The caller waits for the stores.
-// The loop is not unrolled: unrolled, ptxas overlaps two round trips and spills (120 bytes of reloads per tile at d = 128).
+// Unrolled only for d = 256 (one CTA per SM, registers to spare: 540 -> 518 us at N = 8192, 16 heads); at the 96 registers of
+// the d = 128 kernels ptxas would overlap two round trips and spill (80 to 120 bytes of reloads per tile: 34.9 against
+// 32.9 us for 8 heads, B = 2, N = 2048).
 template <int D>
 __device__ __forceinline__ void rescale_columns(uint32_t t_o, float rsc)
 {
@@ -373,7 +375,7 @@ __device__ __forceinline__ void rescale_columns(uint32_t t_o, float rsc)
     };
     uint32_t rl[1];
     tmem_ld1(t_o + D, rl);
-#pragma unroll 1
+#pragma unroll (D > 128 ? D / 64 : 1)
     for (int cc = 0; cc < D / 64; ++cc) {
         uint32_t r0[32], r1[32];
         tmem_ld32(t_o + cc * 64, r0);

@@ -56,7 +56,7 @@ namespace pairk {
 // wait must not be two phases behind.
 enum { QF = 0, QD = 1, SFR = 2, PGO = 3, SF = 4, PV = 6, MR = 8, OE = 10, HALF = 12,
        KF = 24, KE = 27, VF = 30, VE = 33, WF = 36, WE = 38, CL = 40, KSF = 41, N_BARS = 49 };
-constexpr uint32_t WAIT_POLLS = 1u << 20;
+constexpr uint32_t WAIT_POLLS = 1u << 18;            // a poll may keep the thread suspended for up to about 4 us
 struct Work {                         // one pair of query blocks
     int n_max;                        // key tiles to load; 0: no more work
     int bh_kv;
@@ -223,8 +223,8 @@ attention_fwd_pair_kernel(const __grid_constant__ CUtensorMap tmap_q, const __gr
                 uint32_t idle = 0;
                 bool ok = true;
                 while (jv < n_max) {
-                    if (++idle > WAIT_POLLS || ((idle & 63u) == 63u && ld_flag(abort_flag))) {
-                        if (idle > WAIT_POLLS) fail(1);
+                    if (++idle > 4 * WAIT_POLLS || ((idle & 63u) == 63u && ld_flag(abort_flag))) {
+                        if (idle > 4 * WAIT_POLLS) fail(1);
                         ok = false;
                         break;
                     }
@@ -463,7 +463,7 @@ attention_fwd_pair_kernel(const __grid_constant__ CUtensorMap tmap_q, const __gr
             bool first[2] = {true, true}, done[2] = {false, false};
             uint32_t idle = 0;
             while (!(done[0] && done[1])) {
-                if (++idle > WAIT_POLLS || ((idle & 63u) == 63u && ld_flag(abort_flag))) { if (idle > WAIT_POLLS) fail(7); break; }
+                if (++idle > 4 * WAIT_POLLS || ((idle & 63u) == 63u && ld_flag(abort_flag))) { if (idle > 4 * WAIT_POLLS) fail(7); break; }
 #pragma unroll
                 for (int hf = 0; hf < 2; ++hf) {
                     if (done[hf]) continue;
