@@ -41,25 +41,23 @@ constexpr int SMEM_BYTES = STG_OFF + 16 * 1024 + 1024;
 constexpr int O_COLS = D + 16, QT_COL = 144, S_COL = 256, TMEM_COLS = 512;
 enum { BAR_QFULL = 0, BAR_QFREE = 2, BAR_KF = 4, BAR_KE = 6, BAR_VF = 8, BAR_VE = 10, BAR_SF = 12,
        BAR_PF = 14, BAR_PV = 16, BAR_X = 17, BAR_QT = 25, N_BARS = 26 };
-constexpr uint32_t WAIT_POLLS = 1u << 20;           // each poll blocks for a hardware-defined slice
+constexpr uint32_t WAIT_POLLS = 1u << 18;           // each poll may keep the thread suspended for up to about 4 us
 }  // namespace ws
 
-// Bounded waits.  wait_or_abort polls without blocking (softmax warps and the issuer: a late wake-up sits on
-// the critical path, and a thread suspended in try_wait was seen to notice a completed phase about 1000 clk
-// late).  wait_sleepy lets the hardware suspend the thread for up to a few microseconds per poll, for the
-// producer warp, which waits most of the time and has slack.
+// Bounded waits.  wait_or_abort (softmax warps and the issuer) leaves the suspension time to the hardware, wait_sleepy asks
+// for up to 4 us per poll, for the producer warp, which waits most of the time and has slack.
 __device__ __forceinline__ bool wait_or_abort(uint32_t bar, uint32_t parity, volatile int* abort_flag)
 {
 #pragma unroll 1
     for (uint32_t i = 0; i < ws::WAIT_POLLS; ++i) {
-        if (mbar_test_wait(bar, parity)) return true;
+        if (mbar_try_wait(bar, parity)) return true;
         if ((i & 63u) == 63u && *abort_flag) return false;
     }
     return false;
 }
 __device__ __forceinline__ bool wait_sleepy(uint32_t bar, uint32_t parity, volatile int* abort_flag)
 {
-    for (uint32_t i = 0; i < ws::WAIT_POLLS / 4; ++i) {
+    for (uint32_t i = 0; i < ws::WAIT_POLLS; ++i) {
         if (mbar_try_wait_hint(bar, parity, 4000u)) return true;
         if (*abort_flag) return false;
     }
@@ -291,8 +289,8 @@ attention_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid
             return true;
         };
 
-        // The scores of the next tile are pulled into registers, reduced and published while the
-        // current tile is still being quantized (S is double-buffered), so the row-maximum exchange of
+        // The scores of the next tile are pulled into registers, reduced and published before the P-hat of the
+        // current one is handed over (S is double-buffered), so the row-maximum exchange of
         // a tile is usually complete by the time its turn comes and the KS warps of a row quarter need
         // not run in phase.  g: global tile index; jt, q0: the tile's place in its own item.
         auto fetch_scores = [&](int g, int jt, int q0, float mu, int bh_kv, float (&sc)[KPT]) -> float {
@@ -409,9 +407,10 @@ attention_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid
                 {
                     uint32_t w[NU * 4];
                     const auto qc = p_quant_const<false>(args.c1, mL, A);
-                    constexpr int U_SPLIT = (3 * NU) / 4;
-                    exp_quantize_units<NU, 0, U_SPLIT, DBG>(p, qc, A == 0.f, w, dc, ds);
-                    // next tile (of this item, or the first of the next item): scores and partial maximum
+                    exp_quantize_units<NU, 0, NU, DBG>(p, qc, A == 0.f, w, dc, ds);
+                    // next tile (of this item, or the first of the next item): scores and partial maximum, once the last
+                    // scores of this tile are used up (under three quarters of the quantization, as it was, both tiles' scores
+                    // were live: with try_wait 213 -> 198 us for 32 / 8 heads, N = 4096, causal)
                     const bool in_item = jt + 1 < n_tiles;
                     if (in_item || has_next) {
                         const int nk = in_item ? k : k + 1, njt = in_item ? jt + 1 : 0;
@@ -426,7 +425,6 @@ attention_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid
                             if (!copy_q(nk + 1)) { ok = false; break; }
                         }
                     }
-                    exp_quantize_units<NU, U_SPLIT, NU, DBG>(p, qc, A == 0.f, w, dc, ds);
                     if constexpr (KS == 2) tmem_st32(t_s + kq * (KPT / 2), w);
                     else tmem_st16(t_s + kq * (KPT / 2), w);
                 }
