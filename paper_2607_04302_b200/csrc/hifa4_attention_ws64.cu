@@ -22,8 +22,8 @@
 // signal it free, and S(j+1) runs on the tensor pipe while they work on tile j; the BF16 image of P-hat
 // has its own tensor-memory columns and is the A operand of the P V MMA.
 // One tile is one 64-key HIF4 group of P per row, held by one thread: no row statistic is computed twice.
-//   d = 256: 512 tensor-memory columns: [O | l] 0..271 (an N = 256 MMA for the channels, an N = 16
-//            MMA on the same A operand for the ones block), Q-hat image 272..399 (A operand of
+//   d = 256: 512 tensor-memory columns: [O | l] 0..271 (an N = 128 and an N = 144 MMA on the same A operand:
+//            67 + 72 clk per step of 16 keys; an MMA takes at least 62 clk, so N = 256 and N = 16 took 128 + 60), Q-hat image 272..399 (A operand of
 //            Q K^T from tensor memory), S 400..463, P-hat 464..495.  One CTA per SM.
 //   d = 64:  as d = 128 with [O | l] 0..79 (one N = 80 MMA); 53 KB of shared memory.
 //   d = 128: 256 tensor-memory columns: [O | l] 0..143 (one N = 144 MMA), S 144..207, P-hat
@@ -281,8 +281,8 @@ attention_fwd_ws64_kernel(const __grid_constant__ CUtensorMap tmap_q, const __gr
     } else if (warp == W_PV) {
         // ------------------------------------------------------------------ V^T loads, issuer of [O | l] += P-hat [V | 1]
         if (lane == 0) {
-            constexpr uint32_t idesc_o = umma_idesc_bf16(128, D == 256 ? 256 : O_COLS);
-            constexpr uint32_t idesc_l = umma_idesc_bf16(128, 16);
+            constexpr uint32_t idesc_o = umma_idesc_bf16(128, D == 256 ? 128 : O_COLS);
+            constexpr uint32_t idesc_h = umma_idesc_bf16(128, 144);
             const uint32_t v_lo = umma_desc_lo(v_s);
             load_v(0);
             if (n_tiles > 1) load_v(1);
@@ -296,8 +296,8 @@ attention_fwd_ws64_kernel(const __grid_constant__ CUtensorMap tmap_q, const __gr
 #pragma unroll
                 for (int kk = 0; kk < 4; ++kk) {                // 16 keys per step; channels (+ ones block)
                     umma_bf16_ts_lo(tmem, tmem + P_COL + kk * 8, b0 + kk * 2, idesc_o, kk ? 1u : acc0);
-                    if constexpr (D == 256)                      // N = 272 does not exist: the ones block separately
-                        umma_bf16_ts_lo(tmem + 256, tmem + P_COL + kk * 8, b0 + ((D * 128) >> 4) + kk * 2, idesc_l, kk ? 1u : acc0);
+                    if constexpr (D == 256)                      // N = 272 does not exist: two parts, the ones block in the second
+                        umma_bf16_ts_lo(tmem + 128, tmem + P_COL + kk * 8, b0 + ((128 * 128) >> 4) + kk * 2, idesc_h, kk ? 1u : acc0);
                 }
                 umma_commit(bar(BAR_PV + st));
                 umma_commit(bar(BAR_VE + st));
