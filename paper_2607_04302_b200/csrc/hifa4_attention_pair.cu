@@ -183,7 +183,7 @@ attention_fwd_pair_kernel(const __grid_constant__ CUtensorMap tmap_q, const __gr
         // fall through to the common exit
     } else if (warp == C::W_LD) {
         // ------------------------------------------------------------------ work list, K and V^T loads
-        if (lane == 0) {
+        if (elect_one()) {
             // Order of the pairs: units (KV heads with their G query heads; single query heads under a custom head map) in
             // groups whose K / V images fit in L2 together; inside a group the position in the unit's list of blocks is
             // outermost, and that list runs from the last query block (the heaviest under a causal mask) to the first, all
@@ -410,7 +410,7 @@ attention_fwd_pair_kernel(const __grid_constant__ CUtensorMap tmap_q, const __gr
         }
     } else if (warp < C::W_PV) {
         // ------------------------------------------------------------------ Q loads, issuer of S = Q K^T (one half)
-        if (lane == 0) {
+        if (elect_one()) {
             const int hf = warp - C::W_QK;
             constexpr uint32_t idesc_s = umma_idesc_bf16(128, BC);
             const uint32_t q_s = smem_base + hf * C::Q_HALF, b_h = bar(hf * HALF);
@@ -455,7 +455,7 @@ attention_fwd_pair_kernel(const __grid_constant__ CUtensorMap tmap_q, const __gr
         }
     } else {
         // ------------------------------------------------------------------ issuer of [O | l] += P-hat [V | 1], both halves
-        if (lane == 0) {
+        if (elect_one()) {
             constexpr uint32_t idesc_o = umma_idesc_bf16(128, O_COLS);
             const uint32_t v_lo = umma_desc_lo(v_s);
             int it[2] = {0, 0}, jt[2] = {0, 0}, n_max[2] = {0, 0}, n_tiles[2] = {0, 0}, st[2] = {0, 0};

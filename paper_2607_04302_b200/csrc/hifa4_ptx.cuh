@@ -250,7 +250,8 @@ __device__ __forceinline__ void umma_f8_ss_lo(uint32_t d_tmem, uint32_t a_lo, ui
         "tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], ad, bd, %4, p;\n\t}"
         ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(UMMA_DESC_HI_SW128), "r"(idesc), "r"(accumulate) : "memory");
 }
-// One lane of a converged warp (the same lane every time while the warp stays converged).
+// One lane of a converged warp (the same lane every time while the warp stays converged).  Code that issues MMAs goes inside
+// `if (elect_one())`: behind `lane == 0` the compiler cannot tell that one thread runs it, and an MMA takes 62 clk or more.
 __device__ __forceinline__ bool elect_one()
 {
     uint32_t p;
