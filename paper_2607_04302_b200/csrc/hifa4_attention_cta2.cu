@@ -5,19 +5,23 @@
 // half from its partner, so a tile crosses L2 -> SM once for 256 query rows and half of it sits in each shared memory.
 // That leaves room for S of a whole step of two tiles (N = 128, the full rate of the tensor cores) and for two P-hat
 // buffers, for which d = 256 has no tensor memory with one CTA per tile (there Q takes 128 columns).  16 / 8 heads, causal,
-// N = 8192: 460 us against 487 in the 64-key kernel, 490 against 545 under the power cap (N = 4096, B = 2, non-causal: 458
-// against 498, 486 against 525).
+// N = 8192: 440 us against 487 in the 64-key kernel, 475 against 545 under the power cap (N = 4096, B = 2, non-causal: 448
+// against 498, 475 against 525).
 // Warps of a CTA:
 //   0-7    softmax / quantize: warps 0-3 own the even key tiles, warps 4-7 the odd ones, one thread per row and tile
 //   8-11   history, one thread per row: rescale of [O | l], output
 //   12     one thread: TMA loads of the CTA's Q block and of its half of the K and V^T tiles; in CTA 0 also the work list
-//   13     CTA 0 only, one thread: issuer of all MMAs
+//   13     CTA 0 only, one thread: issuer of S = Q K^T
+//   14, 15 CTA 0 only, one thread each: issuers of [O | l] += P-hat [V | 1], a part each
 // What bounds it: the chain P V(t) - rescale - P V(t+1), since at 256 rows some row's maximum moves in nearly every tile.
 // With the rescale in the softmax warps, which own alternate tiles but finish both tiles of a step together, the chain held
 // them up: 562 us.  P V is therefore issued in two parts, channels 0..127 and channels 128..255 with the ones block, each
 // with its own barriers, so that one part is rescaled while the other is multiplied; and S is issued in four pieces of 64
 // channels, at most two of them in flight, with P V in between (all of S at once: 496 us; pieces of 32 channels, two in
-// flight, leave the tensor cores idle between them: 700 us; three of 64: no difference).
+// flight, leave the tensor cores idle between them: 700 us; three of 64: no difference).  A single issuer that polls for
+// both kinds of work spends 800 clk per part of P V in its loop, next to warps that fill the issue slots: 460 us.
+// (d = 128 in this form, with three groups of softmax warps, stays behind two independent blocks per SM, which hide one
+// another's chain: 2.5 against 2.0 ms at N = 16384, 32 / 8 heads, causal.)
 // N of a cta_group::2 MMA is a multiple of 32 and CTA r supplies the r-th half of its B rows: CTA 0 holds the K rows of a
 // step's first tile, the V^T rows of channels 0..63, 128..191 and 16 rows of ones, CTA 1 the K rows of the second tile, the
 // V^T rows of 64..127, 192..255 and 16 rows of ones.  Tensor memory (columns): channels 0..127, 128..191, ones 16, channels
@@ -32,34 +36,36 @@
 namespace hifa4 {
 
 struct Cta2Cfg {
-    static constexpr int D = 256, BC = 64, K_STAGES = 2, V_STAGES = 4;
-    static constexpr int NSW = 8, W_HIST = 8, W_LD = 12, W_MMA = 13, THREADS = 448;
+    static constexpr int D = 256, BC = 64, QSUB = D / 64;
+    static constexpr int K_STAGES = 2, V_STAGES = 4;
+    static constexpr int NSW = 8, W_HIST = 8, W_LD = 12, W_QK = 13, W_PV = 14, THREADS = 512;
     static constexpr int NU = BC / 8;
-    static constexpr int Q_BYTES = 4 * 16384;               // four sub-tiles of 64 channels x 128 rows
-    static constexpr int K_SUB = 64 * 128, K_STAGE = 4 * K_SUB;      // this CTA's 64 of a step's 128 keys
-    static constexpr int V_STAGE = (64 + 64 + 16) * 128;    // this CTA's rows of both parts, rows of ones
-    static constexpr int V_HI = 64 * 128;                   // second part inside a stage
+    static constexpr int Q_BYTES = QSUB * 16384;            // sub-tiles of 64 channels x 128 rows
+    static constexpr int K_SUB = 64 * 128, K_STAGE = QSUB * K_SUB;     // this CTA's 64 of a step's 128 keys
+    static constexpr int V_ROWS = D / 4;                    // this CTA's channels of either part of P V
+    static constexpr int V_HI = V_ROWS * 128, V_ONES = 2 * V_HI, V_STAGE = V_ONES + 16 * 128;    // second part, ones inside a stage
     static constexpr int K_OFF = Q_BYTES, V_OFF = K_OFF + K_STAGES * K_STAGE;
     static constexpr int STG_OFF = V_OFF + V_STAGES * V_STAGE;         // output staging, 2 KB per history warp
-    static constexpr int MX_OFF = STG_OFF + 4 * 2048;     // running maxima handed from tile t to t+1: [t % 2][128] floats
-    static constexpr int RS_OFF = MX_OFF + 1024;       // rescale factors for the history warps: [t % 4][128] floats
+    static constexpr int MX_OFF = STG_OFF + 4 * 2048;       // running maxima handed from tile t to t+1: [t % 2][128] floats
+    static constexpr int RS_OFF = MX_OFF + 1024;            // rescale factors for the history warps: [t % 4][128] floats
     static constexpr int KSUM_OFF = RS_OFF + 2048;          // Q-Mean: channel sums of a step's 128 keys, slot = step % 4
-    static constexpr int MISC_OFF = KSUM_OFF + 8 * 256;
+    static constexpr int MISC_OFF = KSUM_OFF + 4 * 512;
     static constexpr int SMEM_BYTES = MISC_OFF + 1024 + 1024;
-    static constexpr int HI_COL = 128, L_COL = 192, S_COL = 288, P_COL = S_COL + 128, TMEM_COLS = 512;
+    static constexpr int HI_COL = D / 2, L_COL = D / 2 + V_ROWS, S_COL = D + 32, P_COL = S_COL + 128, TMEM_COLS = 512;
     static_assert(P_COL + 64 <= TMEM_COLS && SMEM_BYTES <= 227 * 1024, "tensor memory or shared memory budget");
-    static_assert(MX_OFF % 1024 == 0 && MISC_OFF % 16 == 0, "addresses below are formed with xor");
+    static_assert(K_OFF % 1024 == 0 && V_STAGE % 1024 == 0 && MX_OFF % 1024 == 0 && MISC_OFF % 16 == 0,
+                  "swizzle atoms, addresses formed with xor, bulk copies");
 };
 
 namespace cta2 {
-// In CTA 0, for both: QF Q blocks landed, KF / VF halves landed, SFR S of a step pulled (16 arrivals), PG[t % 2] P-hat
-// stored (8), RL / RH[t % 2] first / second part of the history rescaled or, at a pair's first tile, output (8), WE[pair % 2]
-// work record read (26), CL answer of the launch control, SC[piece % 2] piece of S complete.  In each CTA: QD last S of the
-// pair complete, KE / VE stage free, SF S of a step complete, PL / PH[t % 2] first / second part of P V complete, MR[t % 4]
-// maxima and rescale factors published (4 arrivals; the softmax warps may be two tiles ahead of the history warps),
-// WF[pair % 2] work record written, KSF[step % 4] Q-Mean key sums landed.
-enum { PL = 0, PH = 2, MR = 4, PG = 8, RL = 10, RH = 12, WF = 14, WE = 16, SF = 18, SFR = 19, QF = 20, QD = 21, CL = 22,
-       KF = 23, KE = 25, VF = 27, VE = 31, KSF = 35, SC = 39, N_BARS = 41 };
+// In CTA 0, for both: QF Q blocks landed, KF / VF halves landed, SFR S of a step pulled (16 arrivals), GL / GH[t % 2] P-hat
+// stored and first / second part of the history rescaled or, at a pair's first tile, output (16), WE[pair % 2] work record
+// read (28), CL answer of the launch control, SC[piece % 2] piece of S complete.  In each CTA: QD last S of the pair
+// complete, KE stage free, SF S of a step complete, PL / PH[t % 2] first / second part of P V complete, PV[t % 4] both, and
+// the V^T stage free (2), MR[t % 4] maxima and rescale factors published (4 arrivals; the softmax warps may be two tiles
+// ahead of the history warps), WF[pair % 2] work record written, KSF[step % 4] Q-Mean key sums landed.
+enum { PL = 0, PH = 2, PV = 4, MR = 8, GL = 12, GH = 14, WF = 16, WE = 18, SF = 20, SFR = 21, QF = 22, QD = 23, CL = 24,
+       KF = 25, KE = 27, VF = 29, KSF = 33, SC = 37, N_BARS = 39 };
 constexpr uint32_t WAIT_POLLS = 1u << 18;            // a poll may keep the thread suspended for up to about 4 us
 struct Work {
     int n_max;                        // steps of two key tiles; 0: no more work
@@ -186,24 +192,29 @@ __device__ __forceinline__ int launch_control_answer(uint32_t src)          // b
                  : "=r"(got), "=r"(x) : "r"(src) : "memory");
     return got ? (int)x : -1;
 }
-// 64 columns of [O | l] at tensor-memory address t times r; the caller waits for the stores.
-__device__ __forceinline__ void scale64(uint32_t t, float r)
+// NC columns of [O | l] at tensor-memory address t times r; the caller waits for the stores.
+template <int NC>
+__device__ __forceinline__ void scale_columns(uint32_t t, float r)
 {
     const uint64_t rr = pack2(r, r);
-    uint32_t a[2][32];
-    tmem_ld32(t, a[0]);
-    tmem_ld32(t + 32, a[1]);
-    tmem_wait_ld();
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
+    for (int c = 0; c < NC; c += 64) {
+        constexpr int H = NC < 64 ? 1 : 2;
+        uint32_t a[H][32];
 #pragma unroll
-        for (int i = 0; i < 32; i += 2) {
-            float x0, x1;
-            unpack2(mul2(pack2(__uint_as_float(a[h][i]), __uint_as_float(a[h][i + 1])), rr), x0, x1);
-            a[h][i] = __float_as_uint(x0);
-            a[h][i + 1] = __float_as_uint(x1);
+        for (int h = 0; h < H; ++h) tmem_ld32(t + c + 32 * h, a[h]);
+        tmem_wait_ld();
+#pragma unroll
+        for (int h = 0; h < H; ++h) {
+#pragma unroll
+            for (int i = 0; i < 32; i += 2) {
+                float x0, x1;
+                unpack2(mul2(pack2(__uint_as_float(a[h][i]), __uint_as_float(a[h][i + 1])), rr), x0, x1);
+                a[h][i] = __float_as_uint(x0);
+                a[h][i + 1] = __float_as_uint(x1);
+            }
+            tmem_st32(t + c + 32 * h, a[h]);
         }
-        tmem_st32(t + 32 * h, a[h]);
     }
 }
 }  // namespace cta2
@@ -236,15 +247,15 @@ attention_fwd_cta2_kernel(const __grid_constant__ CUtensorMap tmap_q, const __gr
         int status_now = rank == 0 && args.d_status ? *reinterpret_cast<volatile int*>(args.d_status) : 0;
         tma_prefetch_desc(&tmap_q); tma_prefetch_desc(&tmap_k); tma_prefetch_desc(&tmap_v);
         for (int s = 0; s < 2; ++s) {
-            mbar_init(bar(PL + s), 1); mbar_init(bar(PH + s), 1); mbar_init(bar(SC + s), 1); mbar_init(bar(MR + s), 4); mbar_init(bar(MR + 2 + s), 4);
-            mbar_init(bar(PG + s), 8); mbar_init(bar(RL + s), 8); mbar_init(bar(RH + s), 8);
-            mbar_init(bar(WF + s), 1); mbar_init(bar(WE + s), 26);
+            mbar_init(bar(PL + s), 1); mbar_init(bar(PH + s), 1); mbar_init(bar(GL + s), 16); mbar_init(bar(GH + s), 16);
+            mbar_init(bar(WF + s), 1); mbar_init(bar(WE + s), 2 * C::NSW + 12); mbar_init(bar(SC + s), 1);
+            mbar_init(bar(KF + s), 1); mbar_init(bar(KE + s), 1);
+        }
+        for (int s = 0; s < 4; ++s) {
+            mbar_init(bar(MR + s), 4); mbar_init(bar(VF + s), 1); mbar_init(bar(PV + s), 2); mbar_init(bar(KSF + s), 1);
         }
         mbar_init(bar(SF), 1); mbar_init(bar(SFR), 16);
         mbar_init(bar(QF), 1); mbar_init(bar(QD), 1); mbar_init(bar(CL), 1);
-        for (int s = 0; s < C::K_STAGES; ++s) { mbar_init(bar(KF + s), 1); mbar_init(bar(KE + s), 1); }
-        for (int s = 0; s < C::V_STAGES; ++s) { mbar_init(bar(VF + s), 1); mbar_init(bar(VE + s), 1); }
-        for (int s = 0; s < 4; ++s) mbar_init(bar(KSF + s), 1);
         fence_barrier_init();
         // nothing the preceding kernel of the stream wrote is touched before this point (programmatic launch)
         asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -264,7 +275,7 @@ attention_fwd_cta2_kernel(const __grid_constant__ CUtensorMap tmap_q, const __gr
     for (int i = tid; i < C::V_STAGES * 128; i += C::THREADS) {        // ones rows under every V^T stage
         const int st = i / 128, off = (i % 128) * 16;
         asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};"
-                     ::"r"(v_s + st * C::V_STAGE + 128 * 128 + off), "r"(0x3F803F80u) : "memory");
+                     ::"r"(v_s + st * C::V_STAGE + C::V_ONES + off), "r"(0x3F803F80u) : "memory");
     }
     fence_proxy_async_smem();
     tc_fence_before();
@@ -344,7 +355,7 @@ attention_fwd_cta2_kernel(const __grid_constant__ CUtensorMap tmap_q, const __gr
                         if (rank == 0) mbar_expect_tx(bar(KF + stk), 2 * C::K_STAGE);
                         const uint32_t kf = at_rank(bar(KF + stk), 0);
 #pragma unroll
-                        for (int s = 0; s < 4; ++s)
+                        for (int s = 0; s < C::QSUB; ++s)
                             load_3d(k_s + stk * C::K_STAGE + s * C::K_SUB, &tmap_k, kf, 64 * s, jk * 2 * BC + 64 * (int)rank, bh_kv);
                         if (QM) {
                             // slot c % 4 held the sums of step c-4: this load follows S(c-2), hence the pull of S(c-3) by the
@@ -363,14 +374,14 @@ attention_fwd_cta2_kernel(const __grid_constant__ CUtensorMap tmap_q, const __gr
                         q_done = true;
                         if (rank == 0) mbar_expect_tx(bar(QF), 2 * C::Q_BYTES);
 #pragma unroll
-                        for (int s = 0; s < 4; ++s) load_3d(smem_base + s * 16384, &tmap_q, qf, 64 * s, q0, bh_q);
+                        for (int s = 0; s < C::QSUB; ++s) load_3d(smem_base + s * 16384, &tmap_q, qf, 64 * s, q0, bh_q);
                     }
-                    if (jv < 2 * jk && mbar_try_wait(bar(VE + stv), phv)) {
+                    if (jv < 2 * jk && mbar_try_wait(bar(PV + stv), phv)) {
                         idle = 0;
-                        if (rank == 0) mbar_expect_tx(bar(VF + stv), 4 * 64 * 128);
+                        if (rank == 0) mbar_expect_tx(bar(VF + stv), 4 * C::V_HI);
                         const uint32_t vf = at_rank(bar(VF + stv), 0);
-                        load_3d(v_s + stv * C::V_STAGE, &tmap_v, vf, jv * BC, 64 * (int)rank, bh_kv);
-                        load_3d(v_s + stv * C::V_STAGE + C::V_HI, &tmap_v, vf, jv * BC, 128 + 64 * (int)rank, bh_kv);
+                        load_3d(v_s + stv * C::V_STAGE, &tmap_v, vf, jv * BC, C::V_ROWS * (int)rank, bh_kv);
+                        load_3d(v_s + stv * C::V_STAGE + C::V_HI, &tmap_v, vf, jv * BC, D / 2 + C::V_ROWS * (int)rank, bh_kv);
                         ++jv;
                         if (++stv == C::V_STAGES) { stv = 0; phv ^= 1u; }
                     }
@@ -391,8 +402,7 @@ attention_fwd_cta2_kernel(const __grid_constant__ CUtensorMap tmap_q, const __gr
         const float LOG2E = 1.4426950408889634f;
         const uint32_t mx_own = smem_base + C::MX_OFF + grp * 512 + r_loc * 4;
         const uint32_t rs_own = smem_base + C::RS_OFF + grp * 512 + r_loc * 4;
-        const uint32_t b_own = bars + 8 * grp;
-        const uint32_t r_own = at_rank(b_own, 0), r_sfr = at_rank(bar(SFR), 0);     // barriers in CTA 0
+        const uint32_t r_own = at_rank(bars + 8 * grp, 0), r_sfr = at_rank(bar(SFR), 0);     // barriers in CTA 0
         int t0 = 0;                                               // tiles before the current pair (even)
         bool ok = true;
         for (int it = 0; ok; ++it) {
@@ -405,9 +415,8 @@ attention_fwd_cta2_kernel(const __grid_constant__ CUtensorMap tmap_q, const __gr
             const float mu_row = (QM && row < N) ? args.q_mu[(size_t)w.bh_q[rank] * N + row] : 0.f;
 
             for (int jt = grp; jt < n_tiles; jt += 2) {
-                const int t = t0 + jt, j0 = jt * BC;               // t % 2 == grp
-                const uint32_t ph = (uint32_t)(t >> 1) & 1u;
-                if (!wait(bar(SF), ph, abort_flag)) { fail(8); ok = false; break; }
+                const int t = t0 + jt, u = t >> 1, j0 = jt * BC;   // t % 2 == grp; step u
+                if (!wait(bar(SF), (uint32_t)u & 1u, abort_flag)) { fail(8); ok = false; break; }
                 tc_fence_after();
                 float p[BC];
                 {
@@ -423,9 +432,8 @@ attention_fwd_cta2_kernel(const __grid_constant__ CUtensorMap tmap_q, const __gr
                 arrive_remote0(r_sfr, lane);
 
                 if (QM) {                                          // Q-Mean correction (line 6): + mu_i * sum_c k~_jc
-                    const int c = t >> 1;
-                    if (!wait(bar(KSF + (c & 3)), (uint32_t)(c >> 2) & 1u, abort_flag)) { fail(15); ok = false; break; }
-                    const uint32_t ks_s = smem_base + C::KSUM_OFF + (c & 3) * 512 + grp * 256;
+                    if (!wait(bar(KSF + (u & 3)), (uint32_t)(u >> 2) & 1u, abort_flag)) { fail(15); ok = false; break; }
+                    const uint32_t ks_s = smem_base + C::KSUM_OFF + (u & 3) * 512 + grp * 256;
                     const uint64_t mu2 = pack2(mu_row, mu_row);
 #pragma unroll
                     for (int i = 0; i < BC / 4; ++i) {
@@ -465,14 +473,15 @@ attention_fwd_cta2_kernel(const __grid_constant__ CUtensorMap tmap_q, const __gr
                 exp_quantize_units<NU, 0, NU, false, false>(p, qc, false, pw, nullptr, nullptr);
                 // this P-hat buffer is free once P V(t-2) has completed
                 if (t >= 2) {
-                    if (!wait(b_own + 8 * PH, (uint32_t)((t - 2) >> 1) & 1u, abort_flag)) { fail(10); ok = false; break; }
+                    if (!wait(bar(PV + ((t - 2) & 3)), (uint32_t)((t - 2) >> 2) & 1u, abort_flag)) { fail(10); ok = false; break; }
                     tc_fence_after();
                 }
                 tmem_st32(t_o + C::P_COL + grp * 32, pw);
                 tmem_wait_st();
                 tc_fence_before();
                 __syncwarp();
-                arrive_remote0(r_own + 8 * PG, lane);
+                arrive_remote0(r_own + 8 * GL, lane);
+                arrive_remote0(r_own + 8 * GH, lane);
             }
             if (!ok) break;
             t0 += n_tiles;
@@ -483,8 +492,11 @@ attention_fwd_cta2_kernel(const __grid_constant__ CUtensorMap tmap_q, const __gr
         // ------------------------------------------------------------------ history: rescale, finalize
         const int quarter = warp & 3, r_loc = quarter * 32 + lane;
         const uint32_t t_o = tmem + ((uint32_t)(quarter * 32) << 16);
-        const uint32_t rs_s = smem_base + C::RS_OFF + r_loc * 4, r_rl = at_rank(bar(RL), 0), r_rh = at_rank(bar(RH), 0);
+        const uint32_t rs_s = smem_base + C::RS_OFF + r_loc * 4, r_gl = at_rank(bar(GL), 0), r_gh = at_rank(bar(GH), 0);
         int t = 0;
+        auto wait_pv = [&](int tile) { return wait(bar(PV + (tile & 3)), (uint32_t)(tile >> 2) & 1u, abort_flag); };
+        // a part of P V(t-1)
+        auto wait_part = [&](int part) { return wait(bar(part + ((t - 1) & 1)), (uint32_t)((t - 1) >> 1) & 1u, abort_flag); };
         bool ok = true;
         for (int it = 0; ok; ++it) {
             if (!wait<true>(bar(WF + (it & 1)), (uint32_t)(it >> 1) & 1u, abort_flag)) { fail(18); break; }
@@ -492,47 +504,44 @@ attention_fwd_cta2_kernel(const __grid_constant__ CUtensorMap tmap_q, const __gr
             const int n_tiles = 2 * w.n_max, q0 = w.q0[rank];
             if (n_tiles == 0) break;
             for (int jt = 0; jt < n_tiles; ++jt, ++t) {
-                const uint32_t i8 = 8 * (t & 1), j8 = i8 ^ 8, ph_prev = (uint32_t)((t - 1) >> 1) & 1u;
-                // P V(t-2) complete: the arrivals below belong to tile t, and no wait on PL or PH can be two phases behind
-                if (t >= 2 && !wait(bar(PH) + i8, (uint32_t)((t - 2) >> 1) & 1u, abort_flag)) { fail(10); ok = false; break; }
                 float rsc = 1.f;
                 if (jt > 0) {
                     if (!wait(bar(MR + (t & 3)), (uint32_t)(t >> 2) & 1u, abort_flag)) { fail(12); ok = false; break; }
                     asm volatile("ld.shared.f32 %0, [%1];" : "=f"(rsc) : "r"(rs_s + (t & 3) * 512) : "memory");
                 }
+                // P V(t-2) complete: the arrivals below belong to tile t, and no wait on PL or PH can be two phases behind
+                if (t >= 2 && !wait_pv(t - 2)) { fail(10); ok = false; break; }
                 // rescale (line 8), each part as soon as P V(t-1) of it has completed
                 const bool any = __any_sync(0xffffffffu, rsc != 1.f);
                 if (any) {
-                    if (!wait(bar(PL) + j8, ph_prev, abort_flag)) { fail(13); ok = false; break; }
+                    if (!wait_part(PL)) { fail(13); ok = false; break; }
                     tc_fence_after();
-                    scale64(t_o, rsc);
-                    scale64(t_o + 64, rsc);
+                    scale_columns<D / 2>(t_o, rsc);
                     tmem_wait_st();
                     tc_fence_before();
                     __syncwarp();
                 }
-                arrive_remote0(r_rl + i8, lane);
+                arrive_remote0(r_gl + 8 * (t & 1), lane);
                 if (any) {
-                    if (!wait(bar(PH) + j8, ph_prev, abort_flag)) { fail(14); ok = false; break; }
+                    if (!wait_part(PH)) { fail(14); ok = false; break; }
                     tc_fence_after();
                     uint32_t rl[1];
                     tmem_ld1(t_o + C::L_COL, rl);
-                    scale64(t_o + C::HI_COL, rsc);
-                    scale64(t_o + C::L_COL + 16, rsc);
+                    scale_columns<C::V_ROWS>(t_o + C::HI_COL, rsc);
+                    scale_columns<C::V_ROWS>(t_o + C::L_COL + 16, rsc);
                     rl[0] = __float_as_uint(__uint_as_float(rl[0]) * rsc);
                     tmem_st1(t_o + C::L_COL, rl);
                     tmem_wait_st();
                     tc_fence_before();
                     __syncwarp();
                 }
-                arrive_remote0(r_rh + i8, lane);
+                arrive_remote0(r_gh + 8 * (t & 1), lane);
             }
             if (!ok) break;
 
             // finalize: out = O / l with l rounded to FP16 (line 13)
             // (P V(t-2) first: only then can the other barrier not be two phases behind)
-            if (!wait(bar(PH + (t & 1)), (uint32_t)((t - 2) >> 1) & 1u, abort_flag)) { fail(11); ok = false; break; }
-            if (!wait(bar(PH + ((t - 1) & 1)), (uint32_t)((t - 1) >> 1) & 1u, abort_flag)) { fail(11); ok = false; break; }
+            if (!wait_pv(t - 2) || !wait_pv(t - 1)) { fail(11); ok = false; break; }
             tc_fence_after();
             uint32_t lr[1];
             tmem_ld1(t_o + C::L_COL, lr);
@@ -545,7 +554,7 @@ attention_fwd_cta2_kernel(const __grid_constant__ CUtensorMap tmap_q, const __gr
             const int rows = w.store[rank] ? N - q0 - quarter * 32 : 0;  // rows of the warp inside the sequence (may exceed 32)
             const uint32_t stage = smem_base + C::STG_OFF + (uint32_t)quarter * 2048u;
 #pragma unroll 1
-            for (int cc = 0; cc < 8; ++cc) {
+            for (int cc = 0; cc < D / 32; ++cc) {
                 const int col = cc * 32;
                 uint32_t r[32];
                 tmem_ld32(t_o + col + (col >= C::L_COL ? 16 : 0), r);
@@ -578,75 +587,69 @@ attention_fwd_cta2_kernel(const __grid_constant__ CUtensorMap tmap_q, const __gr
             __syncwarp();
             arrive_remote0(at_rank(bar(WE + (it & 1)), 0), lane);
         }
-    } else if (rank == 0) {
+    } else if (rank == 0 && warp == C::W_QK) {
+        // ------------------------------------------------------------------ issuer of S = Q K^T (CTA 0)
         if (elect_one()) {
-        // ------------------------------------------------------------------ issuer of all MMAs (CTA 0)
-        constexpr uint32_t idesc_s = umma_idesc_bf16(256, 2 * BC), idesc_l = umma_idesc_bf16(256, 128), idesc_h = umma_idesc_bf16(256, 160);
-        const uint32_t q_lo = umma_desc_lo(smem_base), k_lo = umma_desc_lo(k_s), v_lo = umma_desc_lo(v_s);
-        int stk = 0, stv = 0, us = 0, t = 0;                  // ring stages; steps whose S, tiles whose P V has been issued
-        int sc = 0, ch = 0;                                   // pieces of S issued in all, of the current step
-        uint32_t phk = 0, phv = 0;
-        bool ok = true;
-        for (int it = 0; ok; ++it) {
-            if (!wait<true>(bar(WF + (it & 1)), (uint32_t)(it >> 1) & 1u, abort_flag)) { fail(19); break; }
-            const int n = work[it & 1].n_max;
-            if (n == 0) break;
-            arrive_remote(at_rank(bar(WE + (it & 1)), 0));
-            if (!wait(bar(QF), (uint32_t)it & 1u, abort_flag)) { fail(3); break; }
-            // The parts of P V are issued as they become ready, S of the next step in pieces in between: the chain
-            // P V(t) - rescale - P V(t+1) must not wait behind all of S (1024 clk), so at most two pieces are in flight.
-            int ju = 0, part = 0;                             // next step of S; next part of P V (two per tile)
-            uint32_t idle = 0;
-            while (part < 4 * n) {
-                if (++idle > 4 * WAIT_POLLS || ((idle & 63u) == 63u && flag(abort_flag))) {
-                    if (idle > 4 * WAIT_POLLS) fail(7);
-                    ok = false;
-                    break;
-                }
-                const uint32_t ph = (uint32_t)(t >> 1) & 1u, a = tmem + C::P_COL + (t & 1) * 32, acc0 = part >= 2 ? 1u : 0u;
-                const uint32_t b0 = v_lo + stv * (C::V_STAGE >> 4);
-                if ((part & 1) == 0 ? mbar_test_wait(bar(PG + (t & 1)), ph) && mbar_test_wait(bar(RL + (t & 1)), ph) && mbar_test_wait(bar(VF + stv), phv)
-                                    : mbar_test_wait(bar(RH + (t & 1)), ph)) {
-                    idle = 0;
-                    tc_fence_after();
-                    if ((part & 1) == 0) {
+            constexpr uint32_t idesc_s = umma_idesc_bf16(256, 2 * BC);
+            const uint32_t q_lo = umma_desc_lo(smem_base), k_lo = umma_desc_lo(k_s);
+            int st = 0, u = 0, sc = 0;                        // ring stage; steps, pieces of S issued
+            uint32_t ph = 0;
+            bool ok = true;
+            for (int it = 0; ok; ++it) {
+                if (!wait<true>(bar(WF + (it & 1)), (uint32_t)(it >> 1) & 1u, abort_flag)) { fail(19); break; }
+                const int n = work[it & 1].n_max;
+                if (n == 0) break;
+                arrive_remote(at_rank(bar(WE + (it & 1)), 0));
+                if (!wait(bar(QF), (uint32_t)it & 1u, abort_flag)) { fail(3); break; }
+                for (int j = 0; ok && j < n; ++j, ++u) {      // K halves landed, S(u-1) in registers
+                    if (!wait(bar(KF + st), ph, abort_flag)) { fail(4); ok = false; break; }
+                    if (u > 0 && !wait(bar(SFR), (uint32_t)(u - 1) & 1u, abort_flag)) { fail(6); ok = false; break; }
+                    // in pieces of 64 channels, at most two in flight: a P V that becomes ready meanwhile must not wait for all of S
+                    for (int ch = 0; ch < C::QSUB; ++ch, ++sc) {
+                        if (sc >= 2 && !wait(bar(SC + (sc & 1)), (uint32_t)((sc >> 1) - 1) & 1u, abort_flag)) { fail(2); ok = false; break; }
+                        tc_fence_after();
+                        const uint32_t a0 = q_lo + ch * (16384 >> 4), b0 = k_lo + st * (C::K_STAGE >> 4) + ch * (C::K_SUB >> 4);
 #pragma unroll
-                        for (int kk = 0; kk < 4; ++kk)        // 16 keys per step
-                            mma_ts(tmem, a + kk * 8, b0 + kk * 2, idesc_l, kk ? 1u : acc0);
-                        commit(bar(PL + (t & 1)));
-                    } else {
-#pragma unroll
-                        for (int kk = 0; kk < 4; ++kk)
-                            mma_ts(tmem + C::HI_COL, a + kk * 8, b0 + (C::V_HI >> 4) + kk * 2, idesc_h, kk ? 1u : acc0);
-                        commit(bar(PH + (t & 1)));
-                        commit(bar(VE + stv));
-                        if (++stv == C::V_STAGES) { stv = 0; phv ^= 1u; }
-                        ++t;
+                        for (int kk = 0; kk < 4; ++kk)        // 16 channels per step
+                            mma_ss(tmem + C::S_COL, a0 + kk * 2, b0 + kk * 2, idesc_s, (ch | kk) ? 1u : 0u);
+                        commit_local(bar(SC + (sc & 1)));
                     }
-                    ++part;
+                    if (!ok) break;
+                    commit(bar(SF));
+                    commit(bar(KE + st));
+                    if (++st == C::K_STAGES) { st = 0; ph ^= 1u; }
                 }
-                if (ju < n && (sc >= 2 ? mbar_test_wait(bar(SC + (sc & 1)), (uint32_t)((sc >> 1) - 1) & 1u) : true) &&
-                    (ch > 0 || ((us == 0 || mbar_test_wait(bar(SFR), (uint32_t)(us - 1) & 1u)) && mbar_test_wait(bar(KF + stk), phk)))) {
-                    idle = 0;
+                if (ok) commit(bar(QD));
+            }
+        }
+    } else if (rank == 0) {
+        // ------------------------------------------------------------------ issuers of [O | l] += P-hat [V | 1] (CTA 0), a part each
+        if (elect_one()) {
+            const int hi = warp - C::W_PV;
+            const uint32_t idesc = hi ? umma_idesc_bf16(256, D / 2 + 32) : umma_idesc_bf16(256, D / 2);
+            const uint32_t d = tmem + (hi ? C::HI_COL : 0), b_lo = umma_desc_lo(v_s + (hi ? C::V_HI : 0));
+            const uint32_t go = bar(hi ? GH : GL), part = bar(hi ? PH : PL);
+            int st = 0, t = 0;                                // ring stage, tile
+            uint32_t ph = 0;
+            bool ok = true;
+            for (int it = 0; ok; ++it) {
+                if (!wait<true>(bar(WF + (it & 1)), (uint32_t)(it >> 1) & 1u, abort_flag)) { fail(22); break; }
+                const int n_tiles = 2 * work[it & 1].n_max;
+                if (n_tiles == 0) break;
+                arrive_remote(at_rank(bar(WE + (it & 1)), 0));
+                for (int jt = 0; jt < n_tiles; ++jt, ++t) {   // V^T halves landed; P-hat stored and this part rescaled
+                    if (!wait(bar(VF + st), ph, abort_flag)) { fail(9); ok = false; break; }
+                    if (!wait(go + 8 * (t & 1), (uint32_t)(t >> 1) & 1u, abort_flag)) { fail(7); ok = false; break; }
                     tc_fence_after();
-                    const uint32_t a0 = q_lo + ch * (16384 >> 4), b0 = k_lo + stk * (C::K_STAGE >> 4) + ch * (C::K_SUB >> 4);
+                    const uint32_t a = tmem + C::P_COL + (t & 1) * 32, b0 = b_lo + st * (C::V_STAGE >> 4), acc0 = jt > 0 ? 1u : 0u;
 #pragma unroll
-                    for (int kk = 0; kk < 4; ++kk)            // 16 channels per step
-                        mma_ss(tmem + C::S_COL, a0 + kk * 2, b0 + kk * 2, idesc_s, (ch | kk) ? 1u : 0u);
-                    commit_local(bar(SC + (sc & 1)));
-                    ++sc;
-                    if (++ch == 4) {
-                        ch = 0;
-                        commit(bar(SF));
-                        commit(bar(KE + stk));
-                        if (++ju == n) commit(bar(QD));
-                        ++us;
-                        if (++stk == C::K_STAGES) { stk = 0; phk ^= 1u; }
-                    }
+                    for (int kk = 0; kk < 4; ++kk) mma_ts(d, a + kk * 8, b0 + kk * 2, idesc, kk ? 1u : acc0);      // 16 keys per step
+                    commit(part + 8 * (t & 1));
+                    commit(bar(PV + st));
+                    if (++st == C::V_STAGES) { st = 0; ph ^= 1u; }
                 }
             }
         }
-    }
     }
 
     tc_fence_before();
@@ -665,7 +668,7 @@ static int launch_cta2(const hifa4_shape& sh, const hifa4_qkv& qkv, const AttnAr
     CUtensorMap mq, mk, mv;
     if (!make_bf16_map(&mq, qkv.q_mma, (uint64_t)sh.B * sh.Hq, sh.N, C::D, 128)) return HIFA4_ERR_CUDA;
     if (!make_bf16_map(&mk, qkv.k_mma, (uint64_t)sh.B * sh.Hkv, sh.N, C::D, 64)) return HIFA4_ERR_CUDA;
-    if (!make_bf16_map(&mv, qkv.v_mma, (uint64_t)sh.B * sh.Hkv, C::D, sh.N, 64)) return HIFA4_ERR_CUDA;
+    if (!make_bf16_map(&mv, qkv.v_mma, (uint64_t)sh.B * sh.Hkv, C::D, sh.N, C::V_ROWS)) return HIFA4_ERR_CUDA;
     auto kern = attention_fwd_cta2_kernel<QM>;
     static SmemOptIn opt_in;
     if (!opt_in.ensure(kern, C::SMEM_BYTES)) return HIFA4_ERR_CUDA;
