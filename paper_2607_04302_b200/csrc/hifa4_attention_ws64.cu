@@ -28,6 +28,10 @@
 //   d = 128: 256 tensor-memory columns: [O | l] 0..143 (one N = 144 MMA), S 144..207, P-hat
 //            208..239; Q-hat stays in shared memory (SS-form Q K^T).  101 KB of shared memory, so two
 //            CTAs share an SM and fill each other's synchronisation gaps.
+// Where there is no second block for every SM (four_groups_pay below), d = 64 and 128 run with four groups of softmax warps,
+// 16 in all, one CTA per SM: then a tile's own work (2500 clk in a group) limits two groups to 1250 clk per tile, and four
+// of them to the chain P V(j) - rescale - P V(j+1), about 1000.  With the tensor memory of the absent CTA, S has two buffers
+// and every group its own P-hat columns, so that only a warp that rescales waits for the previous P V.
 // The issuers sit inside `if (elect_one())`, not `if (lane == 0)`: the compiler then knows that one thread runs the code, and
 // an MMA of M = 128, K = 16 takes 9 clk at N = 16, 32 at N = 64 with A in tensor memory, 48 with A in shared memory, 64 at
 // N = 128, instead of 62, 62, 62 and 68 (d = 256, N = 8192, 16 heads, causal: 519 -> 487 us, 550 -> 544 under the power cap).
@@ -45,10 +49,11 @@ namespace hifa4 {
 
 // F8: the kind::f8f6f4 experiment (d = 128): Q and K tiles are one byte per element, S has one accumulator per
 // 64-channel group, 304 tensor-memory columns, hence one CTA per SM.
-template <int D_, bool F8 = false>
+template <int D_, bool F8 = false, int NG_ = 2>
 struct WS64 {
     static constexpr int D = D_, BC = 64, STAGES = 2;
-    static constexpr int NSW = 8, THREADS = (NSW + 2) * 32, W_QK = NSW, W_PV = NSW + 1;   // two groups of 4 softmax warps
+    static constexpr int NG = NG_;                          // groups of 4 softmax warps; group g owns the tiles jt % NG == g
+    static constexpr int NSW = 4 * NG, THREADS = (NSW + 2) * 32, W_QK = NSW, W_PV = NSW + 1;
     static constexpr int NU = BC / 8;                       // 8 level-2 units (64 keys) per thread and tile
     static constexpr int QSUB = D / 64;                     // 64-channel sub-tiles of Q and K
     static constexpr int Q_BYTES = F8 ? 128 * D : QSUB * 16384;
@@ -61,9 +66,9 @@ struct WS64 {
     static constexpr int MISC_OFF = V_OFF + STAGES * V_STAGE;
     static constexpr int KSUM_SLOTS = 8;                    // Q-Mean: channel sums of a tile's 64 keys; slot = tile % 8
     static constexpr int KSUM_BYTES = F8 ? 512 : 256;       // (F8: the two group scales of each of the tile's keys instead)
-    static constexpr int KSUM_OFF = MISC_OFF + 256;
-    static constexpr int MX_OFF = KSUM_OFF + KSUM_SLOTS * KSUM_BYTES;  // running maxima handed from tile j to tile j+1: [2][128] floats
-    static constexpr int SMEM_USED = MX_OFF + 2 * 512 + 1024;
+    static constexpr int KSUM_OFF = MISC_OFF + 512;
+    static constexpr int MX_OFF = KSUM_OFF + KSUM_SLOTS * KSUM_BYTES;  // running maxima handed from tile j to tile j+1: [NG][128] floats
+    static constexpr int SMEM_USED = MX_OFF + NG * 512 + 1024;
     // F8 allocates all 512 tensor-memory columns: it asks for more than half of the SM's shared memory as well, so
     // that a second CTA never becomes resident only to block in the tensor-memory allocator
     static constexpr int SMEM_BYTES = (F8 && SMEM_USED < 120 * 1024) ? 120 * 1024 : SMEM_USED;
@@ -71,19 +76,20 @@ struct WS64 {
     static constexpr bool Q_IN_TMEM = (D == 256);
     static constexpr int QT_COL = 272;                      // d = 256 only
     static constexpr int S_COL = (D == 256) ? 400 : 144;
-    static constexpr int P_COL = S_COL + (F8 ? 128 : 64);
-    static constexpr int TMEM_COLS = (D == 256 || F8) ? 512 : 256;
-    static constexpr int CTAS_PER_SM = (D == 256 || F8) ? 1 : 2;
+    static constexpr int SB = NG > 2 ? 2 : 1;               // buffers for S; four groups also have a P-hat buffer each
+    static constexpr int P_COL = S_COL + (F8 ? 128 : 64 * SB);
+    static constexpr int TMEM_COLS = (D == 256 || F8 || NG > 2) ? 512 : 256;
+    static constexpr int CTAS_PER_SM = (D == 256 || F8 || NG > 2) ? 1 : 2;
 };
 namespace ws64 {
-// Index s = tile % 2 everywhere.  QKGO[s]: K stage s has landed and S is free (4 arrivals + 1 + bytes); PVGO[s]:
-// V^T stage s has landed, the image of P-hat is stored and [O | l] rescaled (4 arrivals + 1 + bytes); KE / VE:
-// stage free (MMA commit); SF[s]: S complete; PV[s]: P V complete; MR[s]: running maxima after the tile
-// published (4 arrivals); KSF[tile % 8]: Q-Mean key sums landed (a barrier per slot); QT: Q-hat image copied to tensor memory.
-// Two barriers per kind because each group of softmax warps sees every second tile only: a parity wait
-// must observe every phase of its barrier.
-enum { BAR_Q = 0, BAR_QKGO = 1, BAR_KE = 3, BAR_PVGO = 5, BAR_VE = 7, BAR_SF = 9, BAR_PV = 11, BAR_KSF = 13,
-       BAR_MR = 21, BAR_QT = 23, N_BARS = 24 };
+// QKGO[tile % 2]: K stage has landed and S is free (4 arrivals + 1 + bytes); PVGO[tile % NG]: V^T stage has landed, the
+// image of P-hat is stored and [O | l] rescaled (4 arrivals + 1 + bytes); KE / VE[tile % 2]: stage free (MMA commit);
+// SF[tile % NG]: S complete; PV[tile % NG]: P V complete; MR[tile % NG]: running maxima after the tile published (4
+// arrivals); KSF[tile % 8]: Q-Mean key sums landed (a barrier per slot); QT: Q-hat image copied to tensor memory.
+// NG barriers where each group of softmax warps sees every NG-th tile only: a parity wait must observe every phase of its
+// barrier.
+enum { BAR_Q = 0, BAR_QKGO = 1, BAR_KE = 3, BAR_VE = 5, BAR_PVGO = 7, BAR_SF = 11, BAR_PV = 15, BAR_KSF = 19,
+       BAR_MR = 27, BAR_QT = 31, N_BARS = 32 };
 constexpr uint32_t WAIT_POLLS = 1u << 18;            // a poll may keep the thread suspended for up to about 4 us
 }  // namespace ws64
 
@@ -117,13 +123,14 @@ static __device__ __forceinline__ void arrive_lane0(uint32_t bar, int lane)
 // to 28, exact) with one FP32 scale S/4 per (row, 64-channel group); S = Q K^T runs as two accumulators, one per
 // channel group, and the softmax threads bind them: acc = (qs0 ks0_j) S0 + (qs1 ks1_j) S1, every product exact and
 // the sum rounded once.  Measured against the BF16-image form, not a default path.
-template <int DH, bool DBG, bool PF32, bool QM, bool SELFTEST = false, bool QRAW = false, bool F8QK = false>
-__global__ void __launch_bounds__(WS64<DH, F8QK>::THREADS, WS64<DH, F8QK>::CTAS_PER_SM)
+template <int DH, bool DBG, bool PF32, bool QM, bool SELFTEST = false, bool QRAW = false, bool F8QK = false, int NG = 2>
+__global__ void __launch_bounds__(WS64<DH, F8QK, NG>::THREADS, WS64<DH, F8QK, NG>::CTAS_PER_SM)
 attention_fwd_ws64_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ CUtensorMap tmap_k,
                            const __grid_constant__ CUtensorMap tmap_v, const __grid_constant__ AttnArgs args)
 {
     using namespace ws64;
-    using C = WS64<DH, F8QK>;
+    using C = WS64<DH, F8QK, NG>;
+    static_assert(NG == 2 || (DH != 256 && !DBG && !PF32 && !SELFTEST && !QRAW && !F8QK), "four groups: the plain paths");
     static_assert(!QRAW || (DH == 128 && !QM && !DBG), "raw-Q launch: d = 128, no Q-Mean, no dump");
     static_assert(!F8QK || (DH == 128 && !QM && !DBG && !QRAW && !SELFTEST), "f8f6f4 experiment: d = 128, plain path");
     constexpr int D = C::D, BC = C::BC, STAGES = C::STAGES, NSW = C::NSW, THREADS = C::THREADS;
@@ -186,8 +193,8 @@ attention_fwd_ws64_kernel(const __grid_constant__ CUtensorMap tmap_q, const __gr
     };
     auto load_v = [&](int jt) {                               // V^T tile jt into stage jt % 2
         const int st = jt & 1;
-        mbar_expect_tx(bar(BAR_PVGO + st), D * 128);
-        tma_load_3d(v_s + st * V_STAGE, &tmap_v, bar(BAR_PVGO + st), jt * BC, 0, bh_kv);
+        mbar_expect_tx(bar(BAR_PVGO + (jt & (NG - 1))), D * 128);
+        tma_load_3d(v_s + st * V_STAGE, &tmap_v, bar(BAR_PVGO + (jt & (NG - 1))), jt * BC, 0, bh_kv);
     };
 
     if (warp == W_QK && lane == 0) {
@@ -200,10 +207,11 @@ attention_fwd_ws64_kernel(const __grid_constant__ CUtensorMap tmap_q, const __gr
         mbar_init(bar(BAR_Q), 1);
         for (int s = 0; s < STAGES; ++s) {
             mbar_init(bar(BAR_QKGO + s), 5); mbar_init(bar(BAR_KE + s), 1);
-            mbar_init(bar(BAR_PVGO + s), 5); mbar_init(bar(BAR_VE + s), 1);
-            mbar_init(bar(BAR_SF + s), 1); mbar_init(bar(BAR_PV + s), 1);
+            mbar_init(bar(BAR_VE + s), 1);
             for (int t = 0; t < 4; ++t) mbar_init(bar(BAR_KSF + 2 * t + s), 1);
-            mbar_init(bar(BAR_MR + s), 4);
+        }
+        for (int s = 0; s < NG; ++s) {
+            mbar_init(bar(BAR_PVGO + s), 5); mbar_init(bar(BAR_SF + s), 1); mbar_init(bar(BAR_PV + s), 1); mbar_init(bar(BAR_MR + s), 4);
         }
         mbar_init(bar(BAR_QT), NSW);
         fence_barrier_init();
@@ -269,10 +277,10 @@ attention_fwd_ws64_kernel(const __grid_constant__ CUtensorMap tmap_q, const __gr
                     for (int kk = 0; kk < D / 16; ++kk) {      // D / 16 steps of 16 channels
                         const uint32_t kb = b0 + (kk >> 2) * (K_SUB >> 4) + (kk & 3) * 2;
                         if constexpr (C::Q_IN_TMEM) umma_bf16_ts_lo(tmem + S_COL, tmem + QT_COL + kk * 8, kb, idesc_s, kk ? 1u : 0u);
-                        else umma_bf16_ss_lo(tmem + S_COL, q_lo + (kk >> 2) * (16384 >> 4) + (kk & 3) * 2, kb, idesc_s, kk ? 1u : 0u);
+                        else umma_bf16_ss_lo(tmem + S_COL + (C::SB > 1 ? st * 64 : 0), q_lo + (kk >> 2) * (16384 >> 4) + (kk & 3) * 2, kb, idesc_s, kk ? 1u : 0u);
                     }
                 }
-                umma_commit(bar(BAR_SF + st));
+                umma_commit(bar(BAR_SF + (jt & (NG - 1))));
                 umma_commit(bar(BAR_KE + st));
                 if (jt + 2 < n_tiles) {                        // refill the stage once this MMA has read it
                     if (!wait64(bar(BAR_KE + st), ph, abort_flag)) { fail(1); break; }
@@ -291,17 +299,17 @@ attention_fwd_ws64_kernel(const __grid_constant__ CUtensorMap tmap_q, const __gr
             for (int jt = 0; jt < n_tiles; ++jt) {            // V^T tile landed, P-hat(jt) stored, history rescaled
                 const int st = jt & 1;
                 const uint32_t ph = (uint32_t)(jt >> 1) & 1u;
-                if (!wait64(bar(BAR_PVGO + st), ph, abort_flag, SELFTEST ? (1u << 6) : WAIT_POLLS)) { fail(7); break; }
+                if (!wait64(bar(BAR_PVGO + (jt & (NG - 1))), (uint32_t)(jt / NG) & 1u, abort_flag, SELFTEST ? (1u << 6) : WAIT_POLLS)) { fail(7); break; }
                 tc_fence_after();
                 const uint32_t b0 = v_lo + st * (V_STAGE >> 4);
                 const uint32_t acc0 = jt > 0 ? 1u : 0u;
 #pragma unroll
                 for (int kk = 0; kk < 4; ++kk) {                // 16 keys per step; channels (+ ones block)
-                    umma_bf16_ts_lo(tmem, tmem + P_COL + kk * 8, b0 + kk * 2, idesc_o, kk ? 1u : acc0);
+                    umma_bf16_ts_lo(tmem, tmem + P_COL + (NG > 2 ? (jt & (NG - 1)) * 32 : 0) + kk * 8, b0 + kk * 2, idesc_o, kk ? 1u : acc0);
                     if constexpr (D == 256)                      // N = 272 does not exist: two parts, the ones block in the second
                         umma_bf16_ts_lo(tmem + 128, tmem + P_COL + kk * 8, b0 + ((128 * 128) >> 4) + kk * 2, idesc_h, kk ? 1u : acc0);
                 }
-                umma_commit(bar(BAR_PV + st));
+                umma_commit(bar(BAR_PV + (jt & (NG - 1))));
                 umma_commit(bar(BAR_VE + st));
                 if (jt + 2 < n_tiles) {                        // refill the stage once this MMA has read it
                     if (!wait64(bar(BAR_VE + st), ph, abort_flag)) { fail(2); break; }
@@ -311,7 +319,7 @@ attention_fwd_ws64_kernel(const __grid_constant__ CUtensorMap tmap_q, const __gr
         }
     } else {
         // ------------------------------------------------------------------ softmax / quantize
-        const int grp = warp >> 2, quarter = warp & 3;            // tile parity owned, row quarter
+        const int grp = warp >> 2, quarter = warp & 3;            // tiles owned, row quarter
         const int kq = grp;                                       // channel half in the Q-hat copy and in the epilogue
         const int r_loc = quarter * 32 + lane;                    // row inside the tile = TMEM lane
         const int row = q0 + r_loc;
@@ -329,7 +337,7 @@ attention_fwd_ws64_kernel(const __grid_constant__ CUtensorMap tmap_q, const __gr
             qs0 = args.q_gs[((size_t)bh_q * N + row) * 2];
             qs1 = args.q_gs[((size_t)bh_q * N + row) * 2 + 1];
         }
-        float* mx_s = reinterpret_cast<float*>(smem_gen + C::MX_OFF);   // [2][128]
+        float* mx_s = reinterpret_cast<float*>(smem_gen + C::MX_OFF);   // [NG][128]
         float m_run = -INFINITY;
         bool ok = true;
 
@@ -369,13 +377,15 @@ attention_fwd_ws64_kernel(const __grid_constant__ CUtensorMap tmap_q, const __gr
             __syncwarp();
             arrive_lane0(bar(BAR_QT), lane);
         }
-        if (grp == 0) arrive_lane0(bar(BAR_QKGO), lane);          // S is free for tile 0
+        if (grp < C::SB) arrive_lane0(bar(BAR_QKGO + grp), lane); // the S buffers are free for the first tiles
 
-        for (int jt = grp; ok && jt < n_tiles; jt += 2) {
+        const int g_prev = (grp + NG - 1) & (NG - 1);             // the owner of the tile before
+        for (int jt = grp; ok && jt < n_tiles; jt += NG) {
             const int j0 = jt * BC;
-            const int st = jt & 1;                                 // = grp
-            const uint32_t ph = (uint32_t)(jt >> 1) & 1u;          // phase parity of this group's barriers
-            if (!wait64(bar(BAR_SF + st), ph, abort_flag)) { fail(8); ok = false; break; }
+            const int st = jt & 1;
+            const uint32_t ph = (uint32_t)(jt / NG) & 1u;          // phase parity of this group's barriers
+            const uint32_t ph_prev = (uint32_t)((jt - 1) / NG) & 1u;
+            if (!wait64(bar(BAR_SF + grp), ph, abort_flag)) { fail(8); ok = false; break; }
             tc_fence_after();
             float p[BC];
             if constexpr (F8QK) {
@@ -400,15 +410,16 @@ attention_fwd_ws64_kernel(const __grid_constant__ CUtensorMap tmap_q, const __gr
                 }
             } else {
                 uint32_t r[BC];
-                tmem_ld32(t_lane + S_COL, reinterpret_cast<uint32_t(&)[32]>(r[0]));
-                tmem_ld32(t_lane + S_COL + 32, reinterpret_cast<uint32_t(&)[32]>(r[32]));
+                const uint32_t t_s = t_lane + S_COL + (C::SB > 1 ? st * 64 : 0);
+                tmem_ld32(t_s, reinterpret_cast<uint32_t(&)[32]>(r[0]));
+                tmem_ld32(t_s + 32, reinterpret_cast<uint32_t(&)[32]>(r[32]));
                 tmem_wait_ld();
 #pragma unroll
                 for (int i = 0; i < BC; ++i) p[i] = __uint_as_float(r[i]);
             }
-            tc_fence_before();                                 // S(jt) is in registers: S(jt+1) may overwrite it
+            tc_fence_before();                                 // S(jt) is in registers: S(jt+SB) may overwrite it
             __syncwarp();
-            if (jt + 1 < n_tiles) arrive_lane0(bar(BAR_QKGO + (st ^ 1)), lane);
+            if (jt + C::SB < n_tiles) arrive_lane0(bar(BAR_QKGO + ((jt + C::SB) & 1)), lane);
 
             if (QM) {                                          // Q-Mean correction (line 6): + mu_i * sum_c k~_jc
                 if (!wait64(bar(BAR_KSF + (jt & 7)), (uint32_t)(jt >> 3) & 1u, abort_flag)) { fail(15); ok = false; break; }
@@ -428,18 +439,18 @@ attention_fwd_ws64_kernel(const __grid_constant__ CUtensorMap tmap_q, const __gr
                 for (int i = 0; i < BC; ++i) p[i] = (j0 + i > key_lim) ? -INFINITY : p[i];
             }
             const float mx = max64(p);                         // row maximum = maximum of the tile's single 64-key group
-            // running maximum after the previous tile, from its owner (the other group)
+            // running maximum after the previous tile, from its owner
             if (jt > 0) {
-                if (!wait64(bar(BAR_MR + (st ^ 1)), (uint32_t)((jt - 1) >> 1) & 1u, abort_flag)) { fail(12); ok = false; break; }
-                m_run = mx_s[(st ^ 1) * 128 + r_loc];
+                if (!wait64(bar(BAR_MR + g_prev), ph_prev, abort_flag)) { fail(12); ok = false; break; }
+                m_run = mx_s[g_prev * 128 + r_loc];
             }
             // running maximum and rescale factor (lines 7-8), both FP16 values.  No branch: r = 1 exactly
             // when the maximum did not move; at jt = 0 (m = -inf) r = 0 is never applied.
             const float m_new = fmaxf(m_run, f16_round(mx * args.c0));
             if (jt + 1 < n_tiles) {                            // hand it to the owner of the next tile
-                mx_s[st * 128 + r_loc] = m_new;
+                mx_s[grp * 128 + r_loc] = m_new;
                 __syncwarp();
-                arrive_lane0(bar(BAR_MR + st), lane);
+                arrive_lane0(bar(BAR_MR + grp), lane);
             }
             const float rsc = f16_round(ex2_approx((m_run - m_new) * LOG2E));
             m_run = m_new;
@@ -457,21 +468,39 @@ attention_fwd_ws64_kernel(const __grid_constant__ CUtensorMap tmap_q, const __gr
             uint32_t w[NU * 4];
             const auto qc = p_quant_const<PF32>(args.c1, mL, A);
             exp_quantize_units<NU, 0, NU, DBG, PF32>(p, qc, A == 0.f, w, dc, ds);
-            // the P-hat columns and [O | l] are free once P V of the previous tile has completed
-            if (jt > 0) {
-                if (!wait64(bar(BAR_PV + (st ^ 1)), (uint32_t)((jt - 1) >> 1) & 1u, abort_flag)) { fail(10); ok = false; break; }
-                tc_fence_after();
+            if constexpr (NG > 2) {
+                // the group's P-hat columns are free once P V(jt-NG) has completed; only a rescale waits for P V(jt-1)
+                if (jt >= NG) {
+                    if (!wait64(bar(BAR_PV + grp), (uint32_t)(jt / NG - 1) & 1u, abort_flag)) { fail(9); ok = false; break; }
+                    tc_fence_after();
+                }
+                tmem_st32(t_lane + P_COL + grp * 32, w);
+                if (jt > 0 && __any_sync(0xffffffffu, rsc != 1.f)) {
+                    if (!wait64(bar(BAR_PV + g_prev), ph_prev, abort_flag)) { fail(10); ok = false; break; }
+                    tc_fence_after();
+                    rescale_columns<D>(t_lane, rsc);           // history (line 8)
+                }
+            } else {
+                // the P-hat columns and [O | l] are free once P V of the previous tile has completed
+                if (jt > 0) {
+                    if (!wait64(bar(BAR_PV + g_prev), ph_prev, abort_flag)) { fail(10); ok = false; break; }
+                    tc_fence_after();
+                }
+                tmem_st32(t_lane + P_COL, w);
+                if (jt > 0 && __any_sync(0xffffffffu, rsc != 1.f)) rescale_columns<D>(t_lane, rsc);   // history (line 8)
             }
-            tmem_st32(t_lane + P_COL, w);
-            if (jt > 0 && __any_sync(0xffffffffu, rsc != 1.f)) rescale_columns<D>(t_lane, rsc);   // history (line 8)
             tmem_wait_st();
             tc_fence_before();
             __syncwarp();
-            if (!SELFTEST) arrive_lane0(bar(BAR_PVGO + st), lane);
+            if (!SELFTEST) arrive_lane0(bar(BAR_PVGO + grp), lane);
         }
 
-        // finalize: out = O / l with l rounded to FP16 (line 13); half kq writes channels (d/2)*kq..
-        if (ok && wait64(bar(BAR_PV + ((n_tiles - 1) & 1)), (uint32_t)((n_tiles - 1) >> 1) & 1u, abort_flag)) {
+        if (NG > 2 && ok && grp < 2 && grp < n_tiles) {        // first the group's own last P V: only then can the wait for the
+            const int k = (n_tiles - 1 - grp) / NG;             // last one not be two phases behind
+            if (!wait64(bar(BAR_PV + grp), (uint32_t)k & 1u, abort_flag)) { fail(14); ok = false; }
+        }
+        // finalize: out = O / l with l rounded to FP16 (line 13); groups 0 and 1, half kq writes channels (d/2)*kq..
+        if (ok && grp < 2 && wait64(bar(BAR_PV + ((n_tiles - 1) & (NG - 1))), (uint32_t)((n_tiles - 1) / NG) & 1u, abort_flag)) {
             tc_fence_after();
             constexpr int NC = D / 2 / 32;                     // 32-column chunks of this thread's channel half
             uint32_t lr[4], rbuf[2][32];
@@ -542,7 +571,7 @@ attention_fwd_ws64_kernel(const __grid_constant__ CUtensorMap tmap_q, const __gr
                 }
                 if (cc + 1 < NC) tmem_wait_ld();
             }
-        } else if (ok) {
+        } else if (ok && grp < 2) {
             fail(11);
         }
     }
@@ -554,10 +583,10 @@ attention_fwd_ws64_kernel(const __grid_constant__ CUtensorMap tmap_q, const __gr
 
 bool make_u8_map(CUtensorMap* m, void* base, uint64_t heads, uint64_t rows, uint64_t cols, uint32_t box_rows);
 
-template <int DH, bool DBG, bool PF32, bool QM, bool SELFTEST = false, bool QRAW = false, bool F8QK = false>
+template <int DH, bool DBG, bool PF32, bool QM, bool SELFTEST = false, bool QRAW = false, bool F8QK = false, int NG = 2>
 static int launch_ws64(const hifa4_shape& sh, const hifa4_qkv& qkv, const AttnArgs& args, cudaStream_t st)
 {
-    using C = WS64<DH, F8QK>;
+    using C = WS64<DH, F8QK, NG>;
     CUtensorMap mq, mk, mv;
     if constexpr (F8QK) {
         if (!make_u8_map(&mq, const_cast<void*>(args.q_f8), (uint64_t)sh.B * sh.Hq, sh.N, DH, 128)) return HIFA4_ERR_CUDA;
@@ -567,11 +596,25 @@ static int launch_ws64(const hifa4_shape& sh, const hifa4_qkv& qkv, const AttnAr
         if (!make_bf16_map(&mk, qkv.k_mma, (uint64_t)sh.B * sh.Hkv, sh.N, DH, C::BC)) return HIFA4_ERR_CUDA;
     }
     if (!make_bf16_map(&mv, qkv.v_mma, (uint64_t)sh.B * sh.Hkv, DH, sh.N, DH)) return HIFA4_ERR_CUDA;
-    auto kern = attention_fwd_ws64_kernel<DH, DBG, PF32, QM, SELFTEST, QRAW, F8QK>;
+    auto kern = attention_fwd_ws64_kernel<DH, DBG, PF32, QM, SELFTEST, QRAW, F8QK, NG>;
     static SmemOptIn opt_in;
     if (!opt_in.ensure(kern, C::SMEM_BYTES)) return HIFA4_ERR_CUDA;
     const unsigned grid = (unsigned)(((sh.N + 127) / 128) * sh.Hq * sh.B);
     return launch_dependent(kern, grid, C::THREADS, C::SMEM_BYTES, st, mq, mk, mv, args) == cudaSuccess ? HIFA4_OK : HIFA4_ERR_CUDA;
+}
+
+// Whether four groups of softmax warps, one block per SM, are faster than two groups and two blocks per SM (d = 64 and 128):
+// as long as every block has an SM to itself (d = 64: N = 1024, 8 heads 14.1 -> 12.5 us, N = 4096, 4 heads 44 -> 36; d = 128:
+// 16.7 -> 16.2, 50 -> 47), and under a causal mask, where the last blocks are short ones, a good way beyond (256 blocks:
+// d = 64, N = 2048 27.6 -> 23.8, 4096 49 -> 37, 8192 91 -> 66; d = 128 32.2 -> 30.6, 56 -> 48, 102 -> 84; 288 blocks N = 1536
+// 22.6 -> 22.0 and 26.7 -> 27.9; 320 blocks N = 2048 29.5 -> 32.4 and 34 -> 41), less far for short rows (N = 1024: 192 blocks
+// 15.3 -> 14.0 and 18.4 -> 16.8, 256 blocks 16.6 -> 17.0 and 20.1 -> 21.0; non-causal, 256 blocks 22.6 -> 24.8, 39.1 -> 40.4).
+static bool four_groups_pay(const hifa4_shape& sh, const AttnArgs& args)
+{
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return false;
+    const long long blocks = (long long)((sh.N + 127) / 128) * sh.Hq * sh.B;
+    return blocks <= sms || (args.causal && (3 * blocks <= 4 * sms || (sh.N > 1024 && 4 * blocks <= 7 * sms)));
 }
 
 template <int DH>
@@ -599,6 +642,11 @@ static int launch_ws64_d(const hifa4_shape& sh, const hifa4_qkv& qkv, const Attn
             if (args.qmean) return HIFA4_ERR_UNSUPPORTED;
             return dbg ? launch_ws64<DH, true, true, false>(sh, qkv, args, st) : launch_ws64<DH, false, true, false>(sh, qkv, args, st);
         }
+    }
+    if constexpr (DH != 256) {
+        if (!dbg && four_groups_pay(sh, args))
+            return args.qmean ? launch_ws64<DH, false, false, true, false, false, false, 4>(sh, qkv, args, st)
+                              : launch_ws64<DH, false, false, false, false, false, false, 4>(sh, qkv, args, st);
     }
     if (args.qmean)
         return dbg ? launch_ws64<DH, true, false, true>(sh, qkv, args, st) : launch_ws64<DH, false, false, true>(sh, qkv, args, st);
