@@ -37,3 +37,17 @@ def test_scan_matches_torch(S, Hq, Hkv, N, d, dtype, head_map):
     p99 = float(mag[int(np.ceil(0.99 * mag.size)) - 1])
     top_k, top_q = float(mag[-1]), float(q.float().abs().max())
     assert stats[0].item() == np.float32(top_k / p99) and stats[1].item() == np.float32(top_k / top_q)
+
+
+@pytest.mark.parametrize("S", [1, 2, 99, 100, 101, 200, 301])
+def test_p99_aggregator_is_the_nearest_rank(S):
+    """Around the sample counts where the rank leaves the maximum, with ties at the top (a magnitude out of five per sample)."""
+    from paper_2607_04302_b200 import binding as hb
+    gen = torch.Generator(device=DEV).manual_seed(S)
+    q, k = (torch.randint(1, 6, (S, 2, 3, 64), generator=gen, device=DEV).bfloat16() for _ in range(2))
+    k[:, :, :, 7] = 0                                                    # an aggregate of zero: s = 1
+    rank = max(1, -(-99 * S // 100))
+    kagg, qagg = (t.float().abs().amax(2).sort(0).values[rank - 1].double() for t in (k, q))
+    s, _ = hb.smooth_calibrate(q, k, hb.MODE_STRONG | hb.AGG_P99)
+    want = torch.where(kagg > 0, (kagg / qagg).sqrt(), torch.ones_like(kagg))
+    assert torch.allclose(s.double(), want, rtol=1e-6, atol=0)           # double pow on both sides, rounded once
