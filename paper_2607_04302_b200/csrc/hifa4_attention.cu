@@ -450,7 +450,7 @@ int launch_attention(const hifa4_shape& sh, const HeadMap& map, const hifa4_qkv&
         return HIFA4_ERR_UNSUPPORTED;
     }
     if (!q_raw && !f8 && a.dbg.n_blocks == 0 && attention_pair_pays(sh, prm))
-        return launch_attention_pair(sh, qkv, a, st);
+        return launch_attention_pair(sh, qkv, a, prm.Bc, st);
     if (!q_raw && !f8 && a.dbg.n_blocks == 0 && attention_cta2_pays(sh, prm, a.unit_heads))
         return launch_attention_cta2(sh, qkv, a, st);
     if (sh.d == 64 && prm.Bc == 64) return launch_attention_ws64(sh, qkv, a, st);

@@ -446,7 +446,7 @@ int launch_attention_ws(const hifa4_shape& sh, const hifa4_qkv& qkv, const AttnA
 // Warp-specialised kernels for Bc = 64, d = 64, 128 or 256 (hifa4_attention_ws64.cu).
 int launch_attention_ws64(const hifa4_shape& sh, const hifa4_qkv& qkv, const AttnArgs& args, cudaStream_t st);
 // The same with two query blocks per CTA that share the K / V tiles, d = 128 (hifa4_attention_pair.cu).
-int launch_attention_pair(const hifa4_shape& sh, const hifa4_qkv& qkv, const AttnArgs& args, cudaStream_t st);
+int launch_attention_pair(const hifa4_shape& sh, const hifa4_qkv& qkv, const AttnArgs& args, int Bc, cudaStream_t st);
 // The same on pairs of SMs, d = 256 (hifa4_attention_cta2.cu).
 bool attention_cta2_pays(const hifa4_shape& sh, const hifa4_attn_params& prm, int unit_heads);
 int launch_attention_cta2(const hifa4_shape& sh, const hifa4_qkv& qkv, const AttnArgs& args, cudaStream_t st);

@@ -1,4 +1,4 @@
-// Warp-specialised HiFA4 attention forward for Bc = 64, d = 128 (Algorithm 1 lines 4-13) with two 128-row query blocks per
+// Warp-specialised HiFA4 attention forward for Bc = 64 or 128, d = 128 (Algorithm 1 lines 4-13) with two 128-row query blocks per
 // CTA that share the K and V^T tiles.
 //
 // The two blocks ("halves") belong to query heads of one KV head, so every K and V^T tile is loaded once for 256
@@ -21,7 +21,9 @@
 // all pairs of a CTA (t per half, c for the tiles loaded); barrier phases follow those numbers.
 // Tensor memory, per half: [O | l] d+16 columns, S 64, P-hat 32 (2 x 240 of 512 columns at d = 128).  Output goes
 // through 2 KB of shared memory per warp, so that stores cover whole 64-byte row pieces.
-// Template flag: Q-Mean (key sums staged in eight slots by the loader, as in the 64-key kernel).
+// Template flags: Q-Mean (key sums staged in eight slots by the loader, as in the 64-key kernel); B128: 128-key tiles, each a
+// pair of 64-key ones whose owners exchange their maxima (one more hand-off per tile, one rescale less).  Against the
+// 128-key kernel (hifa4_attention_ws.cu), 32 / 8 heads, causal: N = 4096 213 -> 191 us, N = 8192 722 -> 637.
 // Every wait is bounded (see hifa4_attention_ws.cu for the failure protocol).
 #include "hifa4_attention.cuh"
 
@@ -37,8 +39,9 @@ struct PairCfg {
     static constexpr int K_OFF = 2 * Q_HALF;
     static constexpr int V_OFF = K_OFF + STAGES * K_STAGE;
     static constexpr int STG_OFF = V_OFF + STAGES * V_STAGE;   // output staging, 2 KB per softmax warp
-    static constexpr int MX_OFF = STG_OFF + NSW * 2048;     // running maxima handed from tile t to t+1: [half][t % 2][128] floats
-    static constexpr int KSUM_OFF = MX_OFF + 2 * 2 * 512;   // Q-Mean: channel sums of a tile's 64 keys, slot = tile % 8
+    static constexpr int MX_OFF = STG_OFF + NSW * 2048;     // running maxima handed from tile t to t+1: [half][t % 2][128] floats;
+                                                            // 128-key tiles: maxima of the halves of a tile, [half][t % 4][128]
+    static constexpr int KSUM_OFF = MX_OFF + 2 * 4 * 512;   // Q-Mean: channel sums of a tile's 64 keys, slot = tile % 8
     static constexpr int MISC_OFF = KSUM_OFF + 8 * 256;
     static constexpr int SMEM_BYTES = MISC_OFF + 1024 + 1024;
     static constexpr int O_COLS = D + 16;
@@ -50,12 +53,12 @@ struct PairCfg {
 namespace pairk {
 // Per half (HALF barriers each, half 1 after half 0): QF Q landed, QD last S of the pair complete (Q may be replaced), SFR
 // S buffer free (4 arrivals), SF[t % 2] S complete, PGO P-hat stored and history rescaled (4), PV[t % 2] P V complete,
-// MR[t % 2] running maxima published (4), OE output columns read (8).  Ring (index = stage): KF / VF tile landed, KE / VE
+// MR[t % 2] (128-key tiles: t % 4) maxima published (4), OE output columns read (8).  Ring (index = stage): KF / VF tile landed, KE / VE
 // tile read by both halves.  WF / WE[pair % 2]: work record written / read by all (20); CL: answer of the launch control;
 // KSF[tile % 8].  SF, PV and MR come in twos because each group of softmax warps sees every second tile only: a parity
 // wait must not be two phases behind.
-enum { QF = 0, QD = 1, SFR = 2, PGO = 3, SF = 4, PV = 6, MR = 8, OE = 10, HALF = 12,
-       KF = 24, KE = 27, VF = 30, VE = 33, WF = 36, WE = 38, CL = 40, KSF = 41, N_BARS = 49 };
+enum { QF = 0, QD = 1, SFR = 2, PGO = 3, SF = 4, PV = 6, MR = 8, OE = 12, HALF = 16,
+       KF = 32, KE = 35, VF = 38, VE = 41, WF = 44, WE = 46, CL = 48, KSF = 49, N_BARS = 57 };
 constexpr uint32_t WAIT_POLLS = 1u << 18;            // a poll may keep the thread suspended for up to about 4 us
 struct Work {                         // one pair of query blocks
     int n_max;                        // key tiles to load; 0: no more work
@@ -112,7 +115,7 @@ static __device__ __forceinline__ int launch_control_answer(uint32_t src)   // b
     return got ? (int)x : -1;
 }
 
-template <bool QM>
+template <bool QM, bool B128>
 __global__ void __launch_bounds__(PairCfg::THREADS, 1)
 attention_fwd_pair_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ CUtensorMap tmap_k,
                           const __grid_constant__ CUtensorMap tmap_v, const __grid_constant__ AttnArgs args)
@@ -147,8 +150,9 @@ attention_fwd_pair_kernel(const __grid_constant__ CUtensorMap tmap_q, const __gr
             const int b = h * HALF;
             mbar_init(bar(b + QF), 1); mbar_init(bar(b + QD), 1); mbar_init(bar(b + SFR), 4); mbar_init(bar(b + PGO), 4);
             for (int s = 0; s < 2; ++s) {
-                mbar_init(bar(b + SF + s), 1); mbar_init(bar(b + PV + s), 1); mbar_init(bar(b + MR + s), 4);
+                mbar_init(bar(b + SF + s), 1); mbar_init(bar(b + PV + s), 1);
             }
+            for (int s = 0; s < 4; ++s) mbar_init(bar(b + MR + s), 4);
             mbar_init(bar(b + OE), 8);
             mbar_init(bar(WF + h), 1); mbar_init(bar(WE + h), 20);
         }
@@ -206,7 +210,7 @@ attention_fwd_pair_kernel(const __grid_constant__ CUtensorMap tmap_q, const __gr
                     for (int hf = 0; hf < 2; ++hf) {
                         const int r = 2 * p + hf, qi = r / G, q0 = (n_qt - 1 - qi) * 128;
                         const int last_key = args.causal ? min(q0 + 127, N - 1) : N - 1;
-                        const int n = r < blocks ? last_key / BC + 1 : 0;
+                        const int n = r >= blocks ? 0 : B128 ? 2 * (last_key / 128 + 1) : last_key / BC + 1;
                         w.n[hf] = n;
                         w.q0[hf] = q0;
                         w.bh_q[hf] = b * args.Hq + h0 + (r - qi * G);
@@ -237,8 +241,10 @@ attention_fwd_pair_kernel(const __grid_constant__ CUtensorMap tmap_q, const __gr
                         if (QM) {
                             // slot c % 8 held the sums of tile c-8: this load follows S(c-3) of both halves, hence their pull
                             // of S(c-4) by the warps that read the slot during tile c-8 or by warps that waited for them since
+                            // (B128: a tile may lie past the last key; its scores are masked whatever is added to them)
+                            const int key = B128 ? min(jk * BC, N - BC) : jk * BC;
                             mbar_expect_tx(bar(KSF + (c & 7)), 256);
-                            bulk_load(smem_base + C::KSUM_OFF + (c & 7) * 256, args.k_sum + (size_t)bh_kv * N + jk * BC, 256, bar(KSF + (c & 7)));
+                            bulk_load(smem_base + C::KSUM_OFF + (c & 7) * 256, args.k_sum + (size_t)bh_kv * N + key, 256, bar(KSF + (c & 7)));
                             ++c;
                         }
                         if (jk == max(n_max - 3, 0)) launch_control_ask(smem_base + CL_OFF, bar(CL));
@@ -264,7 +270,7 @@ attention_fwd_pair_kernel(const __grid_constant__ CUtensorMap tmap_q, const __gr
         const int r_loc = quarter * 32 + lane;                    // row inside the block = TMEM lane
         const uint32_t t_o = tmem + ((uint32_t)(quarter * 32) << 16) + hf * C::H_COLS;   // [O | l], then S, then P-hat
         const float LOG2E = 1.4426950408889634f;
-        const uint32_t mx_own = smem_base + C::MX_OFF + hf * 1024 + grp * 512 + r_loc * 4;
+        const uint32_t mx_own = smem_base + C::MX_OFF + hf * 2048 + grp * 512 + r_loc * 4;
         const uint32_t b_h = bar(hf * HALF), b_own = b_h + 8 * grp, b_oth = b_own ^ 8;   // (b_h is a multiple of 16)
         int t0 = 0;                                               // tiles of this half before the current pair
         int c0 = 0;                                               // tiles loaded before the current pair
@@ -317,18 +323,31 @@ attention_fwd_pair_kernel(const __grid_constant__ CUtensorMap tmap_q, const __gr
                     for (int i = 0; i < BC; ++i) p[i] = (j0 + i > key_lim) ? -INFINITY : p[i];
                 }
                 const float mx = max64(p);                         // row maximum = maximum of the tile's single 64-key group
-                // running maximum after the previous tile, from its owner (the other group)
-                if (jt > 0) {
+                float oth = -INFINITY;
+                if constexpr (B128) {
+                    // 128-key tile = tiles t and t ^ 1: both groups take the maximum over both halves and keep the running
+                    // maximum for themselves; its second half finds the history rescaled.  Four slots and barriers: those
+                    // of tile t serve tile t+4, after P V(t+1), hence after the other group has read them.
+                    const float own = f16_round(mx * args.c0);
+                    const uint32_t sl = (uint32_t)(t & 2) * 512u, b_mr = b_h + 8 * MR + 8 * (t & 2);
+                    asm volatile("st.shared.f32 [%0], %1;" ::"r"(mx_own + sl), "f"(own) : "memory");
+                    __syncwarp();
+                    arrive0(b_mr + 8 * grp, lane);
+                    if (!wait_pair(b_mr + 8 * (grp ^ 1), (uint32_t)(t >> 2) & 1u, abort_flag)) { fail(12); ok = false; break; }
+                    asm volatile("ld.shared.f32 %0, [%1];" : "=f"(oth) : "r"((mx_own ^ 512u) + sl) : "memory");
+                } else if (jt > 0) {                               // running maximum after the previous tile, from its owner
                     if (!wait_pair(b_oth + 8 * MR, ph_prev, abort_flag)) { fail(12); ok = false; break; }
                     asm volatile("ld.shared.f32 %0, [%1];" : "=f"(m_run) : "r"(mx_own ^ 512u) : "memory");
                 }
                 // running maximum and rescale factor (lines 7-8), both FP16 values.  No branch: r = 1 exactly
                 // when the maximum did not move; at jt = 0 (m = -inf) r = 0 is never applied.
-                const float m_new = fmaxf(m_run, f16_round(mx * args.c0));
-                asm volatile("st.shared.f32 [%0], %1;" ::"r"(mx_own), "f"(m_new) : "memory");   // for the owner of the next tile
-                __syncwarp();
-                arrive0(b_own + 8 * MR, lane);
-                const float rsc = f16_round(ex2_approx((m_run - m_new) * LOG2E));
+                const float m_new = fmaxf(B128 ? fmaxf(m_run, oth) : m_run, f16_round(mx * args.c0));
+                if (!B128) {
+                    asm volatile("st.shared.f32 [%0], %1;" ::"r"(mx_own), "f"(m_new) : "memory");   // for the owner of the next tile
+                    __syncwarp();
+                    arrive0(b_own + 8 * MR, lane);
+                }
+                const float rsc = B128 && (t & 1) ? 1.f : f16_round(ex2_approx((m_run - m_new) * LOG2E));
                 m_run = m_new;
                 const float mL = m_run * LOG2E;
                 const float A = p_of_score<false>(mx, args.c1, mL); // = max of P over the group (monotone map)
@@ -509,7 +528,7 @@ attention_fwd_pair_kernel(const __grid_constant__ CUtensorMap tmap_q, const __gr
     if (warp == C::W_LD) { __syncwarp(); tmem_dealloc(tmem, C::TMEM_COLS); }
 }
 
-template <bool QM>
+template <bool QM, bool B128>
 static int launch_pair(const hifa4_shape& sh, const hifa4_qkv& qkv, const AttnArgs& args, cudaStream_t st)
 {
     using C = PairCfg;
@@ -517,7 +536,7 @@ static int launch_pair(const hifa4_shape& sh, const hifa4_qkv& qkv, const AttnAr
     if (!make_bf16_map(&mq, qkv.q_mma, (uint64_t)sh.B * sh.Hq, sh.N, C::D, 128)) return HIFA4_ERR_CUDA;
     if (!make_bf16_map(&mk, qkv.k_mma, (uint64_t)sh.B * sh.Hkv, sh.N, C::D, C::BC)) return HIFA4_ERR_CUDA;
     if (!make_bf16_map(&mv, qkv.v_mma, (uint64_t)sh.B * sh.Hkv, C::D, sh.N, C::D)) return HIFA4_ERR_CUDA;
-    auto kern = attention_fwd_pair_kernel<QM>;
+    auto kern = attention_fwd_pair_kernel<QM, B128>;
     static SmemOptIn opt_in;
     if (!opt_in.ensure(kern, C::SMEM_BYTES)) return HIFA4_ERR_CUDA;
     const int blocks = (sh.N + 127) / 128 * args.unit_heads;
@@ -531,23 +550,26 @@ static int launch_pair(const hifa4_shape& sh, const hifa4_qkv& qkv, const AttnAr
 // from 1.5 pairs per SM up (N = 2048, 8 / 2 heads: 128 pairs 44 against 35 us, 192 pairs 44 against 43, 256 pairs 46 against
 // 54, 320 pairs 60 against 64).  Non-causal pairs are all equal and come in whole waves (N = 1024, 8 / 2 heads: 64 pairs 26
 // against 18 us, 96 pairs 26 against 28, 160 pairs 47 against 42, 256 pairs 48 against 53, 320 pairs 69 against 66, 512 pairs
-// 91 against 96).
+// 91 against 96).  128-key tiles, against hifa4_attention_ws.cu: causal from 1.6 pairs per SM up (N = 2048, 28 and 32 heads: 224
+// pairs 66 against 63 us, 256 pairs 67 against 70; N = 1024, 64 heads 43 against 48), non-causal by the same waves (N = 1024, B =
+// 4, 32 heads 116 against 122; N = 4096, 32 heads 376 against 372).
 bool attention_pair_pays(const hifa4_shape& sh, const hifa4_attn_params& prm)
 {
-    if (sh.d != 128 || prm.Bc != 64 || prm.normalizer || prm.p_dtype == HIFA4_F32) return false;
+    if (sh.d != 128 || (prm.Bc != 64 && prm.Bc != 128) || prm.normalizer || prm.p_dtype == HIFA4_F32) return false;
     int dev = 0, sms = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0)
         return false;
     const long long blocks = (long long)((sh.N + 127) / 128) * sh.Hq * sh.B, pairs = (blocks + 1) / 2;
-    if (prm.causal) return 2 * pairs >= 3 * sms;
+    if (prm.causal) return prm.Bc == 128 ? 5 * pairs >= 8 * sms : 2 * pairs >= 3 * sms;
     const long long waves = (pairs + sms - 1) / sms, full = blocks / (2 * sms), rest = blocks % (2 * sms);
     return (double)waves <= 1.1 * ((double)full + (rest == 0 ? 0.0 : rest <= sms ? 0.67 : 1.0));
 }
 
-int launch_attention_pair(const hifa4_shape& sh, const hifa4_qkv& qkv, const AttnArgs& args, cudaStream_t st)
+int launch_attention_pair(const hifa4_shape& sh, const hifa4_qkv& qkv, const AttnArgs& args, int Bc, cudaStream_t st)
 {
     if (sh.d != 128) return HIFA4_ERR_UNSUPPORTED;
-    return args.qmean ? launch_pair<true>(sh, qkv, args, st) : launch_pair<false>(sh, qkv, args, st);
+    if (Bc == 128) return args.qmean ? launch_pair<true, true>(sh, qkv, args, st) : launch_pair<false, true>(sh, qkv, args, st);
+    return args.qmean ? launch_pair<true, false>(sh, qkv, args, st) : launch_pair<false, false>(sh, qkv, args, st);
 }
 
 }  // namespace hifa4

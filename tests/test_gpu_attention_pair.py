@@ -44,3 +44,22 @@ def test_two_block_kernel_is_bit_identical(name):
     for _ in range(2):
         hb.attention_fwd(qkv, causal, qmean=qmean, out=out, d_status=status)
     assert bool((out == 2.0).all()) and int(status.item()) == 9
+
+
+@pytest.mark.parametrize("B, Hq, Hkv, N, causal, qmean, head_map", [
+    (4, 32, 8, 1024, True, False, None), (4, 28, 4, 832, True, False, None),      # an odd number of 64-key tiles: N ends inside a tile
+    (8, 9, 9, 1152, True, False, None), (64, 16, 8, 64, False, False, None), (4, 24, 4, 1344, False, False, None),
+    (4, 32, 8, 1024, True, True, None), (8, 28, 4, 832, True, True, None), (8, 8, 4, 1088, True, False, [3, 0, 0, 2, 1, 3, 3, 0]),
+])
+def test_two_block_kernel_with_128_key_tiles(B, Hq, Hkv, N, causal, qmean, head_map):
+    """Against the 128-key kernel (hifa4_attention_ws.cu), which the dump launch always runs."""
+    from paper_2607_04302_b200 import binding as hb
+    cfg = synth.config("C2", B=B, Hq=Hq, Hkv=Hkv, N=N, causal=causal)
+    q, k, v = synth.make_qkv_device(cfg, DEV)
+    qkv = hb.quantize_qkv(q, k, v, q_to_kv=head_map, qmean=qmean)
+    status = torch.zeros(1, dtype=torch.int32, device=DEV)
+    want, _ = hb.attention_fwd(qkv, causal, Bc=128, qmean=qmean, debug_blocks=[(0, 0, 0)], d_status=status)
+    for dt, ref in ((hb.F32, want), (hb.F16, want.half()), (hb.BF16, want.bfloat16())):
+        assert torch.equal(hb.attention_fwd(qkv, causal, Bc=128, qmean=qmean, out_dtype=dt, d_status=status), ref)
+    assert torch.equal(hb.attention_fwd_raw(q, k, v, None, None, causal, Bc=128, q_to_kv=head_map, qmean=qmean, d_status=status), want)
+    assert int(status.item()) == 0
