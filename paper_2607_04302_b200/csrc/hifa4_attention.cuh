@@ -157,7 +157,9 @@ __device__ __forceinline__ float p_of_score(float acc, float c1, float mL)
 //   q = RN(p * (2/S) 2^-s)          2/S = hi + lo in two FP16 constants (the mantissas 4/(4+M) repeat with a period
 //                                   that divides 12, so one FP16 constant errs by 2^-12, which is not enough):
 //                                   q = fma(p, hi, RN(p * lo)).  Exactly on every rounding tie and on the right side
-//                                   of it everywhere else
+//                                   of it everywhere else (P exceeds 1 where the running maximum, an FP16 value, was
+//                                   rounded down: up to e^8 for scaled scores of 16384 to 32768.  For S >= 10 lo is
+//                                   a subnormal with a few bits, which is all that a correction of 2^-12 needs)
 //   y = q + 1.5 * 2^(9+k) 2^-s      rounds q to the nearest multiple of the subgroup's step, ties to even;
 //                                   the low bits of y are the element code m
 //   v = fma_bf16(y, c, -n)          the bit pattern of y read as BF16 is 2^E (1 + m/128) with E known from k and s, so
@@ -166,8 +168,8 @@ __device__ __forceinline__ float p_of_score(float acc, float c1, float mL)
 // is read off the bit pattern of its largest q: need = number of thresholds 3.5, 7 (1.75 S, 3.5 S) exceeded, then
 // k_t = max(need_t, need_other - 1) (that is the pair rule: the level-2 bit is set iff max(need) = 2 or min(need) >= 1,
 // and a subgroup that needs no shift of its own still gets one when its partner needs two); the two subgroups of a unit
-// share packed 16-bit integer operations.  tests/test_p_quantizer_arithmetic.py checks the scheme on every FP16 P, every
-// scale code and every shift.
+// share packed 16-bit integer operations.  tests/test_p_quantizer_arithmetic.py checks the scheme on every finite FP16 P
+// under every scale a group maximum can select and every shift.
 // The FP32-P variant keeps the FP32 form of the same scheme: q = RZ(p * (4/S)) (exactly on ties, see e6m2_inv4),
 // y = q + 1.5 * 2^(23+k), v = fma(y, S/4, -magic*S/4), two elements per f32x2 operation.
 template <bool PF32> struct PQuantConst;        // per (row, 64-key group, tile) constants of the fused quantizer
@@ -208,7 +210,7 @@ __device__ __forceinline__ PQuantConst<PF32> p_quant_const(float c1, float mL, f
         const uint32_t sh = (uint32_t)((small ? 37 : 49) - e) * 0x04000400u;
         const uint32_t top = (small ? 12u : 0u) * 0x04000400u;
         k.hi = __byte_perm(0x3A663C00u, 0x38923955u, sel) + sh;            // RN16(4/(4+M)) * 2^(49-e-s)
-        k.lo = M ? k.hi - 0x30003000u : 0u;                                // hi * 2^-12
+        k.lo = M ? h2_mul(k.hi, 0x0C000C00u) : 0u;                         // RN16(hi * 2^-12): subnormal from S = 10 up
         k.tadd = 0xC0FFC0FFu + top;                                        // 1023 - bits(3.5 * 2^-s), per half
         k.magic = 0x62006200u - top;                                       // 768 * 2^-s
         const uint32_t m5 = (uint32_t)M << 5;

@@ -1,10 +1,11 @@
 """The packed FP16 arithmetic of the in-register quantizer of P (hifa4_attention.cuh), restated in numpy: on every
-FP16 value of P in [0, 1] under every E6M2 scale a group maximum can select and every shift, the element code is the
-round-to-nearest-even of the exact quotient, the shift thresholds are exact and the BF16 FMA returns code * step."""
+finite non-negative FP16 value of P (above 1 too: the running maximum may have been rounded down) under every E6M2 scale a
+group maximum can select and every shift, the element code is the round-to-nearest-even of the exact quotient, the shift
+thresholds are exact and the BF16 FMA returns code * step."""
 import numpy as np
 import pytest
 
-P = np.arange(0, 0x3C01, dtype=np.uint16).view(np.float16).astype(np.float64)
+P = np.arange(0, 0x7C00, dtype=np.uint16).view(np.float16).astype(np.float64)
 HI = (0x3C00, 0x3A66, 0x3955, 0x3892)              # RN16(4 / (4 + M))
 
 
@@ -37,10 +38,11 @@ def test_packed_fp16_quantizer_is_exact(M):
             continue
         e = code >> 2
         S = 2.0 ** (e - 48) * (1 + M / 4)
-        p = P[P <= min(1.0 if s == 0 else 2.0 ** -12 * (1 - 2.0 ** -11), 7 * S)]
+        p = P[P <= min(65504.0 if s == 0 else 2.0 ** -12 * (1 - 2.0 ** -11), 7 * S)]
         hi_bits = HI[M] + ((49 - e - s) << 10)
-        hi, lo = f16(hi_bits), f16(hi_bits - 0x3000) if M else 0.0
-        assert np.isfinite(hi)
+        hi = f16(hi_bits)
+        lo = float(rn16(np.float64(hi * 2.0 ** -12))) if M else 0.0
+        assert np.isfinite(hi) and hi_bits >> 10 > 0
         q = rn16(p * hi + rn16(p * lo))            # exact in double before the one rounding of the FMA
         need = np.maximum(bits16(q) + 1023 - (0x4300 - (s << 10)), 0) >> 10
         assert (need == (p > 1.75 * S).astype(int) + (p > 3.5 * S)).all()
