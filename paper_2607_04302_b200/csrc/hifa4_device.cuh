@@ -100,7 +100,7 @@ template <> __device__ __forceinline__ uint32_t max16<__nv_bfloat16>(uint32_t a,
     return r;
 }
 
-// Magnitudes of a packed pair; smaller of two packed BF16 pairs.
+// Magnitudes of a packed pair.
 template <typename T> __device__ __forceinline__ uint32_t abs16(uint32_t a);
 template <> __device__ __forceinline__ uint32_t abs16<__half>(uint32_t a)
 {
@@ -112,12 +112,6 @@ template <> __device__ __forceinline__ uint32_t abs16<__nv_bfloat16>(uint32_t a)
 {
     uint32_t r;
     asm("abs.bf16x2 %0, %1;" : "=r"(r) : "r"(a));
-    return r;
-}
-__device__ __forceinline__ uint32_t min16_bf16(uint32_t a, uint32_t b)
-{
-    uint32_t r;
-    asm("min.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
     return r;
 }
 

@@ -1,5 +1,5 @@
 // Smooth-QK scaling fused with HIF4 quantization (Algorithm 1 lines 1 and 3).  Q, K and V are quantized by one
-// launch: 128-bit coalesced loads, one 8-lane team per 64-element group, shuffle reductions,
+// launch: 128-bit coalesced loads, a team of four lanes per 64-element group, shuffle reductions,
 // packed f32x2 arithmetic.
 #include <type_traits>
 
@@ -70,8 +70,10 @@ template <> __device__ __forceinline__ uint32_t unit_shifts<__half>(uint32_t At,
 
 // xw: the 16 values as packed pairs (words 0-3 unit j, 4-7 unit j + 4), already smoothed and rounded to T.  Returns the
 // BF16 image in xw; CODES: also the packed nibbles of the two units and the group's metadata word (same on every lane).
+// False: the group's maximum lies above 7 S of the largest scale (in FP16: it is an infinity, a smoothed product may round to
+// one; 7 S is not an FP16 value), what was formed is void and quantize16_general has to do it.
 template <typename T, bool CODES>
-__device__ __forceinline__ void quantize16(uint32_t (&xw)[8], int j, uint32_t (&nib)[2], uint32_t& meta_word)
+__device__ __forceinline__ bool quantize16(uint32_t (&xw)[8], int j, uint32_t (&nib)[2], uint32_t& meta_word)
 {
     uint32_t At[2];                                               // {subgroup 0, subgroup 1} of each unit
 #pragma unroll
@@ -87,12 +89,6 @@ __device__ __forceinline__ void quantize16(uint32_t (&xw)[8], int j, uint32_t (&
     float A, Ah;
     Pair16<T>::unpack(A2, Ah, A);
     const Group g = group_of(A);                                  // A = 0 gives code 0 and an all-zero group
-    if (std::is_same<T, __nv_bfloat16>::value && A > 401408.f) {  // above 7 S of the largest scale: saturate
-#pragma unroll
-        for (int i = 0; i < 8; ++i) xw[i] = max16<T>(min16_bf16(xw[i], 0x48C448C4u), 0xC8C4C8C4u);
-        At[0] = min16_bf16(At[0], 0x48C448C4u);
-        At[1] = min16_bf16(At[1], 0x48C448C4u);
-    }
     uint32_t ks[2];
 #pragma unroll
     for (int u = 0; u < 2; ++u) {
@@ -140,6 +136,53 @@ __device__ __forceinline__ void quantize16(uint32_t (&xw)[8], int j, uint32_t (&
         part |= __shfl_xor_sync(0xffffffffu, part, 2);
         meta_word = part | ((g.s_bits >> 21) - 316u);             // + scale code 4 (exponent - 79) + mantissa
     }
+    return A <= 401408.f;
+}
+
+// The same for any values: widened, and clamped where the maximum exceeds 7 S.  A warp that has a group for it runs it over
+// all its shares, after the usual form, in a function of its own (see requantize).
+template <typename T, bool CODES>
+__device__ __forceinline__ void quantize16_general(uint32_t (&xw)[8], int j, uint32_t (&nib)[2], uint32_t& meta_word)
+{
+    float a[4], A = 0.f;                                          // maxima of the lane's subgroups and of the group
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+        float x[4];
+        Pair16<T>::unpack(xw[2 * t], x[0], x[1]);
+        Pair16<T>::unpack(xw[2 * t + 1], x[2], x[3]);
+        a[t] = fmaxf(max3(fabsf(x[0]), fabsf(x[1]), fabsf(x[2])), fabsf(x[3]));
+        A = fmaxf(A, a[t]);
+    }
+    A = fmaxf(A, __shfl_xor_sync(0xffffffffu, A, 1));
+    A = fmaxf(A, __shfl_xor_sync(0xffffffffu, A, 2));
+    const Hif4Group g = hif4_group(A);
+    uint32_t part = 0;
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+        float x[8], y[8];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) Pair16<T>::unpack(xw[4 * u + i], x[2 * i], x[2 * i + 1]);
+        if (A > g.top) {
+#pragma unroll
+            for (int i = 0; i < 8; ++i) x[i] = fminf(fmaxf(x[i], -g.top), g.top);
+            a[2 * u] = fminf(a[2 * u], g.top);
+            a[2 * u + 1] = fminf(a[2 * u + 1], g.top);
+        }
+        uint32_t w[4];
+        int l2, k0, k1;
+        hif4_unit(x, a[2 * u], a[2 * u + 1], g, w, y, l2, k0, k1);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) xw[4 * u + i] = w[i];
+        if (CODES) {
+            nib[u] = hif4_unit_nibbles(y);
+            part |= hif4_unit_meta(j + 4 * u, l2, k0, k1);
+        }
+    }
+    if (CODES) {
+        part |= __shfl_xor_sync(0xffffffffu, part, 1);
+        part |= __shfl_xor_sync(0xffffffffu, part, 2);
+        meta_word = part | (uint32_t)g.code;
+    }
 }
 
 struct QuantJob {                     // one launch quantizes Q, K and V (any of them may be absent)
@@ -162,9 +205,9 @@ constexpr int QUANT_THREADS = 256;
 
 // Q and K: groups along d.  One head is N*d/16 lane shares; a CTA takes 256 * UPT consecutive ones, thread t the shares t,
 // t + 256 (all loads are issued before any arithmetic).  The shares of a thread have their channels, hence their Smooth-QK
-// factors, in common.
-template <typename T, int UPT, bool CODES, bool QM>
-__device__ __forceinline__ void quantize_rows_cta(const uint16_t* __restrict__ x, const float* __restrict__ scale,
+// factors, in common.  Returns whether the usual form did for all of them.
+template <typename T, int UPT, bool CODES, bool QM, bool GENERAL>
+__device__ __forceinline__ bool quantize_rows_cta(const uint16_t* __restrict__ x, const float* __restrict__ scale,
                                                   int kv_row, long long head, unsigned blk_in_head, int N, int d,
                                                   uint8_t* __restrict__ codes, uint32_t* __restrict__ meta,
                                                   uint16_t* __restrict__ img, float* __restrict__ mu_out,
@@ -187,6 +230,7 @@ __device__ __forceinline__ void quantize_rows_cta(const uint16_t* __restrict__ x
         const float4* sp = reinterpret_cast<const float4*>(scale + (long long)kv_row * d + c0);
         sv[0] = __ldg(sp); sv[1] = __ldg(sp + 1); sv[2] = __ldg(sp + 8); sv[3] = __ldg(sp + 9);
     }
+    bool done = true;
 #pragma unroll
     for (int r = 0; r < UPT; ++r) {
         const long long grp = g0 + r * (QUANT_THREADS / 4);
@@ -229,7 +273,8 @@ __device__ __forceinline__ void quantize_rows_cta(const uint16_t* __restrict__ x
             }
         }
         uint32_t nib[2], mw;
-        quantize16<T, CODES>(xw, j, nib, mw);
+        if constexpr (GENERAL) quantize16_general<T, CODES>(xw, j, nib, mw);
+        else done &= quantize16<T, CODES>(xw, j, nib, mw);
         uint4* dst = reinterpret_cast<uint4*>(img) + grp * 8 + j;
         dst[0] = make_uint4(xw[0], xw[1], xw[2], xw[3]);
         dst[4] = make_uint4(xw[4], xw[5], xw[6], xw[7]);
@@ -240,36 +285,39 @@ __device__ __forceinline__ void quantize_rows_cta(const uint16_t* __restrict__ x
             if (j == 0) meta[grp] = mw;
         }
     }
+    return done;
 }
 
 // V: groups of 64 tokens per channel; outputs are stored transposed ([.., d, N]).  Half a CTA (128 threads) transposes a
 // 64-token x 64-channel tile through shared memory.  The tile is kept as 64 rows of 8 16-byte chunks, chunk c of row r
 // stored at position c ^ f(r) with f(r) = 2 (r / 8) mod 8 + r / 32, so that both the row-wise 16-byte stores and the
 // column-wise 4-byte reads (a thread reads two adjacent channels of 8 consecutive tokens, a warp 8 channel pairs x 4
-// lanes) are free of bank conflicts.
-template <typename T, bool CODES>
-__device__ __forceinline__ void quantize_tokens_half(uint4* tile, bool valid, const uint16_t* __restrict__ x, long long bh, int tok0,
+// lanes) are free of bank conflicts.  The general form reads its values from global memory instead.
+template <typename T, bool CODES, bool GENERAL>
+__device__ __forceinline__ bool quantize_tokens_half(uint4* tile, bool valid, const uint16_t* __restrict__ x, long long bh, int tok0,
                                                      int ch0, int N, int d, uint8_t* __restrict__ codes,
                                                      uint32_t* __restrict__ meta, uint16_t* __restrict__ img)
 {
     const int tid = threadIdx.x & 127;
+    const uint16_t* src = x + (bh * N + tok0) * (long long)d + ch0;
     auto swz = [](int r) { return ((r >> 3) * 2 & 7) + (r >> 5); };
-    if (valid) {
-        const uint16_t* src = x + (bh * N + tok0) * (long long)d + ch0;
-        uint4 v[4];
+    if constexpr (!GENERAL) {
+        if (valid) {
+            uint4 v[4];
 #pragma unroll
-        for (int it = 0; it < 4; ++it) {
-            const int idx = tid + it * 128;
-            v[it] = __ldg(reinterpret_cast<const uint4*>(src + (long long)(idx >> 3) * d) + (idx & 7));
-        }
+            for (int it = 0; it < 4; ++it) {
+                const int idx = tid + it * 128;
+                v[it] = __ldg(reinterpret_cast<const uint4*>(src + (long long)(idx >> 3) * d) + (idx & 7));
+            }
 #pragma unroll
-        for (int it = 0; it < 4; ++it) {
-            const int idx = tid + it * 128, r = idx >> 3;
-            tile[r * 8 + ((idx & 7) ^ swz(r))] = v[it];
+            for (int it = 0; it < 4; ++it) {
+                const int idx = tid + it * 128, r = idx >> 3;
+                tile[r * 8 + ((idx & 7) ^ swz(r))] = v[it];
+            }
         }
+        __syncthreads();
     }
-    __syncthreads();
-    if (!valid) return;
+    if (!valid) return true;
     const int cp = tid >> 2, j = tid & 3;                          // channel pair, lane of the team
     const uint32_t* tw = reinterpret_cast<const uint32_t*>(tile);
     uint32_t wa[8], wb[8];                                         // channels 2 cp and 2 cp + 1, token pairs
@@ -278,16 +326,25 @@ __device__ __forceinline__ void quantize_tokens_half(uint4* tile, bool valid, co
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
             const int r = 8 * (j + 4 * u) + 2 * i;
-            const int pos = (((cp >> 2) ^ swz(r)) << 2) | (cp & 3);
-            const uint32_t t0 = tw[r * 32 + pos], t1 = tw[(r + 1) * 32 + pos];
+            uint32_t t0, t1;
+            if constexpr (GENERAL) {
+                t0 = __ldg(reinterpret_cast<const uint32_t*>(src + (long long)r * d) + cp);
+                t1 = __ldg(reinterpret_cast<const uint32_t*>(src + (long long)(r + 1) * d) + cp);
+            } else {
+                const int pos = (((cp >> 2) ^ swz(r)) << 2) | (cp & 3);
+                t0 = tw[r * 32 + pos];
+                t1 = tw[(r + 1) * 32 + pos];
+            }
             wa[4 * u + i] = __byte_perm(t0, t1, 0x5410);
             wb[4 * u + i] = __byte_perm(t0, t1, 0x7632);
         }
+    bool done = true;
 #pragma unroll
     for (int c = 0; c < 2; ++c) {
         uint32_t (&xw)[8] = c ? wb : wa;
         uint32_t nib[2], mw;
-        quantize16<T, CODES>(xw, j, nib, mw);
+        if constexpr (GENERAL) quantize16_general<T, CODES>(xw, j, nib, mw);
+        else done &= quantize16<T, CODES>(xw, j, nib, mw);
         const long long orow = bh * d + ch0 + 2 * cp + c;             // row of the transposed outputs
         uint4* dst = reinterpret_cast<uint4*>(img + orow * (long long)N + tok0) + j;
         dst[0] = make_uint4(xw[0], xw[1], xw[2], xw[3]);
@@ -299,6 +356,40 @@ __device__ __forceinline__ void quantize_tokens_half(uint4* tile, bool valid, co
             if (j == 0) meta[orow * (N / 64) + tok0 / 64] = mw;
         }
     }
+    return done;
+}
+
+template <typename T, int UPT, bool CODES, bool QM, bool GENERAL>
+__device__ __forceinline__ bool quantize_cta(const QuantJob& job, uint4* tiles)
+{
+    unsigned blk = blockIdx.x;
+    if (blk < job.q_blocks + job.k_blocks) {
+        const bool is_q = blk < job.q_blocks;
+        if (!is_q) blk -= job.q_blocks;
+        const unsigned head = blk / job.row_blocks_per_head;             // b * H + h
+        const unsigned in_head = blk - head * job.row_blocks_per_head;
+        if (is_q)
+            return quantize_rows_cta<T, UPT, CODES, QM, GENERAL>(job.q, job.s, job.qmap.kv_of[head % (unsigned)job.Hq], head, in_head, job.N,
+                                 job.d, job.q_codes, job.q_meta, job.q_img, job.q_mu, nullptr);
+        return quantize_rows_cta<T, UPT, CODES, QM, GENERAL>(job.k, job.inv_s, (int)(head % (unsigned)job.Hkv), head, in_head, job.N, job.d,
+                                 job.k_codes, job.k_meta, job.k_img, nullptr, job.k_sum);
+    }
+    blk -= job.q_blocks + job.k_blocks;
+    const unsigned half = threadIdx.x >> 7, t = 2 * blk + half;
+    const unsigned tok_blocks = job.N / 64, ch_blocks = job.d / 64;
+    const unsigned tb = t % tok_blocks, rest = t / tok_blocks;
+    const unsigned cb = rest % ch_blocks, bh = rest / ch_blocks;
+    return quantize_tokens_half<T, CODES, GENERAL>(tiles + half * (64 * 8), t < job.v_tiles, job.v, bh, tb * 64, cb * 64, job.N, job.d,
+                                                   job.v_codes, job.v_meta, job.v_img);
+}
+
+// Out of line, and from the inputs in global memory on, so that nothing of the usual path lives across it: a branch to the general
+// form inside quantize16, even one that is never taken, costs 1 to 6 % (the shares of a thread no longer interleave), and an
+// inlined second pass 2 to 8 % (spills at the 64 registers of four CTAs per SM).
+template <typename T, int UPT, bool CODES, bool QM>
+__device__ __noinline__ void requantize(const QuantJob& job)
+{
+    quantize_cta<T, UPT, CODES, QM, true>(job, nullptr);
 }
 
 template <typename T, int UPT, bool CODES, bool QM>
@@ -310,27 +401,9 @@ quantize_qkv_kernel(const __grid_constant__ QuantJob job)
     // same behind its predecessor (back-to-back calls: 44.2 -> 42.8 us at N = 8192, 30.6 -> 28.9 us for a whole d = 64 prefill)
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    unsigned blk = blockIdx.x;
-    if (blk < job.q_blocks + job.k_blocks) {
-        const bool is_q = blk < job.q_blocks;
-        if (!is_q) blk -= job.q_blocks;
-        const unsigned head = blk / job.row_blocks_per_head;             // b * H + h
-        const unsigned in_head = blk - head * job.row_blocks_per_head;
-        if (is_q)
-            quantize_rows_cta<T, UPT, CODES, QM>(job.q, job.s, job.qmap.kv_of[head % (unsigned)job.Hq], head, in_head, job.N, job.d,
-                                 job.q_codes, job.q_meta, job.q_img, job.q_mu, nullptr);
-        else
-            quantize_rows_cta<T, UPT, CODES, QM>(job.k, job.inv_s, (int)(head % (unsigned)job.Hkv), head, in_head, job.N, job.d,
-                                 job.k_codes, job.k_meta, job.k_img, nullptr, job.k_sum);
-    } else {
-        blk -= job.q_blocks + job.k_blocks;
-        __shared__ uint4 tiles[2][64 * 8];
-        const unsigned half = threadIdx.x >> 7, t = 2 * blk + half;
-        const unsigned tok_blocks = job.N / 64, ch_blocks = job.d / 64;
-        const unsigned tb = t % tok_blocks, rest = t / tok_blocks;
-        const unsigned cb = rest % ch_blocks, bh = rest / ch_blocks;
-        quantize_tokens_half<T, CODES>(tiles[half], t < job.v_tiles, job.v, bh, tb * 64, cb * 64, job.N, job.d, job.v_codes, job.v_meta, job.v_img);
-    }
+    __shared__ uint4 tiles[2 * 64 * 8];
+    const bool done = quantize_cta<T, UPT, CODES, QM, false>(job, tiles);
+    if (!__all_sync(0xffffffffu, done)) requantize<T, UPT, CODES, QM>(job);
 }
 
 // ------------------------------------------------------------------------------- launchers

@@ -38,3 +38,27 @@ def test_extreme_magnitudes_match_the_oracle(dtype):
     x = (x.clamp(-65504, 65504) if dtype == "fp16" else x).to(synth.torch_dtype(cfg))[None, None]
     qkv = hb.quantize_qkv(x.to(DEV), x.to(DEV), x.to(DEV))
     parity.check_quantized(cfg, x, x, x, None, None, qkv)
+
+
+def test_fp16_overflow_saturates_like_the_oracle():
+    """A smoothed FP16 product above 65504 rounds to infinity and saturates at the largest HIF4 magnitude (7 times the largest
+    scale), as does an infinity of the input; the other elements of its group keep their values.  The query quantizer inside
+    the attention kernel must agree with the stand-alone one bit for bit."""
+    from paper_2607_04302_b200 import binding as hb
+    gen = torch.Generator().manual_seed(3)
+    cfg = synth.config("C3", N=128, Hq=2, Hkv=1, dtype="fp16", causal=False)
+    q, k, v = (torch.randn((1, h, 128, 128), generator=gen) for h in (2, 1, 1))
+    q *= torch.exp2(torch.linspace(-8, 13, 128))[:, None]
+    k *= torch.exp2(torch.linspace(13, -8, 128))[:, None]
+    v[..., 5, 3] = float("inf")
+    v[..., 70:72, 9] = -float("inf")
+    s = torch.exp2(torch.randint(-4, 5, (1, 128), generator=gen).float()) * 1.25
+    inv_s = 1.0 / s
+    q, k, v = (x.half() for x in (q, k, v))
+    assert torch.isinf((q.float() * s).half()).any() and torch.isinf((k.float() * inv_s).half()).any()
+    qd, kd, vd, sd, isd = (x.to(DEV) for x in (q, k, v, s, inv_s))
+    qkv = hb.quantize_qkv(qd, kd, vd, sd, isd)
+    parity.check_quantized(cfg, q, k, v, sd, isd, qkv)
+    want = hb.attention_fwd(qkv, False)
+    kv = hb.quantize_qkv(None, kd, vd, sd, isd, Hq=2)
+    assert torch.equal(hb.attention_fwd_qraw(qd, sd, kv, False).view(torch.int32), want.view(torch.int32))
