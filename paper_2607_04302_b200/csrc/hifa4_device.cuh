@@ -100,6 +100,21 @@ template <> __device__ __forceinline__ uint32_t max16<__nv_bfloat16>(uint32_t a,
     return r;
 }
 
+// The same, but a NaN wins.
+template <typename T> __device__ __forceinline__ uint32_t max16_nan(uint32_t a, uint32_t b);
+template <> __device__ __forceinline__ uint32_t max16_nan<__half>(uint32_t a, uint32_t b)
+{
+    uint32_t r;
+    asm("max.NaN.f16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
+    return r;
+}
+template <> __device__ __forceinline__ uint32_t max16_nan<__nv_bfloat16>(uint32_t a, uint32_t b)
+{
+    uint32_t r;
+    asm("max.NaN.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
+    return r;
+}
+
 // Magnitudes of a packed pair.
 template <typename T> __device__ __forceinline__ uint32_t abs16(uint32_t a);
 template <> __device__ __forceinline__ uint32_t abs16<__half>(uint32_t a)
@@ -209,8 +224,8 @@ __device__ __forceinline__ uint32_t hif4_unit_meta(int j, int a, int k0, int k1)
 
 // One thread quantizes one whole 64-element group (Algorithm 1 lines 1 and 3) held in registers as 32 words of
 // 16-bit pairs (element 2i in the low half of word i): the words are replaced by the BF16 image of
-// HIF4(round_in(x * s)).  scale: the 64 Smooth-QK factors of these elements or null.  Same arithmetic as the 8-lane
-// team of the stand-alone quantizer (hif4_group / hif4_unit), with the group constants formed once and no shuffles;
+// HIF4(round_in(x * s)).  scale: the 64 Smooth-QK factors of these elements or null.  Same arithmetic as the general form
+// of the stand-alone quantizer (hif4_group / hif4_unit), with the group constants formed once and no shuffles;
 // the packed codes are not formed (the caller consumes the image at once).
 template <typename T>
 __device__ __forceinline__ void hif4_quantize64_regs(uint32_t (&xw)[32], const float* __restrict__ scale)
@@ -248,7 +263,7 @@ __device__ __forceinline__ void hif4_quantize64_regs(uint32_t (&xw)[32], const f
         for (int i = 0; i < 4; ++i) Pair16<T>::unpack(xw[4 * u + i], x[2 * i], x[2 * i + 1]);
         if (sat) {
 #pragma unroll
-            for (int i = 0; i < 8; ++i) x[i] = fminf(fmaxf(x[i], -g.top), g.top);
+            for (int i = 0; i < 8; ++i) x[i] = x[i] > g.top ? g.top : x[i] < -g.top ? -g.top : x[i];     // a NaN stays one
         }
         const float a0 = fmaxf(max3(fabsf(x[0]), fabsf(x[1]), fabsf(x[2])), fabsf(x[3]));
         const float a1 = fmaxf(max3(fabsf(x[4]), fabsf(x[5]), fabsf(x[6])), fabsf(x[7]));

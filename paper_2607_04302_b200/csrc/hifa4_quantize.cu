@@ -71,21 +71,22 @@ template <> __device__ __forceinline__ uint32_t unit_shifts<__half>(uint32_t At,
 // xw: the 16 values as packed pairs (words 0-3 unit j, 4-7 unit j + 4), already smoothed and rounded to T.  Returns the
 // BF16 image in xw; CODES: also the packed nibbles of the two units and the group's metadata word (same on every lane).
 // False: the group's maximum lies above 7 S of the largest scale (in FP16: it is an infinity, a smoothed product may round to
-// one; 7 S is not an FP16 value), what was formed is void and quantize16_general has to do it.
+// one; 7 S is not an FP16 value), or the group holds a NaN, whose bit pattern would run into its neighbours' nibbles.  What was
+// formed is then void and quantize16_general has to do it.
 template <typename T, bool CODES>
 __device__ __forceinline__ bool quantize16(uint32_t (&xw)[8], int j, uint32_t (&nib)[2], uint32_t& meta_word)
 {
-    uint32_t At[2];                                               // {subgroup 0, subgroup 1} of each unit
+    uint32_t At[2];                                               // {subgroup 0, subgroup 1} of each unit; a NaN wins
 #pragma unroll
     for (int u = 0; u < 2; ++u) {
-        const uint32_t m0 = max16<T>(abs16<T>(xw[4 * u]), abs16<T>(xw[4 * u + 1]));
-        const uint32_t m1 = max16<T>(abs16<T>(xw[4 * u + 2]), abs16<T>(xw[4 * u + 3]));
-        At[u] = max16<T>(__byte_perm(m0, m1, 0x5410), __byte_perm(m0, m1, 0x7632));
+        const uint32_t m0 = max16_nan<T>(abs16<T>(xw[4 * u]), abs16<T>(xw[4 * u + 1]));
+        const uint32_t m1 = max16_nan<T>(abs16<T>(xw[4 * u + 2]), abs16<T>(xw[4 * u + 3]));
+        At[u] = max16_nan<T>(__byte_perm(m0, m1, 0x5410), __byte_perm(m0, m1, 0x7632));
     }
-    uint32_t A2 = max16<T>(At[0], At[1]);
-    A2 = max16<T>(A2, __byte_perm(A2, A2, 0x1032));
-    A2 = max16<T>(A2, __shfl_xor_sync(0xffffffffu, A2, 1));
-    A2 = max16<T>(A2, __shfl_xor_sync(0xffffffffu, A2, 2));
+    uint32_t A2 = max16_nan<T>(At[0], At[1]);
+    A2 = max16_nan<T>(A2, __byte_perm(A2, A2, 0x1032));
+    A2 = max16_nan<T>(A2, __shfl_xor_sync(0xffffffffu, A2, 1));
+    A2 = max16_nan<T>(A2, __shfl_xor_sync(0xffffffffu, A2, 2));
     float A, Ah;
     Pair16<T>::unpack(A2, Ah, A);
     const Group g = group_of(A);                                  // A = 0 gives code 0 and an all-zero group
@@ -144,7 +145,7 @@ __device__ __forceinline__ bool quantize16(uint32_t (&xw)[8], int j, uint32_t (&
 template <typename T, bool CODES>
 __device__ __forceinline__ void quantize16_general(uint32_t (&xw)[8], int j, uint32_t (&nib)[2], uint32_t& meta_word)
 {
-    float a[4], A = 0.f;                                          // maxima of the lane's subgroups and of the group
+    float a[4], A = 0.f;                                          // maxima of the lane's subgroups and of the group; a NaN loses
 #pragma unroll
     for (int t = 0; t < 4; ++t) {
         float x[4];
@@ -164,7 +165,7 @@ __device__ __forceinline__ void quantize16_general(uint32_t (&xw)[8], int j, uin
         for (int i = 0; i < 4; ++i) Pair16<T>::unpack(xw[4 * u + i], x[2 * i], x[2 * i + 1]);
         if (A > g.top) {
 #pragma unroll
-            for (int i = 0; i < 8; ++i) x[i] = fminf(fmaxf(x[i], -g.top), g.top);
+            for (int i = 0; i < 8; ++i) x[i] = x[i] > g.top ? g.top : x[i] < -g.top ? -g.top : x[i];     // a NaN stays one
             a[2 * u] = fminf(a[2 * u], g.top);
             a[2 * u + 1] = fminf(a[2 * u + 1], g.top);
         }

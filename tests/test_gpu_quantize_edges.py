@@ -62,3 +62,27 @@ def test_fp16_overflow_saturates_like_the_oracle():
     want = hb.attention_fwd(qkv, False)
     kv = hb.quantize_qkv(None, kd, vd, sd, isd, Hq=2)
     assert torch.equal(hb.attention_fwd_qraw(qd, sd, kv, False).view(torch.int32), want.view(torch.int32))
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "fp16"])
+def test_nan_spoils_no_other_element(dtype):
+    """A NaN in the input gives a NaN in the image and takes no part in the maxima; every other element of its group, its packed
+    nibble included, is what it is with a zero in that place (infinities saturate beside it)."""
+    from paper_2607_04302_b200 import binding as hb
+    gen = torch.Generator().manual_seed(5)
+    cfg = synth.config("C3", N=128, Hq=1, Hkv=1, dtype=dtype)
+    x = torch.randn((1, 1, 128, 128), generator=gen)
+    x[0, 0, 40, 70] = float("inf")
+    bad = torch.rand(x.shape, generator=gen) < 0.05
+    bad[0, 0, 40, 66] = True
+    x = x.to(synth.torch_dtype(cfg))
+    xd = torch.where(bad, torch.full_like(x, float("nan")), x).to(DEV)
+    qkv = hb.quantize_qkv(xd, xd, xd)
+    ref = hb.quantize_qkv(*(torch.where(bad, torch.zeros_like(x), x).to(DEV) for _ in range(3)))
+    for n in "qkv":
+        b = (bad.transpose(2, 3) if n == "v" else bad).to(DEV)
+        assert torch.equal(getattr(qkv, n + "_meta"), getattr(ref, n + "_meta"))
+        c, r = (torch.stack((t & 15, t >> 4), -1).flatten(-2) for t in (getattr(qkv, n + "_codes"), getattr(ref, n + "_codes")))
+        assert torch.equal(c[~b], r[~b])
+        c, r = getattr(qkv, n + "_mma"), getattr(ref, n + "_mma")
+        assert torch.equal(c[~b], r[~b]) and bool(torch.isnan(c[b]).all())
