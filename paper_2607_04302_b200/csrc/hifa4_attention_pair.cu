@@ -55,10 +55,10 @@ namespace pairk {
 // S buffer free (4 arrivals), SF[t % 2] S complete, PGO P-hat stored and history rescaled (4), PV[t % 2] P V complete,
 // MR[t % 2] (128-key tiles: t % 4) maxima published (4), OE output columns read (8).  Ring (index = stage): KF / VF tile landed, KE / VE
 // tile read by both halves.  WF / WE[pair % 2]: work record written / read by all (20); CL: answer of the launch control;
-// KSF[tile % 8].  SF, PV and MR come in twos because each group of softmax warps sees every second tile only: a parity
-// wait must not be two phases behind.
+// KSF[tile % 8]; AB, per half: its softmax warps have come to a pair without a block for it (8, Q-Mean only).  SF, PV and MR
+// come in twos because each group of softmax warps sees every second tile only: a parity wait must not be two phases behind.
 enum { QF = 0, QD = 1, SFR = 2, PGO = 3, SF = 4, PV = 6, MR = 8, OE = 12, HALF = 16,
-       KF = 32, KE = 35, VF = 38, VE = 41, WF = 44, WE = 46, CL = 48, KSF = 49, N_BARS = 57 };
+       KF = 32, KE = 35, VF = 38, VE = 41, WF = 44, WE = 46, CL = 48, KSF = 49, AB = 57, N_BARS = 59 };
 constexpr uint32_t WAIT_POLLS = 1u << 18;            // a poll may keep the thread suspended for up to about 4 us
 struct Work {                         // one pair of query blocks
     int n_max;                        // key tiles to load; 0: no more work
@@ -154,7 +154,7 @@ attention_fwd_pair_kernel(const __grid_constant__ CUtensorMap tmap_q, const __gr
             }
             for (int s = 0; s < 4; ++s) mbar_init(bar(b + MR + s), 4);
             mbar_init(bar(b + OE), 8);
-            mbar_init(bar(WF + h), 1); mbar_init(bar(WE + h), 20);
+            mbar_init(bar(WF + h), 1); mbar_init(bar(WE + h), 20); mbar_init(bar(AB + h), 8);
         }
         mbar_init(bar(CL), 1);
         for (int s = 0; s < 8; ++s) mbar_init(bar(KSF + s), 1);
@@ -240,8 +240,10 @@ attention_fwd_pair_kernel(const __grid_constant__ CUtensorMap tmap_q, const __gr
                             tma_load_3d(k_s + stk * C::K_STAGE + s * C::K_SUB, &tmap_k, bar(KF + stk), 64 * s, jk * BC, bh_kv);
                         if (QM) {
                             // slot c % 8 held the sums of tile c-8: this load follows S(c-3) of both halves, hence their pull
-                            // of S(c-4) by the warps that read the slot during tile c-8 or by warps that waited for them since
-                            // (B128: a tile may lie past the last key; its scores are masked whatever is added to them)
+                            // of S(c-4) by the warps that read the slot during tile c-8 or by warps that waited for them since;
+                            // a half without a block frees the pair's tiles only after its warps have come to that pair
+                            // (tests/test_pair_keysum_order.py).  (B128: a tile may lie past the last key; its scores are masked
+                            // whatever is added to them)
                             const int key = B128 ? min(jk * BC, N - BC) : jk * BC;
                             mbar_expect_tx(bar(KSF + (c & 7)), 256);
                             bulk_load(smem_base + C::KSUM_OFF + (c & 7) * 256, args.k_sum + (size_t)bh_kv * N + key, 256, bar(KSF + (c & 7)));
@@ -281,6 +283,7 @@ attention_fwd_pair_kernel(const __grid_constant__ CUtensorMap tmap_q, const __gr
             const int n_max = w.n_max;
             if (n_max == 0) break;
             const int n_tiles = w.n[hf], q0 = w.q0[hf];
+            if (QM && n_tiles == 0) arrive0(bar(AB + hf), lane);
             const int row = q0 + r_loc;
             float m_run = -INFINITY;
             const float mu_row = (QM && n_tiles > 0 && row < N) ? args.q_mu[(size_t)w.bh_q[hf] * N + row] : 0.f;
@@ -434,7 +437,7 @@ attention_fwd_pair_kernel(const __grid_constant__ CUtensorMap tmap_q, const __gr
             constexpr uint32_t idesc_s = umma_idesc_bf16(128, BC);
             const uint32_t q_s = smem_base + hf * C::Q_HALF, b_h = bar(hf * HALF);
             const uint32_t q_lo = umma_desc_lo(q_s), k_lo = umma_desc_lo(k_s), d_s = tmem + hf * C::H_COLS + C::S_COL;
-            int t = 0, st = 0, nq = 0;                        // tile, ring stage, Q loads so far
+            int t = 0, st = 0, nq = 0, nab = 0;               // tile, ring stage, Q loads so far, pairs without a block
             uint32_t ph = 0;
             bool ok = true;
             for (int it = 0; ok; ++it) {
@@ -450,6 +453,9 @@ attention_fwd_pair_kernel(const __grid_constant__ CUtensorMap tmap_q, const __gr
                     for (int s = 0; s < C::QSUB; ++s) tma_load_3d(q_s + s * 16384, &tmap_q, b_h + 8 * QF, 64 * s, q0, bh_q);
                     if (!wait_pair(b_h + 8 * QF, (uint32_t)nq & 1u, abort_flag)) { fail(3); break; }
                     ++nq;
+                } else if (QM) {                              // key-sum slots: the warps may still be at the pair before
+                    if (!wait_pair(bar(AB + hf), (uint32_t)nab & 1u, abort_flag)) { fail(20); break; }
+                    ++nab;
                 }
                 for (int jt = 0; jt < n_max; ++jt) {          // S(t): K tile landed, S(t-1) in registers
                     if (!wait_pair(bar(KF + st), ph, abort_flag)) { fail(4); ok = false; break; }

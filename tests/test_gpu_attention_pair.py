@@ -19,6 +19,8 @@ CASES = {
     "non-causal-ragged": (4, 24, 4, 1344, False, False, None),
     "qmean": (4, 32, 8, 1024, True, True, None),
     "qmean-odd-group": (4, 28, 4, 832, True, True, None),               # halves of different length share the key-sum slots
+    "qmean-odd-block-count": (7, 14, 14, 640, False, True, None),       # a half without a block, ten and 14 tiles, after a pair
+    "qmean-odd-block-count-14-tiles": (2, 37, 37, 896, False, True, None),      # on the same SM: the key-sum slots go round
     "head-map": (8, 8, 4, 1088, True, False, [3, 0, 0, 2, 1, 3, 3, 0]),
 }
 
@@ -49,7 +51,7 @@ def test_two_block_kernel_is_bit_identical(name):
 @pytest.mark.parametrize("B, Hq, Hkv, N, causal, qmean, head_map", [
     (4, 32, 8, 1024, True, False, None), (4, 28, 4, 832, True, False, None),      # an odd number of 64-key tiles: N ends inside a tile
     (8, 9, 9, 1152, True, False, None), (64, 16, 8, 64, False, False, None), (4, 24, 4, 1344, False, False, None),
-    (4, 32, 8, 1024, True, True, None), (8, 28, 4, 832, True, True, None), (8, 8, 4, 1088, True, False, [3, 0, 0, 2, 1, 3, 3, 0]),
+    (4, 32, 8, 1024, True, True, None), (8, 28, 4, 832, True, True, None), (7, 14, 14, 640, False, True, None), (8, 8, 4, 1088, True, False, [3, 0, 0, 2, 1, 3, 3, 0]),
 ])
 def test_two_block_kernel_with_128_key_tiles(B, Hq, Hkv, N, causal, qmean, head_map):
     """Against the 128-key kernel (hifa4_attention_ws.cu), which the dump launch always runs."""
