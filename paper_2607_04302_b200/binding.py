@@ -155,7 +155,8 @@ def _check(rc: int, where: str):
 
 # Host time per call matters for short prompts (two launches of 4 and 8 us): pointers travel as plain integers (argtypes
 # turn them into void*), the stream is read as a handle (0.2 us; building a torch.cuda.Stream object takes 3.3 us), and
-# outputs come from empty_like (1.4 us against 2.4 us for torch.empty with a shape).
+# outputs come from empty_like (1.4 us against 2.4 us for torch.empty with a shape) where a tensor of their shape is at hand
+# (the buffers of a QuantizedQKV may be flat views of an arena, of any element type).
 def _ptr(t):
     return None if t is None else t.data_ptr()
 
@@ -340,7 +341,7 @@ def attention_fwd(qkv: QuantizedQKV, causal: bool, Bc: int = 64, out_dtype=F32, 
     prm = _params(causal, Bc, out_dtype, Br=Br, softmax_scale=softmax_scale, qmean=int(qmean),
                   normalizer=int(normalizer), p_dtype=p_dtype)
     if out is None:
-        out = _empty_out(qkv.q_mma, out_dtype)
+        out = qkv.q_mma.new_empty((qkv.B, qkv.Hq, qkv.N, qkv.d), dtype=_TORCH_DT[out_dtype])
     st = qkv.struct()
     dbg_p, dump = None, None
     if debug_blocks:
