@@ -157,10 +157,11 @@ const char* hifa4_status_string(int status);
 /* Self-test of the failure path of the device-side waits (no counterpart in the paper; for deployment
  * checks and for the test-suite).  Launches the Bc = 64, d = 128 attention kernel in an instantiation
  * whose softmax warps withhold the arrival that releases the P V product and whose issuer gives up
- * waiting for it after 2^6 polls (a fraction of a millisecond) instead of 2^18.  When that wait runs out
- * every TMA load has landed and no MMA is in flight; the kernel records HIFA4_ERR_TIMEOUT + 16 * 7 (site 7:
- * the issuer's wait for P V) in *d_status (required, device int, zero on entry), raises the CTA's abort flag,
- * every role leaves through the common exit that frees tensor memory, and the call returns normally.
+ * waiting for it after 2^6 polls (at most a fraction of a millisecond) instead of 2^18.  That wait begins
+ * only when every TMA load has landed and no MMA is in flight.  When it runs out the kernel records
+ * HIFA4_ERR_TIMEOUT + 16 * 7 (site 7: the issuer's wait for P V) in *d_status (required, device int, zero on
+ * entry), raises the CTA's abort flag, every role leaves through the common exit that frees tensor memory, and
+ * the call returns normally.
  * `out` is not written.  Arguments as hifa4_attention_fwd (prm: Bc = 64, no variant flags; shape: d = 128);
  * a one-CTA problem (N <= 128, one head) is what the test-suite uses.  Nothing hangs, faults or traps. */
 int hifa4_selftest_wait_timeout(const hifa4_shape* shape, const hifa4_qkv* qkv, const hifa4_attn_params* prm,

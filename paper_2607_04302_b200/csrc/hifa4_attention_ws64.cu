@@ -114,9 +114,11 @@ static __device__ __forceinline__ void arrive_lane0(uint32_t bar, int lane)
                  ::"r"(bar), "r"(lane) : "memory");
 }
 
-// SELFTEST: the instantiation behind hifa4_selftest_wait_timeout.  Its softmax warps withhold the arrival that
-// releases P V and the issuer's wait for it gives up after 2^6 polls instead of 2^18; by then every TMA load
-// has landed and no MMA is in flight, so the CTA leaves through the ordinary failure exit.
+// SELFTEST: the instantiation behind hifa4_selftest_wait_timeout.  Its softmax warps withhold the arrival that releases P V,
+// and the issuer's wait for it gives up after 2^6 polls instead of 2^18 (a poll has no least duration).  Only the first two
+// tiles are loaded and multiplied, their V^T loads count on barriers of their own, and the issuer first waits, with the full
+// limit, for those loads and for both S = Q K^T: when the short wait begins, every TMA load has landed and no MMA is in flight,
+// so the CTA can leave through the ordinary failure exit however soon it runs out.
 // QRAW: the Q tensor map is over the raw 16-bit Q; the softmax threads smooth and HIF4-quantize their CTA's 128 rows
 // in shared memory (Algorithm 1 line 1) before the first S = Q K^T, so Q-hat never travels through HBM.
 // F8QK: the kind::f8f6f4 experiment.  Q-hat and K-hat arrive as E4M3 images of element x micro-exponent (integers up
@@ -193,8 +195,9 @@ attention_fwd_ws64_kernel(const __grid_constant__ CUtensorMap tmap_q, const __gr
     };
     auto load_v = [&](int jt) {                               // V^T tile jt into stage jt % 2
         const int st = jt & 1;
-        mbar_expect_tx(bar(BAR_PVGO + (jt & (NG - 1))), D * 128);
-        tma_load_3d(v_s + st * V_STAGE, &tmap_v, bar(BAR_PVGO + (jt & (NG - 1))), jt * BC, 0, bh_kv);
+        const uint32_t go = bar(SELFTEST ? BAR_KSF + st : BAR_PVGO + (jt & (NG - 1)));
+        mbar_expect_tx(go, D * 128);
+        tma_load_3d(v_s + st * V_STAGE, &tmap_v, go, jt * BC, 0, bh_kv);
     };
 
     if (warp == W_QK && lane == 0) {
@@ -261,7 +264,8 @@ attention_fwd_ws64_kernel(const __grid_constant__ CUtensorMap tmap_q, const __gr
             const uint32_t q_lo = umma_desc_lo(q_s), k_lo = umma_desc_lo(k_s);
             bool ok = wait64(bar(C::Q_IN_TMEM || QRAW ? BAR_QT : BAR_Q), 0, abort_flag);
             if (!ok) fail(3);
-            for (int jt = 0; ok && jt < n_tiles; ++jt) {      // S(jt): K tile landed, S(jt-1) in registers
+            const int n_issue = SELFTEST ? min(n_tiles, STAGES) : n_tiles;
+            for (int jt = 0; ok && jt < n_issue; ++jt) {      // S(jt): K tile landed, S(jt-1) in registers
                 const int st = jt & 1;
                 const uint32_t ph = (uint32_t)(jt >> 1) & 1u;
                 if (!wait64(bar(BAR_QKGO + st), ph, abort_flag)) { fail(4); break; }
@@ -282,7 +286,7 @@ attention_fwd_ws64_kernel(const __grid_constant__ CUtensorMap tmap_q, const __gr
                 }
                 umma_commit(bar(BAR_SF + (jt & (NG - 1))));
                 umma_commit(bar(BAR_KE + st));
-                if (jt + 2 < n_tiles) {                        // refill the stage once this MMA has read it
+                if (jt + 2 < n_issue) {                        // refill the stage once this MMA has read it
                     if (!wait64(bar(BAR_KE + st), ph, abort_flag)) { fail(1); break; }
                     load_k(jt + 2);
                 }
@@ -296,6 +300,13 @@ attention_fwd_ws64_kernel(const __grid_constant__ CUtensorMap tmap_q, const __gr
             const uint32_t v_lo = umma_desc_lo(v_s);
             load_v(0);
             if (n_tiles > 1) load_v(1);
+            if constexpr (SELFTEST) {                          // KE[tile]: S of the tile complete, hence Q and its K tile landed
+                bool quiet = true;
+                for (int jt = 0; quiet && jt < min(n_tiles, STAGES); ++jt)
+                    quiet = wait64(bar(BAR_KSF + jt), 0, abort_flag) && wait64(bar(BAR_SF + jt), 0, abort_flag) &&
+                            wait64(bar(BAR_KE + jt), 0, abort_flag);
+                if (!quiet) fail(2);
+            }
             for (int jt = 0; jt < n_tiles; ++jt) {            // V^T tile landed, P-hat(jt) stored, history rescaled
                 const int st = jt & 1;
                 const uint32_t ph = (uint32_t)(jt >> 1) & 1u;

@@ -282,7 +282,7 @@ def test_nonzero_status_word_makes_every_kernel_family_a_no_op(hb, par, d, Bc, n
 
 def test_expired_device_wait_is_reported_and_leaves_the_device_usable(hb, par):
     """The failure path of the bounded device-side waits, exercised without hanging or faulting anything: the
-    self-test instantiation withholds the arrival that releases P V, the issuer's wait runs out after 2^12 polls,
+    self-test instantiation withholds the arrival that releases P V, the issuer's wait runs out after 2^6 polls,
     the status word reads HIFA4_ERR_TIMEOUT + 16 * site (site 7 = that wait), the call returns, the output buffer
     is untouched, and the next ordinary call on the same buffers passes parity (tensor memory was freed, no
     barrier stayed armed)."""
