@@ -283,8 +283,7 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_co
 
 fail:
     if (tid == 0 && args.d_status) atomicExch(args.d_status, HIFA4_ERR_TIMEOUT + 16 * fail_site);
-    // give copies and MMAs still in flight a bounded chance to land before the CTA's memory goes away
-    for (int i = 0; i < 64; ++i) { mbar_try_wait(bar_kv, 0); mbar_try_wait(bar_mma, 0); }
+    let_copies_land();                                    // before the CTA's memory goes away
 
 done:
     tc_fence_before();

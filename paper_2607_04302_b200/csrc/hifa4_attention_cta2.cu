@@ -657,6 +657,7 @@ attention_fwd_cta2_kernel(const __grid_constant__ CUtensorMap tmap_q, const __gr
     cluster_sync();                                           // the partner may still arrive on this CTA's barriers
     if (warp == C::W_LD) {
         __syncwarp();
+        if (flag(abort_flag) == 1) let_copies_land();
         asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(C::TMEM_COLS) : "memory");
     }
 }

@@ -531,7 +531,11 @@ attention_fwd_pair_kernel(const __grid_constant__ CUtensorMap tmap_q, const __gr
 
     tc_fence_before();
     __syncthreads();
-    if (warp == C::W_LD) { __syncwarp(); tmem_dealloc(tmem, C::TMEM_COLS); }
+    if (warp == C::W_LD) {
+        __syncwarp();
+        if (ld_flag(abort_flag) == 1) let_copies_land();
+        tmem_dealloc(tmem, C::TMEM_COLS);
+    }
 }
 
 template <bool QM, bool B128>

@@ -19,7 +19,7 @@
 // MMAs issued by one thread complete in order, which is what makes the buffer reuse safe: S(j+2)
 // is issued after PV(j), whose A operand is P-hat(j).
 // Every wait is bounded; a wait that expires raises the abort flag, writes the status word and
-// every role falls through to the common exit (tensor memory is freed).
+// every role falls through to the common exit (copies in flight get time to land, tensor memory is freed).
 #include "hifa4_attention.cuh"
 
 namespace hifa4 {
@@ -557,7 +557,11 @@ attention_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid
 
     tc_fence_before();
     __syncthreads();
-    if (warp == W_MMA) { __syncwarp(); tmem_dealloc(tmem, TMEM_COLS); }
+    if (warp == W_MMA) {
+        __syncwarp();
+        if (*abort_flag == 1) let_copies_land();
+        tmem_dealloc(tmem, TMEM_COLS);
+    }
 }
 
 template <int KS, bool DBG, bool QM>

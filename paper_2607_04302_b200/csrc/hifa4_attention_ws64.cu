@@ -589,7 +589,13 @@ attention_fwd_ws64_kernel(const __grid_constant__ CUtensorMap tmap_q, const __gr
 
     tc_fence_before();
     __syncthreads();
-    if (warp == W_QK) { __syncwarp(); tmem_dealloc(tmem, TMEM_COLS); }
+    if (warp == W_QK) {
+        __syncwarp();
+        int gave_up;                                           // (through the shared window: a generic pointer kept until here spills)
+        asm volatile("ld.volatile.shared.s32 %0, [%1];" : "=r"(gave_up) : "r"(bars + 8 * N_BARS + 8) : "memory");
+        if (gave_up == 1) let_copies_land();
+        tmem_dealloc(tmem, TMEM_COLS);
+    }
 }
 
 bool make_u8_map(CUtensorMap* m, void* base, uint64_t heads, uint64_t rows, uint64_t cols, uint32_t box_rows);

@@ -75,6 +75,21 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, uint32_
     return false;
 }
 
+// For a CTA that leaves after a wait has run out: gives what is still on its way to its shared and tensor memory (TMA loads,
+// answers of the launch control, MMAs; all of them take microseconds) a millisecond to land.  By the clock, since the barriers
+// they complete on may lack arrivals of the roles that have given up; the polls are bounded as well.
+__device__ __forceinline__ void let_copies_land()
+{
+    uint64_t t0, t;
+    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t0));
+#pragma unroll 1
+    for (uint32_t i = 0; i < (1u << 16); ++i) {
+        asm volatile("nanosleep.u32 1000;");
+        asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+        if (t - t0 >= 1000000u) break;
+    }
+}
+
 // ------------------------------------------------------------------ TMA
 __device__ __forceinline__ void tma_prefetch_desc(const void* tmap)
 {

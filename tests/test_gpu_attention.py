@@ -307,6 +307,26 @@ def test_expired_device_wait_is_reported_and_leaves_the_device_usable(hb, par):
                                  False, status)
 
 
+def test_failure_exit_gives_copies_time_to_land(hb, par):
+    """A CTA that leaves after a wait has run out holds its shared and tensor memory for another millisecond, in which whatever
+    is still on its way to them lands (the self-test's own wait takes a fraction of that)."""
+    cfg = synth.config("C3", N=128, Hq=1, Hkv=1, causal=False)
+    qkv = hb.quantize_qkv(*(t.to(DEV) for t in synth.make_qkv(cfg)))
+    status = torch.zeros(1, dtype=torch.int32, device=DEV)
+    times = []
+    for _ in range(3):
+        status.zero_()
+        a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+        a.record()
+        hb.selftest_wait_timeout(qkv, False, status)
+        b.record()
+        b.synchronize()
+        times.append(a.elapsed_time(b))
+        assert int(status.item()) == 6 + 16 * 7
+    print("ms", times)
+    assert min(times) >= 1.0
+
+
 @pytest.mark.parametrize("dtype,smooth,causal,p_dtype", [("bf16", True, True, "f16"), ("fp16", True, False, "f16"),
                                                          ("bf16", False, True, "f16"), ("fp16", True, True, "f32")])
 def test_in_kernel_query_quantization_is_bit_identical(hb, par, dtype, smooth, causal, p_dtype):
