@@ -28,7 +28,7 @@
 //   d = 128: 256 tensor-memory columns: [O | l] 0..143 (one N = 144 MMA), S 144..207, P-hat
 //            208..239; Q-hat stays in shared memory (SS-form Q K^T).  101 KB of shared memory, so two
 //            CTAs share an SM and fill each other's synchronisation gaps.
-// Where there is no second block for every SM (four_groups_pay below), d = 64 and 128 run with four groups of softmax warps,
+// Where there is no second block for every SM (four_groups_faster in hifa4_dispatch.h), d = 64 and 128 run with four groups of softmax warps,
 // 16 in all, one CTA per SM: then a tile's own work (2500 clk in a group) limits two groups to 1250 clk per tile, and four
 // of them to the chain P V(j) - rescale - P V(j+1), about 1000.  With the tensor memory of the absent CTA, S has two buffers
 // and every group its own P-hat columns, so that only a warp that rescales waits for the previous P V.
@@ -44,6 +44,7 @@
 // the softmax threads before the first S).
 // Every wait is bounded (see hifa4_attention_ws.cu for the failure protocol).
 #include "hifa4_attention.cuh"
+#include "hifa4_dispatch.h"
 
 namespace hifa4 {
 
@@ -620,18 +621,11 @@ static int launch_ws64(const hifa4_shape& sh, const hifa4_qkv& qkv, const AttnAr
     return launch_dependent(kern, grid, C::THREADS, C::SMEM_BYTES, st, mq, mk, mv, args) == cudaSuccess ? HIFA4_OK : HIFA4_ERR_CUDA;
 }
 
-// Whether four groups of softmax warps, one block per SM, are faster than two groups and two blocks per SM (d = 64 and 128):
-// as long as every block has an SM to itself (d = 64: N = 1024, 8 heads 14.1 -> 12.5 us, N = 4096, 4 heads 44 -> 36; d = 128:
-// 16.7 -> 16.2, 50 -> 47), and under a causal mask, where the last blocks are short ones, a good way beyond (256 blocks:
-// d = 64, N = 2048 27.6 -> 23.8, 4096 49 -> 37, 8192 91 -> 66; d = 128 32.2 -> 30.6, 56 -> 48, 102 -> 84; 288 blocks N = 1536
-// 22.6 -> 22.0 and 26.7 -> 27.9; 320 blocks N = 2048 29.5 -> 32.4 and 34 -> 41), less far for short rows (N = 1024: 192 blocks
-// 15.3 -> 14.0 and 18.4 -> 16.8, 256 blocks 16.6 -> 17.0 and 20.1 -> 21.0; non-causal, 256 blocks 22.6 -> 24.8, 39.1 -> 40.4).
 static bool four_groups_pay(const hifa4_shape& sh, const AttnArgs& args)
 {
     int dev = 0, sms = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return false;
-    const long long blocks = (long long)((sh.N + 127) / 128) * sh.Hq * sh.B;
-    return blocks <= sms || (args.causal && (3 * blocks <= 4 * sms || (sh.N > 1024 && 4 * blocks <= 7 * sms)));
+    return four_groups_faster(sh.d, sh.N, args.causal != 0, (long long)((sh.N + 127) / 128) * sh.Hq * sh.B, sms);
 }
 
 template <int DH>
