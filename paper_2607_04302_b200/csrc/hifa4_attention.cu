@@ -408,19 +408,18 @@ int launch_attention(const hifa4_shape& sh, const HeadMap& map, const hifa4_qkv&
         const int n_kv = sh.B * sh.Hkv;
         int want = prm.causal ? (int)(48e6 / per_kv_head) : (per_kv_head * n_kv > 50e6 ? 1 : n_kv);
         if (want < 1) want = 1;
+        a.unit_heads = heads_per_unit(sh);
         if (sh.q_to_kv || sh.Hq % sh.Hkv) {              // custom head map: whole batch elements only
             int g_b = 1;
             for (int c = 1; c <= sh.B && c * sh.Hkv <= want; ++c)
                 if (sh.B % c == 0) g_b = c;
             a.group_heads = g_b * sh.Hq;
-            a.unit_heads = 1;
             a.group_units = g_b * sh.Hq;
         } else {
             int g_kv = 1;
             for (int c = 1; c <= n_kv && c <= want; ++c)
                 if (n_kv % c == 0) g_kv = c;
             a.group_heads = g_kv * (sh.Hq / sh.Hkv);
-            a.unit_heads = sh.Hq / sh.Hkv;
             a.group_units = g_kv;
         }
     }

@@ -26,6 +26,7 @@
 // 128-key kernel (hifa4_attention_ws.cu), 32 / 8 heads, causal: N = 4096 213 -> 191 us, N = 8192 722 -> 637.
 // Every wait is bounded (see hifa4_attention_ws.cu for the failure protocol).
 #include "hifa4_attention.cuh"
+#include "hifa4_dispatch.h"
 
 namespace hifa4 {
 
@@ -554,25 +555,15 @@ static int launch_pair(const hifa4_shape& sh, const hifa4_qkv& qkv, const AttnAr
     return launch_dependent(kern, grid, C::THREADS, C::SMEM_BYTES, st, mq, mk, mv, args) == cudaSuccess ? HIFA4_OK : HIFA4_ERR_CUDA;
 }
 
-// Whether this kernel is the faster one: a pair per SM and wave here, against up to two blocks per SM in the 64-key kernel,
-// where a block that has its SM to itself runs 1.5 times as fast and a full SM takes 1.1 times as long as a pair.
-// Causal: the grid's heaviest pairs start first, and the comparison only depends on how long they are against the whole:
-// from 1.5 pairs per SM up (N = 2048, 8 / 2 heads: 128 pairs 44 against 35 us, 192 pairs 44 against 43, 256 pairs 46 against
-// 54, 320 pairs 60 against 64).  Non-causal pairs are all equal and come in whole waves (N = 1024, 8 / 2 heads: 64 pairs 26
-// against 18 us, 96 pairs 26 against 28, 160 pairs 47 against 42, 256 pairs 48 against 53, 320 pairs 69 against 66, 512 pairs
-// 91 against 96).  128-key tiles, against hifa4_attention_ws.cu: causal from 1.6 pairs per SM up (N = 2048, 28 and 32 heads: 224
-// pairs 66 against 63 us, 256 pairs 67 against 70; N = 1024, 64 heads 43 against 48), non-causal by the same waves (N = 1024, B =
-// 4, 32 heads 116 against 122; N = 4096, 32 heads 376 against 372).
 bool attention_pair_pays(const hifa4_shape& sh, const hifa4_attn_params& prm)
 {
     if (sh.d != 128 || (prm.Bc != 64 && prm.Bc != 128) || prm.normalizer || prm.p_dtype == HIFA4_F32) return false;
     int dev = 0, sms = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0)
         return false;
-    const long long blocks = (long long)((sh.N + 127) / 128) * sh.Hq * sh.B, pairs = (blocks + 1) / 2;
-    if (prm.causal) return prm.Bc == 128 ? 5 * pairs >= 8 * sms : 2 * pairs >= 3 * sms;
-    const long long waves = (pairs + sms - 1) / sms, full = blocks / (2 * sms), rest = blocks % (2 * sms);
-    return (double)waves <= 1.1 * ((double)full + (rest == 0 ? 0.0 : rest <= sms ? 0.67 : 1.0));
+    const int G = heads_per_unit(sh);
+    const long long unit_blocks = (long long)((sh.N + 127) / 128) * G, units = (long long)(sh.Hq / G) * sh.B;
+    return two_blocks_faster(prm.Bc, sh.N, prm.causal != 0, prm.qmean != 0, unit_blocks * units, (unit_blocks + 1) / 2 * units, sms);
 }
 
 int launch_attention_pair(const hifa4_shape& sh, const hifa4_qkv& qkv, const AttnArgs& args, int Bc, cudaStream_t st)

@@ -83,6 +83,8 @@ int launch_attention(const hifa4_shape& shape, const HeadMap& map, const hifa4_q
 // 128 rows x two 64-channel groups) in its default arithmetic or the FP32-P variant, without Q-Mean (the row mean
 // needs the whole row before any group is quantized).
 bool attention_qraw_supported(const hifa4_shape& shape, const hifa4_attn_params& prm);
+// Query heads whose blocks may share K and V^T tiles: those of a KV head, or one under a custom head map.
+inline int heads_per_unit(const hifa4_shape& sh) { return sh.q_to_kv || sh.Hq % sh.Hkv ? 1 : sh.Hq / sh.Hkv; }
 // Whether hifa4_attention_fwd takes the kernel with two query blocks per CTA for this configuration.
 bool attention_pair_pays(const hifa4_shape& shape, const hifa4_attn_params& prm);
 
