@@ -33,20 +33,52 @@ from paper_2607_04302_b200 import synth  # noqa: E402
 METRIC = "4-bit attention prefill TFLOPS on 1 B200; % of dense 4-bit tensor peak"
 UNIT = "TFLOP/s"
 NOMINAL = {"fp4": 9000.0, "fp8": 4500.0, "bf16": 2250.0}      # dense TFLOP/s, context only
-# executed warp instructions per 32 scores (ncu opcode counters) and DRAM bytes per launch, from the captures
-# summarised in profiles/attention_fwd_ws64_C2.md and profiles/attention_fwd_ws_bc128_C2.md
-NCU_INSTR_PER_WARP_SCORE = {"attention_fwd_ws64_kernel<128>": 15.8, "attention_fwd_ws_kernel<4>": 20.8}
-NCU_TRAFFIC_BYTES = {("C2-qwen3-8b-4k", 64): 70.85e6, ("C2-qwen3-8b-4k", 128): 70.31e6}
-# Issue slots the method itself needs per score on this machine (per 32 scores one warp instruction each):
-# exponential 1, scale-subtract FMA 0.5 (packed), FP16 round trip 1.5, row maximum 0.5, subgroup maxima 0.5,
-# shift selection 1.25, scale-and-round 1.5 (packed), BF16 image 0.5, rescale of the history about 0.7,
-# per-row scalars and tensor-memory traffic about 0.6: 8.5.
-ALGORITHMIC_SLOTS_PER_SCORE = 8.5
+# executed warp instructions per 32 scores and DRAM bytes per launch (ncu), from profiles/attention_pair_and_sm_pairs.md
+NCU_INSTR_PER_WARP_SCORE = {"attention_fwd_pair_kernel<0, 0>": 12.2, "attention_fwd_pair_kernel<0, 1>": 12.0,
+                            "attention_fwd_cta2_kernel<0>": 12.7, "attention_fwd_ws64_kernel<128, fp32 P>": 11.3}
+NCU_TRAFFIC_BYTES = {("C2-qwen3-8b-4k", 64): 68.95e6, ("C2-qwen3-8b-4k", 128): 70.42e6, ("C4-gemma2-9b-8k", 64): 233.4e6}
+# Issue slots the method itself needs per score on this machine (per 32 scores one warp instruction each), with P quantized
+# on packed FP16 pairs: exponential 1, scale-subtract FMA 0.5 (packed), FP16 conversion 0.5, row maximum 0.5, scale by the
+# split reciprocal 1, subgroup maxima 0.7, shift selection 1.1, round 0.5, BF16 image 0.5, rescale of the history about 0.7,
+# per-row scalars and tensor-memory traffic about 0.6: 7.6.
+ALGORITHMIC_SLOTS_PER_SCORE = 7.6
 
 
 def attn_flops(cfg) -> float:
     f = 4.0 * cfg.B * cfg.Hq * cfg.N * cfg.N * cfg.d
     return f / 2 if cfg.causal else f
+
+
+def two_blocks_chosen(cfg, sms: int, qmean: bool = False) -> bool:
+    """Whether the library runs this d = 128 workload in the two-block kernel (csrc/hifa4_dispatch.h)."""
+    unit, units = (cfg.N + 127) // 128 * (cfg.Hq // cfg.Hkv), cfg.Hkv * cfg.B
+    blocks, pairs = unit * units, (unit + 1) // 2 * units
+    if cfg.causal and cfg.N > (128 if cfg.Bc == 128 else 320):
+        return 5 * ((blocks + 1) // 2) >= 8 * sms if cfg.Bc == 128 else 2 * ((blocks + 1) // 2) >= 3 * sms
+    if cfg.causal and cfg.Bc == 64 and cfg.N > 256:
+        return 2 * pairs >= 5 * sms
+    waves = -(-pairs // sms)
+    if cfg.Bc == 128:
+        tiles = (cfg.N + 127) // 128 * 2
+        return 3 + (1.7 if qmean else 1.9) * waves * tiles <= -(-blocks // sms) * (tiles + 2)
+    full, rest = divmod(blocks, 2 * sms)
+    tiles = (cfg.N + 63) // 64
+    return 3 + waves * tiles <= (full + (0 if rest == 0 else 0.67 if rest <= sms else 1)) * (tiles + 1.5)
+
+
+def attention_kernel(cfg, *, p_f32=False, qmean=False, f8qk=False, sms=148) -> str:
+    """Name of the attention kernel that the timed step launches."""
+    qm = int(bool(qmean))
+    if f8qk:
+        return "attention_fwd_ws64_kernel<128, f8f6f4 experiment> + 2 x f8_image_kernel"
+    if cfg.d == 128 and not p_f32 and two_blocks_chosen(cfg, sms, qmean):
+        return f"attention_fwd_pair_kernel<{qm}, {int(cfg.Bc == 128)}>"
+    blocks = (cfg.N + 127) // 128 * cfg.Hq * cfg.B
+    if cfg.d == 256 and cfg.Bc == 64 and not p_f32 and blocks > sms:
+        return f"attention_fwd_cta2_kernel<{qm}>"
+    if cfg.Bc == 64:
+        return f"attention_fwd_ws64_kernel<{cfg.d}{', fp32 P' if p_f32 else ''}>"
+    return "attention_fwd_ws_kernel<4>" if cfg.d == 128 else f"attention_fwd_kernel<{cfg.d},{cfg.Bc}>"
 
 
 def measured_peaks():
@@ -658,14 +690,8 @@ def main():
     value = whole_job_tflops(cfg, world, args.steps, total_ms)
     attn_avg_ms = sum(attn_ms) / len(attn_ms)
     achieved = fl / (attn_avg_ms * 1e-3) / 1e12
-    if args.f8qk:
-        kern = "attention_fwd_ws64_kernel<128, f8f6f4 experiment> + 2 x f8_image_kernel"
-    elif cfg.Bc == 64 and cfg.d in (128, 256):
-        kern = f"attention_fwd_ws64_kernel<{cfg.d}>"
-    elif cfg.Bc == 128 and cfg.d == 128:
-        kern = "attention_fwd_ws_kernel<4>"
-    else:
-        kern = f"attention_fwd_kernel<{cfg.d},{cfg.Bc}>"
+    kern = attention_kernel(cfg, p_f32=args.p_f32, qmean=args.qmean, f8qk=args.f8qk,
+                            sms=torch.cuda.get_device_properties(dev).multi_processor_count)
     frac_measured = {"bf16_driver_measured": achieved / peaks["bf16"]}
     if gemm:
         if gemm.get("bf16_tflops"):
@@ -677,7 +703,7 @@ def main():
             frac_measured["fp4_this_run"] = achieved / gemm["fp4_tflops"]
     roofline = {"bound": "tensor", "kernel": kern, "achieved": achieved, "peak": peaks["bf16"],
                 "unit": "TFLOP/s", "frac": achieved / peaks["bf16"], "frac_of_measured": frac_measured,
-                "traffic": NCU_TRAFFIC_BYTES.get((cfg.name, cfg.Bc) if cfg.causal and not args.p_f32 else None),
+                "traffic": NCU_TRAFFIC_BYTES.get((cfg.name, cfg.Bc) if cfg.causal and not args.p_f32 and not args.qmean else None),
                 "peak_source": f"{peaks['source']} cuBLAS bf16 burst (the MMA kind issued is kind::f16 on BF16 images)",
                 "avg_launch_ms": attn_avg_ms,
                 "timed_in": "a second pass of the same steps with one event between the two launches "

@@ -101,3 +101,20 @@ def test_the_cases_of_the_gpu_tests_reach_the_kernels_they_name(rules):
             if rules.four_groups(d, N, int(causal), (N + 127) // 128 * Hq * B, SMS):
                 seen.add((d, (N + 63) // 64 % 4))
     assert seen == {(d, r) for d in (64, 128) for r in range(4)}            # every remainder of tiles by groups
+
+
+def test_bench_names_the_kernel_that_runs(rules):
+    import bench
+    from paper_2607_04302_b200 import synth
+    for Bc in (64, 128):
+        for N in (64, 128, 256, 320, 384, 1024, 1152, 4096):
+            for B, Hq, Hkv in ((1, 1, 1), (1, 32, 8), (4, 28, 4), (8, 8, 8), (20, 8, 8)):
+                for causal in (True, False):
+                    for qmean in (False, True):
+                        cfg = synth.config("C2", B=B, Hq=Hq, Hkv=Hkv, N=N, causal=causal, Bc=Bc)
+                        unit, units = (N + 127) // 128 * (Hq // Hkv), Hkv * B
+                        want = rules.two_blocks(Bc, N, int(causal), int(qmean), unit * units, (unit + 1) // 2 * units, SMS)
+                        assert bench.two_blocks_chosen(cfg, SMS, qmean) == bool(want), (Bc, N, B, Hq, Hkv, causal, qmean)
+    assert bench.attention_kernel(synth.config("C2")) == "attention_fwd_pair_kernel<0, 0>"
+    assert bench.attention_kernel(synth.config("C4")) == "attention_fwd_cta2_kernel<0>"
+    assert bench.attention_kernel(synth.config("C1")) == "attention_fwd_ws64_kernel<128>"
