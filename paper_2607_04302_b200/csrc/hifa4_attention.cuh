@@ -210,7 +210,9 @@ __device__ __forceinline__ PQuantConst<PF32> p_quant_const(float c1, float mL, f
         const uint32_t sh = (uint32_t)((small ? 37 : 49) - e) * 0x04000400u;
         const uint32_t top = (small ? 12u : 0u) * 0x04000400u;
         k.hi = __byte_perm(0x3A663C00u, 0x38923955u, sel) + sh;            // RN16(4/(4+M)) * 2^(49-e-s)
-        k.lo = M ? h2_mul(k.hi, 0x0C000C00u) : 0u;                         // RN16(hi * 2^-12): subnormal from S = 10 up
+        // RN16(hi * 2^-12), subnormal from S = 10 up.  (The factor is chosen, not the product: the other way round the two-block
+        // kernel took 0.6 % longer, 541 against 538 us for 32 / 8 heads, N = 8192, causal.)
+        k.lo = h2_mul(k.hi, M ? 0x0C000C00u : 0u);
         k.tadd = 0xC0FFC0FFu + top;                                        // 1023 - bits(3.5 * 2^-s), per half
         k.magic = 0x62006200u - top;                                       // 768 * 2^-s
         const uint32_t m5 = (uint32_t)M << 5;
