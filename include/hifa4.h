@@ -259,10 +259,12 @@ size_t hifa4_attention_workspace_bytes(const hifa4_shape* shape, const hifa4_att
  *   *_mma images are read).  out: [B,Hq,N,d] of prm->out_dtype.
  *   workspace: at least hifa4_attention_workspace_bytes() bytes (NULL if 0).
  *   dbg: NULL, or a P-hat dump request.
- * Scheduling note (calibration and quantization alike): for Bc = 64 the grid is launched with programmatic stream
- * serialization, i.e. its CTAs may become resident while the preceding kernel
- * of the stream is still draining; they read and write no global memory before
- * that kernel has completed, so the usual stream order of results holds. */
+ * Scheduling note (calibration and quantization alike): the grids are launched
+ * with programmatic stream serialization (all but those of the 128-key and the
+ * one-thread-per-row kernel), i.e. their CTAs may become resident while the
+ * preceding kernel of the stream is still draining; the status word aside, they
+ * read and write no global memory before that kernel has completed, so the usual
+ * stream order of results holds. */
 int hifa4_attention_fwd(const hifa4_shape* shape, const hifa4_qkv* qkv,
                         const hifa4_attn_params* prm, void* out, void* workspace,
                         const hifa4_debug* dbg, int* d_status, void* stream);
@@ -313,10 +315,11 @@ int hifa4_attention_fwd_f8qk(const hifa4_shape* shape, const hifa4_qkv* qkv,
 size_t hifa4_attention_raw_workspace_bytes(const hifa4_shape* shape, const hifa4_attn_params* prm);
 
 /* Algorithm 1 end to end on raw post-RoPE Q/K/V: hifa4_quantize_qkv into
- * `workspace`, then hifa4_attention_fwd; where hifa4_attention_fwd_qraw supports
- * the configuration, only K and V are quantized into the workspace and Q is
- * quantized inside the attention kernel (same result).  s, inv_s as in
- * hifa4_quantize_qkv. */
+ * `workspace`, then hifa4_attention_fwd (same result).  What the workspace holds
+ * afterwards is not defined: only the operand images that the attention kernel
+ * reads are formed, no codes and no metadata, and for large problems that
+ * hifa4_attention_fwd_qraw supports those of K and V only, Q being quantized
+ * inside the attention kernel.  s, inv_s as in hifa4_quantize_qkv. */
 int hifa4_attention_fwd_raw(const hifa4_shape* shape, const void* q, const void* k, const void* v,
                             const float* s, const float* inv_s, const hifa4_attn_params* prm,
                             void* out, void* workspace, size_t workspace_bytes,

@@ -334,7 +334,10 @@ int hifa4_attention_fwd_raw(const hifa4_shape* shape, const void* q, const void*
     if ((s == nullptr) != (inv_s == nullptr)) return HIFA4_ERR_INVALID_ARG;
     // K and V here, Q inside the attention kernel: pays once the Q-hat image (written, then read) is large; measured
     // on B200 at d = 128: -1 to -3 % of the two launches from 64k query rows up, slower below.  The kernel with two query
-    // blocks per CTA gains more than that (5 to 10 %) and takes Q-hat, so its sizes go through the quantizer.
+    // blocks per CTA takes Q-hat; where it is the faster one, its sizes go through the quantizer.  Whole calls, that way against
+    // raw Q in the 64-key kernel: under sustained load within 2 % (32 / 8 heads, causal: N = 4096 185 and 185 us, 8192 641 and
+    // 646, 32768 8.93 and 8.99 ms, B = 4 N = 1024 78 and 76, N = 2048 223 and 226, N = 4096 724 and 739); single calls with the
+    // chip idle before them, N = 2048 75 and 83, B = 4 N = 4096 709 and 710, N = 8192 638 and 624, 32768 8.27 and 7.93 ms.
     if (attention_qraw_supported(*shape, *prm) && !attention_pair_pays(*shape, *prm) && (long long)shape->B * shape->Hq * shape->N >= 65536) {
         if ((rc = quantize_common(shape, nullptr, k, v, s, inv_s, &bufs, false, stream))) return rc;
         return hifa4_attention_fwd_qraw(shape, q, s, &bufs, prm, out, (char*)workspace + used, d_status, stream);

@@ -4,8 +4,9 @@
 // The two blocks ("halves") belong to query heads of one KV head, so every K and V^T tile is loaded once for 256
 // query rows instead of once for 128: with one block per CTA and two CTAs per SM the tiles cross L2 -> SM at 9 TB/s,
 // and leaving those loads out altogether made long launches 13-16 % shorter (the clocks of long launches follow the power
-// they draw).  Against that kernel, sustained: 32 / 8 heads causal N = 4096 173 -> 161 us, N = 16384 2.36 -> 2.23 ms, B = 4
-// N = 1024 63 -> 57 us, B = 2 N = 4096 non-causal 630 -> 586 us.  d = 64 stays there (350 against 380 us, 12 / 4 heads, B =
+// they draw).  Against that kernel, sustained: 32 / 8 heads causal N = 2048 52 -> 48 us, N = 4096 168 -> 166, N = 16384 2.31 ->
+// 2.29 ms, B = 4 N = 2048 197 -> 187 us, N = 4096 681 -> 655, non-causal 1233 -> 1205; single calls on an idle chip, which do
+// not reach the power cap, are 1 to 4 % slower from N = 8192 up.  hifa4_dispatch.h says when it is taken.  d = 64 stays there (350 against 380 us, 12 / 4 heads, B =
 // 2, N = 8192: its tiles are half as large and its softmax share twice).  Apart from the
 // shared tiles the halves run independently of one another, each as the 64-key kernel (hifa4_attention_ws64.cu) runs a
 // CTA.  Warps:
