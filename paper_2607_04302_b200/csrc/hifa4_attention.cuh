@@ -27,6 +27,7 @@ struct AttnArgs {
     int group_heads;              // CTA order: groups of this many (batch, query head) pairs, one group after the other
     int unit_heads, group_units;  // two-block kernel: query heads per unit (G, or 1 under a custom head map), units per group
     float c0, c1;                 // sigma, sigma * log2(e)
+    float2 c1c1;                  // {c1, c1}, the operand of packed instructions as it stands
     int normalizer;               // 1: l accumulates the unquantized P (mismatched), not P-hat
     unsigned long long* hist;     // mass-error histogram [n_bins + 2] or null
     int n_bins;
@@ -151,24 +152,24 @@ __device__ __forceinline__ float p_of_score(float acc, float c1, float mL)
 
 // Arithmetic of the fused form.  P is FP16, so the quantizer runs on packed FP16 pairs from the conversion on and
 // hands over a packed BF16 image: no widening back to FP32, no repacking.  The softmax warps are bound by instruction
-// issue: 13.9 executed warp instructions per score (polls included) instead of the 15.8 of the FP32 form, and the
-// attention of 32 / 8 heads at d = 128, causal, takes 178 instead of 187 us at N = 4096, 2.04 instead of 2.16 ms at
-// N = 16384 (B200, CUDA events).  In units of S/2:
-//   q = RN(p * (2/S) 2^-s)          2/S = hi + lo in two FP16 constants (the mantissas 4/(4+M) repeat with a period
-//                                   that divides 12, so one FP16 constant errs by 2^-12, which is not enough):
-//                                   q = fma(p, hi, RN(p * lo)).  Exactly on every rounding tie and on the right side
-//                                   of it everywhere else (P exceeds 1 where the running maximum, an FP16 value, was
-//                                   rounded down: up to e^8 for scaled scores of 16384 to 32768.  For S >= 10 lo is
-//                                   a subnormal with a few bits, which is all that a correction of 2^-12 needs)
-//   y = q + 1.5 * 2^(9+k) 2^-s      rounds q to the nearest multiple of the subgroup's step, ties to even;
-//                                   the low bits of y are the element code m
-//   v = fma_bf16(y, c, -n)          the bit pattern of y read as BF16 is 2^E (1 + m/128) with E known from k and s, so
-//                                   one BF16 FMA with c = step * 128 * 2^-E, n = step * 128 gives m * step exactly
-// s is 0 or 12: it keeps 2/S finite in FP16 for groups whose maximum is below 2^-12.  The shift k of a 4-key subgroup
-// is read off the bit pattern of its largest q: need = number of thresholds 3.5, 7 (1.75 S, 3.5 S) exceeded, then
+// issue and by the power the SM draws: against a quantizer that multiplied by one reciprocal split into two constants (a product
+// and an FMA per pair, then an addition; shift constants by five operations instead of three) the attention of 32 / 8 heads at
+// d = 128, causal, takes 142 instead of 152 us at N = 4096 and 504 instead of 539 at N = 8192 (B200, back to back, two-block
+// kernel).  In units of S/2:
+//   q = RN(p * c1)                  c1 * c2 = 2/S up to 7e-5, two FP16 factors per mantissa of S, c2 near 1 (one FP16 constant
+//   y = fma(q, c2, 2^(9+k))         errs by 2^-12, which is not enough).  The factors are chosen so that the rounding of q lands on
+//                                   the side of a rounding tie on which p lies, and for p on the tie on the side of the even
+//                                   multiple: the FMA rounds p * 2/S to the nearest multiple of the subgroup's step, ties to
+//                                   even, exactly.  The low bits of y are the element code m
+//   v = fma_bf16(y, c, -n)          the bit pattern of y read as BF16 is 2^E (1 + m/128) with E known from k, so one BF16 FMA
+//                                   with c = step * 128 * 2^-E, n = step * 128 gives m * step exactly
+// (P exceeds 1 where the running maximum, an FP16 value, was rounded down: up to e^8 for scaled scores of 16384 to 32768.)
+// Groups whose maximum is below 2^-12 move a factor 2^12 from c1 to c2: c1 stays finite.  The shift k of a 4-key subgroup
+// is read off the bit pattern of its largest q: need = number of thresholds 1.75 S, 3.5 S that p exceeds, then
 // k_t = max(need_t, need_other - 1) (that is the pair rule: the level-2 bit is set iff max(need) = 2 or min(need) >= 1,
-// and a subgroup that needs no shift of its own still gets one when its partner needs two); the two subgroups of a unit
-// share packed 16-bit integer operations.  tests/test_p_quantizer_arithmetic.py checks the scheme on every finite FP16 P
+// and a subgroup that needs no shift of its own still gets one when its partner needs two), which is the need of
+// max(q_t, q_other / 2); the two subgroups of a unit share packed 16-bit integer operations, whose sum carries k straight
+// into the exponent of the magic constant.  tests/test_p_quantizer_factors.py checks the scheme on every finite FP16 P
 // under every scale a group maximum can select and every shift.
 // The FP32-P variant keeps the FP32 form of the same scheme: q = RZ(p * (4/S)) (exactly on ties, see e6m2_inv4),
 // y = q + 1.5 * 2^(23+k), v = fma(y, S/4, -magic*S/4), two elements per f32x2 operation.
@@ -180,17 +181,17 @@ template <> struct PQuantConst<true> {
 };
 template <> struct PQuantConst<false> {
     uint64_t c1c1, nml;
-    uint32_t hi, lo, tadd, magic, c, n;          // packed pairs of equal halves
+    uint32_t f1, f2, tadd, n;                    // packed pairs of equal halves: c1, c2, threshold, -step * 128 at k = 0
     uint32_t s4_bits;                            // P-hat dump only
 };
 
 // Constants from the group maximum A of P.  A = 0 (every key masked) needs no branch: the scale stays finite, every p
 // is 0 and every product below is an exact zero.
 template <bool PF32>
-__device__ __forceinline__ PQuantConst<PF32> p_quant_const(float c1, float mL, float A)
+__device__ __forceinline__ PQuantConst<PF32> p_quant_const(const float2& c1c1, float mL, float A)
 {
     PQuantConst<PF32> k;
-    k.c1c1 = pack2(c1, c1);
+    k.c1c1 = reinterpret_cast<const uint64_t&>(c1c1);
     k.nml = pack2(-mL, -mL);
     if constexpr (PF32) {
         const int code = e6m2_code_for_max(A);
@@ -203,22 +204,16 @@ __device__ __forceinline__ PQuantConst<PF32> p_quant_const(float c1, float mL, f
         k.inv44 = pack2(inv4, inv4);
         k.s44 = pack2(S4, S4);
     } else {
-        const bool small = A < 0x1p-12f;
-        const int code = e6m2_code_for_max(fmaxf(A, 0x1p-24f));
-        const int e = code >> 2, M = code & 3;
-        const uint32_t sel = 0x1010u + 0x2222u * (uint32_t)M;              // both halves = entry M of a table of four
-        const uint32_t sh = (uint32_t)((small ? 37 : 49) - e) * 0x04000400u;
-        const uint32_t top = (small ? 12u : 0u) * 0x04000400u;
-        k.hi = __byte_perm(0x3A663C00u, 0x38923955u, sel) + sh;            // RN16(4/(4+M)) * 2^(49-e-s)
-        // RN16(hi * 2^-12), subnormal from S = 10 up.  (The factor is chosen, not the product: the other way round the two-block
-        // kernel took 0.6 % longer, 541 against 538 us for 32 / 8 heads, N = 8192, causal.)
-        k.lo = h2_mul(k.hi, M ? 0x0C000C00u : 0u);
-        k.tadd = 0xC0FFC0FFu + top;                                        // 1023 - bits(3.5 * 2^-s), per half
-        k.magic = 0x62006200u - top;                                       // 768 * 2^-s
-        const uint32_t m5 = (uint32_t)M << 5;
-        k.c = (((uint32_t)(e + (small ? 111 : 15)) << 7) | m5) * 0x00010001u;
-        k.n = (0x8000u | ((uint32_t)(e + 84) << 7) | m5) * 0x00010001u;
-        k.s4_bits = ((uint32_t)((code >> 2) + 77) << 23) | ((uint32_t)M << 21);
+        // t: the upper bits of S, the smallest E6M2 value with 7 S >= A, as a float (exponent, two mantissa bits).  The constant
+        // is below 1/7 by less than 2^-25: the product never exceeds S where A = 7 S, and A has 11 significant bits
+        const uint32_t t = (__float_as_uint(fmaxf(A, 0x1p-24f) * __uint_as_float(0x3E124924u)) + 0x1FFFFFu) >> 21;
+        const uint32_t sel = 0x1010u + 0x2222u * (t & 3u);                 // both halves = entry M of a table of four
+        const uint32_t top = A < 0x1p-12f ? 0x30003000u : 0u;              // 2^12
+        k.f1 = __byte_perm(0x3C923C00u, 0x3E303F38u, sel) + (127u - (t >> 2)) * 0x04000400u - top;
+        k.f2 = __byte_perm(0x3D9A4000u, 0x39E939E9u, sel) + top;
+        k.tadd = __byte_perm(0x22FF24FFu, 0x1F421F42u, sel) + top;         // 1023 - bits(RN(1.75 S c1)) + bits(512)
+        k.n = t * 0x00200020u + 0x76807680u;                               // 0x8000 | bits(step * 128), - bits(512) >> 3
+        k.s4_bits = (t << 21) - (2u << 23);
     }
     return k;
 }
@@ -252,29 +247,28 @@ __device__ __forceinline__ void quantize_unit(const uint32_t (&p)[4], const PQua
 {
     uint32_t q[4];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) q[i] = h2_fma(p[i], k.hi, h2_mul(p[i], k.lo));
+    for (int i = 0; i < 4; ++i) q[i] = h2_mul(p[i], k.f1);
     const uint32_t a = h2_max(q[0], q[1]), b = h2_max(q[2], q[3]);
     const uint32_t At = h2_max(__byte_perm(a, b, 0x5410), __byte_perm(a, b, 0x7632));     // {subgroup 0, subgroup 1}
-    const uint32_t x = __viaddmax_s16x2(At, k.tadd, 0u);
-    const uint32_t ks = __viaddmax_s16x2(__byte_perm(x, x, 0x1032), 0xFC00FC00u, x);      // max(x_t, x_other - 1024)
-    const uint32_t kk = ks & 0x0C000C00u;                                                  // k_t << 10
-    const uint32_t magic = kk | k.magic;
-    const uint32_t t = kk >> 3;                                                            // k_t << 7
-    const uint32_t n = k.n + t, c = k.c + t - kk;
+    const uint32_t Bt = __viaddmax_s16x2(__byte_perm(At, At, 0x1032), 0xFC00FC00u, At);   // max(A_t, A_other / 2)
+    const uint32_t x = __viaddmax_s16x2(Bt, k.tadd, 0x60006000u);                          // bits(512 * 2^k) + fraction
+    const uint32_t magic = x & 0xFC00FC00u;                                                // 512 * 2^k
+    const uint32_t n = k.n + (magic >> 3);                                                 // -step * 128 (+ k << 7)
+    const uint32_t c = n - magic - 0x40804080u;                                            // step * 128 * 2^-E, E = 65 + 8 k
     const uint32_t magic0 = dup_lo(magic), magic1 = dup_hi(magic);
     uint32_t y[4];
-    y[0] = h2_add(q[0], magic0);
-    y[1] = h2_add(q[1], magic0);
-    y[2] = h2_add(q[2], magic1);
-    y[3] = h2_add(q[3], magic1);
+    y[0] = h2_fma(q[0], k.f2, magic0);
+    y[1] = h2_fma(q[1], k.f2, magic0);
+    y[2] = h2_fma(q[2], k.f2, magic1);
+    y[3] = h2_fma(q[3], k.f2, magic1);
     w[0] = bf2_fma(y[0], dup_lo(c), dup_lo(n));
     w[1] = bf2_fma(y[1], dup_lo(c), dup_lo(n));
     w[2] = bf2_fma(y[2], dup_hi(c), dup_hi(n));
     w[3] = bf2_fma(y[3], dup_hi(c), dup_hi(n));
     codes[0] = __byte_perm(y[0], y[1], 0x6420) & 0x0F0F0F0Fu;
     codes[1] = __byte_perm(y[2], y[3], 0x6420) & 0x0F0F0F0Fu;
-    ks0 = (int)((kk & 0xFFFFu) << 13);
-    ks1 = (int)((kk >> 16) << 13);
+    ks0 = (int)(((magic - 0x60006000u) & 0xFFFFu) << 13);
+    ks1 = (int)(((magic - 0x60006000u) >> 16) << 13);
 }
 // The packed operations pair key i of subgroup 0 with key i of subgroup 1, so that one pair of per-subgroup constants
 // (magic, c) serves four packed operations.  On bit patterns, with x_t = max(bits(At_t) + tadd, 0) = need_t * 2^23 +
@@ -342,21 +336,20 @@ __device__ __forceinline__ void exp_quantize_units(const float (&acc)[NU * 8], c
     }
 }
 
-// Maximum of 64 values: eight chains of eight (three-input maxima), then one chain over the eight.
+// Maximum of 64 values in 32 three-input maxima: seven chains of nine, then one chain over their results and the last value.
 __device__ __forceinline__ float max64(const float (&p)[64])
 {
-    float t8[8];
+    float t[8];
 #pragma unroll
-    for (int c = 0; c < 8; ++c) {
-        float t = max3(p[8 * c], p[8 * c + 1], p[8 * c + 2]);
-        t = max3(t, p[8 * c + 3], p[8 * c + 4]);
-        t = max3(t, p[8 * c + 5], p[8 * c + 6]);
-        t8[c] = fmaxf(t, p[8 * c + 7]);
+    for (int c = 0; c < 7; ++c) {
+        t[c] = max3(p[9 * c], p[9 * c + 1], p[9 * c + 2]);
+        t[c] = max3(t[c], p[9 * c + 3], p[9 * c + 4]);
+        t[c] = max3(t[c], p[9 * c + 5], p[9 * c + 6]);
+        t[c] = max3(t[c], p[9 * c + 7], p[9 * c + 8]);
     }
-    float mx = max3(t8[0], t8[1], t8[2]);
-    mx = max3(mx, t8[3], t8[4]);
-    mx = max3(mx, t8[5], t8[6]);
-    return fmaxf(mx, t8[7]);
+    t[7] = p[63];
+    const float mx = max3(max3(t[0], t[1], t[2]), t[3], t[4]);
+    return fmaxf(max3(mx, t[5], t[6]), t[7]);
 }
 
 // Rescale of a row's history: the D channels and the normaliser column of [O | l] at tensor-memory address t_o times

@@ -469,7 +469,7 @@ attention_fwd_cta2_kernel(const __grid_constant__ CUtensorMap tmap_q, const __gr
 
                 // P = exp(S - m) in FP16 (line 9), P-hat = HIF4(P) (line 10)
                 uint32_t pw[NU * 4];
-                const auto qc = p_quant_const<false>(args.c1, mL, A);
+                const auto qc = p_quant_const<false>(args.c1c1, mL, A);
                 exp_quantize_units<NU, 0, NU, false, false>(p, qc, false, pw, nullptr, nullptr);
                 // this P-hat buffer is free once P V(t-2) has completed
                 if (t >= 2) {

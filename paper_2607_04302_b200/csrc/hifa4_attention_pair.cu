@@ -70,6 +70,12 @@ struct Work {                         // one pair of query blocks
 };
 }  // namespace pairk
 
+static __device__ __forceinline__ uint64_t fma2_here(uint64_t a, uint64_t b, uint64_t c)      // stays between the loads around it
+{
+    uint64_t r;
+    asm volatile("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
 static __device__ __forceinline__ int ld_flag(uint32_t addr)
 {
     int v;
@@ -314,12 +320,16 @@ attention_fwd_pair_kernel(const __grid_constant__ CUtensorMap tmap_q, const __gr
                     const uint32_t ks_s = smem_base + C::KSUM_OFF + (c & 7) * 256;
                     const uint64_t mu2 = pack2(mu_row, mu_row);
 #pragma unroll
-                    for (int i = 0; i < BC / 4; ++i) {
-                        float4 ks;
+                    for (int i = 0; i < BC; i += 8) {
+                        float4 ka, kb;
                         asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
-                                     : "=f"(ks.x), "=f"(ks.y), "=f"(ks.z), "=f"(ks.w) : "r"(ks_s + 16 * i));
-                        unpack2(fma2(mu2, pack2(ks.x, ks.y), pack2(p[4 * i], p[4 * i + 1])), p[4 * i], p[4 * i + 1]);
-                        unpack2(fma2(mu2, pack2(ks.z, ks.w), pack2(p[4 * i + 2], p[4 * i + 3])), p[4 * i + 2], p[4 * i + 3]);
+                                     : "=f"(ka.x), "=f"(ka.y), "=f"(ka.z), "=f"(ka.w) : "r"(ks_s + 4 * i));
+                        asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
+                                     : "=f"(kb.x), "=f"(kb.y), "=f"(kb.z), "=f"(kb.w) : "r"(ks_s + 4 * i + 16));
+                        unpack2(fma2_here(mu2, pack2(ka.x, ka.y), pack2(p[i], p[i + 1])), p[i], p[i + 1]);
+                        unpack2(fma2_here(mu2, pack2(ka.z, ka.w), pack2(p[i + 2], p[i + 3])), p[i + 2], p[i + 3]);
+                        unpack2(fma2_here(mu2, pack2(kb.x, kb.y), pack2(p[i + 4], p[i + 5])), p[i + 4], p[i + 5]);
+                        unpack2(fma2_here(mu2, pack2(kb.z, kb.w), pack2(p[i + 6], p[i + 7])), p[i + 6], p[i + 7]);
                     }
                 }
                 if ((args.causal && (j0 + BC - 1 > q0)) || (j0 + BC > N)) {   // masked scores become -inf: exp gives exact zeros
@@ -359,7 +369,7 @@ attention_fwd_pair_kernel(const __grid_constant__ CUtensorMap tmap_q, const __gr
 
                 // P = exp(S - m) in FP16 (line 9), P-hat = HIF4(P) (line 10)
                 uint32_t pw[NU * 4];
-                const auto qc = p_quant_const<false>(args.c1, mL, A);
+                const auto qc = p_quant_const<false>(args.c1c1, mL, A);
                 exp_quantize_units<NU, 0, NU, false, false>(p, qc, false, pw, nullptr, nullptr);
                 // the P-hat columns and [O | l] are free once P V of the previous tile has completed
                 if (jt > 0) {

@@ -406,7 +406,7 @@ attention_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid
                 }
                 {
                     uint32_t w[NU * 4];
-                    const auto qc = p_quant_const<false>(args.c1, mL, A);
+                    const auto qc = p_quant_const<false>(args.c1c1, mL, A);
                     exp_quantize_units<NU, 0, NU, DBG>(p, qc, A == 0.f, w, dc, ds);
                     // next tile (of this item, or the first of the next item): scores and partial maximum, once the last
                     // scores of this tile are used up (under three quarters of the quantization, as it was, both tiles' scores

@@ -478,7 +478,7 @@ attention_fwd_ws64_kernel(const __grid_constant__ CUtensorMap tmap_q, const __gr
                 if (args.dbg.p_step) ds = args.dbg.p_step + r_idx * (N / 4) + j0 / 4;
             }
             uint32_t w[NU * 4];
-            const auto qc = p_quant_const<PF32>(args.c1, mL, A);
+            const auto qc = p_quant_const<PF32>(args.c1c1, mL, A);
             exp_quantize_units<NU, 0, NU, DBG, PF32>(p, qc, A == 0.f, w, dc, ds);
             if constexpr (NG > 2) {
                 // the group's P-hat columns are free once P V(jt-NG) has completed; only a rescale waits for P V(jt-1)
