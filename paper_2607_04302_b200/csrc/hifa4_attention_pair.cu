@@ -95,6 +95,26 @@ static __device__ __forceinline__ bool wait_pair(uint32_t bar, uint32_t parity, 
     }
     return false;
 }
+// The same for a whole warp.  The verdict is a vote: the warp stays together where a wait fails, and the compiler knows it, keeps
+// the loop state in uniform registers and no reconvergence state; a waiting warp issues one instruction per poll instead of a
+// loop's worth.
+static __device__ __forceinline__ bool wait_warp(uint32_t bar, uint32_t parity, uint32_t abort_flag)
+{
+    if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+#pragma unroll 1
+    for (uint32_t i = 0; i < pairk::WAIT_POLLS / 4; ++i) {
+        if (__all_sync(0xffffffffu, mbar_try_wait4(bar, parity))) return true;
+        if ((i & 15u) == 15u && __any_sync(0xffffffffu, ld_flag(abort_flag))) return false;
+    }
+    return false;
+}
+// The same where the warps wait longest, for P V and, with 128-key tiles, for the other half's maxima: each thread polls in the
+// plain loop and the vote comes once at the end (32 / 8 heads, N = 4096, causal, 134.4 against 135.3 us).
+static __device__ __forceinline__ bool wait_long(uint32_t bar, uint32_t parity, uint32_t abort_flag)
+{
+    return __all_sync(0xffffffffu, wait_pair(bar, parity, abort_flag));
+}
+static __device__ __forceinline__ int uni(int v) { return __shfl_sync(0xffffffffu, v, 0); }      // the same in all lanes, and the compiler knows
 static __device__ __forceinline__ void arrive0(uint32_t bar, int lane)      // one arrival from lane 0 of a converged warp
 {
     asm volatile("{\n\t.reg .pred p;\n\t"
@@ -142,7 +162,7 @@ attention_fwd_pair_kernel(const __grid_constant__ CUtensorMap tmap_q, const __gr
     constexpr int CL_OFF = C::MISC_OFF + 512;                 // answer of the launch control (16-byte aligned)
     volatile Work* work = reinterpret_cast<volatile Work*>(smem_gen + C::MISC_OFF + 544);    // [2]
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     const int N = args.N;
 
     if (warp == C::W_LD && lane == 0) {
@@ -286,11 +306,11 @@ attention_fwd_pair_kernel(const __grid_constant__ CUtensorMap tmap_q, const __gr
         int c0 = 0;                                               // tiles loaded before the current pair
         bool ok = true;
         for (int it = 0; ok; ++it) {
-            if (!wait_pair(bar(WF + (it & 1)), (uint32_t)(it >> 1) & 1u, abort_flag)) { fail(18); break; }
+            if (!wait_warp(bar(WF + (it & 1)), (uint32_t)(it >> 1) & 1u, abort_flag)) { fail(18); break; }
             volatile Work& w = work[it & 1];
-            const int n_max = w.n_max;
+            const int n_max = uni(w.n_max);
             if (n_max == 0) break;
-            const int n_tiles = w.n[hf], q0 = w.q0[hf];
+            const int n_tiles = uni(w.n[hf]), q0 = uni(w.q0[hf]);
             if (QM && n_tiles == 0) arrive0(bar(AB + hf), lane);
             const int row = q0 + r_loc;
             float m_run = -INFINITY;
@@ -299,7 +319,7 @@ attention_fwd_pair_kernel(const __grid_constant__ CUtensorMap tmap_q, const __gr
             for (int jt = (t0 ^ grp) & 1; jt < n_tiles; jt += 2) {
                 const int t = t0 + jt, j0 = jt * BC;               // t % 2 == grp
                 const uint32_t ph = (uint32_t)(t >> 1) & 1u, ph_prev = (uint32_t)((t - 1) >> 1) & 1u;
-                if (!wait_pair(b_own + 8 * SF, ph, abort_flag)) { fail(8); ok = false; break; }
+                if (!wait_warp(b_own + 8 * SF, ph, abort_flag)) { fail(8); ok = false; break; }
                 tc_fence_after();
                 float p[BC];
                 {
@@ -316,7 +336,7 @@ attention_fwd_pair_kernel(const __grid_constant__ CUtensorMap tmap_q, const __gr
 
                 if (QM) {                                          // Q-Mean correction (line 6): + mu_i * sum_c k~_jc
                     const int c = c0 + jt;
-                    if (!wait_pair(bar(KSF + (c & 7)), (uint32_t)(c >> 3) & 1u, abort_flag)) { fail(15); ok = false; break; }
+                    if (!wait_warp(bar(KSF + (c & 7)), (uint32_t)(c >> 3) & 1u, abort_flag)) { fail(15); ok = false; break; }
                     const uint32_t ks_s = smem_base + C::KSUM_OFF + (c & 7) * 256;
                     const uint64_t mu2 = pack2(mu_row, mu_row);
 #pragma unroll
@@ -337,6 +357,9 @@ attention_fwd_pair_kernel(const __grid_constant__ CUtensorMap tmap_q, const __gr
 #pragma unroll
                     for (int i = 0; i < BC; ++i) p[i] = (j0 + i > key_lim) ? -INFINITY : p[i];
                 }
+                // (no instruction: unties the scores from the two blocks of 32 registers that the loads fill, or ptxas spills 48 bytes)
+#pragma unroll
+                for (int i = 0; i < BC; ++i) asm volatile("" : "+f"(p[i]));
                 const float mx = max64(p);                         // row maximum = maximum of the tile's single 64-key group
                 float oth = -INFINITY;
                 if constexpr (B128) {
@@ -348,10 +371,10 @@ attention_fwd_pair_kernel(const __grid_constant__ CUtensorMap tmap_q, const __gr
                     asm volatile("st.shared.f32 [%0], %1;" ::"r"(mx_own + sl), "f"(own) : "memory");
                     __syncwarp();
                     arrive0(b_mr + 8 * grp, lane);
-                    if (!wait_pair(b_mr + 8 * (grp ^ 1), (uint32_t)(t >> 2) & 1u, abort_flag)) { fail(12); ok = false; break; }
+                    if (!wait_long(b_mr + 8 * (grp ^ 1), (uint32_t)(t >> 2) & 1u, abort_flag)) { fail(12); ok = false; break; }
                     asm volatile("ld.shared.f32 %0, [%1];" : "=f"(oth) : "r"((mx_own ^ 512u) + sl) : "memory");
                 } else if (jt > 0) {                               // running maximum after the previous tile, from its owner
-                    if (!wait_pair(b_oth + 8 * MR, ph_prev, abort_flag)) { fail(12); ok = false; break; }
+                    if (!wait_warp(b_oth + 8 * MR, ph_prev, abort_flag)) { fail(12); ok = false; break; }
                     asm volatile("ld.shared.f32 %0, [%1];" : "=f"(m_run) : "r"(mx_own ^ 512u) : "memory");
                 }
                 // running maximum and rescale factor (lines 7-8), both FP16 values.  No branch: r = 1 exactly
@@ -373,7 +396,7 @@ attention_fwd_pair_kernel(const __grid_constant__ CUtensorMap tmap_q, const __gr
                 exp_quantize_units<NU, 0, NU, false, false>(p, qc, false, pw, nullptr, nullptr);
                 // the P-hat columns and [O | l] are free once P V of the previous tile has completed
                 if (jt > 0) {
-                    if (!wait_pair(b_oth + 8 * PV, ph_prev, abort_flag)) { fail(10); ok = false; break; }
+                    if (!wait_long(b_oth + 8 * PV, ph_prev, abort_flag)) { fail(10); ok = false; break; }
                     tc_fence_after();
                 }
                 tmem_st32(t_o + C::P_COL, pw);
@@ -389,7 +412,7 @@ attention_fwd_pair_kernel(const __grid_constant__ CUtensorMap tmap_q, const __gr
 
             // finalize: out = O / l with l rounded to FP16 (line 13); group grp writes channels (d/2) grp ..
             if (n_tiles > 0) {
-                if (!wait_pair(b_h + 8 * PV + 8 * ((t0 - 1) & 1), (uint32_t)((t0 - 1) >> 1) & 1u, abort_flag)) { fail(11); ok = false; break; }
+                if (!wait_warp(b_h + 8 * PV + 8 * ((t0 - 1) & 1), (uint32_t)((t0 - 1) >> 1) & 1u, abort_flag)) { fail(11); ok = false; break; }
                 tc_fence_after();
                 constexpr int NC = D / 2 / 32;                     // 32-column chunks of this thread's channel half
                 uint32_t lr[1];
@@ -493,17 +516,38 @@ attention_fwd_pair_kernel(const __grid_constant__ CUtensorMap tmap_q, const __gr
     } else {
         // ------------------------------------------------------------------ issuer of [O | l] += P-hat [V | 1], both halves
         if (elect_one()) {
+            // The time between "P-hat stored and history rescaled" and the issue of P V is part of the chain that sets the
+            // tile period (20 ns of sleep between polls cost 2.5 %): everything else that a tile waits for (its V^T stage, the
+            // output of the block before) is seen to ahead, and an armed half costs one poll per round (N = 4096, causal,
+            // 134.1 -> 132.1 us; B = 4, N = 2048, non-causal, 254 -> 250)
             constexpr uint32_t idesc_o = umma_idesc_bf16(128, O_COLS);
             const uint32_t v_lo = umma_desc_lo(v_s);
             int it[2] = {0, 0}, jt[2] = {0, 0}, n_max[2] = {0, 0}, n_tiles[2] = {0, 0}, st[2] = {0, 0};
             uint32_t ph[2] = {0, 0}, t[2] = {0, 0}, no[2] = {0, 0};      // parities of the ring round, the tile and the block count
-            bool first[2] = {true, true}, done[2] = {false, false};
+            bool first[2] = {true, true}, done[2] = {false, false}, armed[2] = {false, false};
             uint32_t idle = 0;
             while (!(done[0] && done[1])) {
                 if (++idle > 4 * WAIT_POLLS || ((idle & 63u) == 63u && ld_flag(abort_flag))) { if (idle > 4 * WAIT_POLLS) fail(7); break; }
 #pragma unroll
                 for (int hf = 0; hf < 2; ++hf) {
-                    if (done[hf]) continue;
+                    if (armed[hf]) {
+                        if (!mbar_test_wait(bar(hf * HALF + PGO), t[hf])) continue;
+                        idle = 0;
+                        tc_fence_after();
+                        const uint32_t b0 = v_lo + st[hf] * (C::V_STAGE >> 4);
+                        const uint32_t acc0 = jt[hf] > 0 ? 1u : 0u;
+#pragma unroll
+                        for (int kk = 0; kk < 4; ++kk)          // 16 keys per step; channels and ones block
+                            umma_bf16_ts_lo(tmem + hf * C::H_COLS, tmem + hf * C::H_COLS + C::P_COL + kk * 8, b0 + kk * 2, idesc_o, kk ? 1u : acc0);
+                        umma_commit(bar(hf * HALF + PV + (int)t[hf]));
+                        umma_commit(bar(VE + st[hf]));
+                        armed[hf] = false;
+                        t[hf] ^= 1u;
+                        if (jt[hf] + 1 == n_tiles[hf]) { no[hf] ^= 1u; first[hf] = false; }
+                        ++jt[hf];
+                        if (++st[hf] == STAGES) { st[hf] = 0; ph[hf] ^= 1u; }
+                    }
+                    if (armed[hf] || done[hf]) continue;
                     if (jt[hf] == n_max[hf]) {                  // next pair
                         if (!mbar_test_wait(bar(WF + (it[hf] & 1)), (uint32_t)(it[hf] >> 1) & 1u)) continue;
                         volatile Work& w = work[it[hf] & 1];
@@ -513,29 +557,18 @@ attention_fwd_pair_kernel(const __grid_constant__ CUtensorMap tmap_q, const __gr
                         if (n_max[hf] == 0) { done[hf] = true; continue; }
                         mbar_arrive(bar(WE + (it[hf] & 1)));
                         ++it[hf];
+                        idle = 0;
                     }
-                    const bool mine = jt[hf] < n_tiles[hf];
-                    // P-hat stored and history rescaled, output of the previous block read, V^T tile landed
-                    if (mine && !mbar_test_wait(bar(hf * HALF + PGO), t[hf])) continue;
-                    if (mine && jt[hf] == 0 && !first[hf] && !mbar_test_wait(bar(hf * HALF + OE), no[hf] ^ 1u)) continue;
-                    if (!mbar_test_wait(bar(VF + st[hf]), ph[hf])) continue;
-                    idle = 0;
-                    if (mine) {
-                        tc_fence_after();
-                        const uint32_t b0 = v_lo + st[hf] * (C::V_STAGE >> 4);
-                        const uint32_t acc0 = jt[hf] > 0 ? 1u : 0u;
-#pragma unroll
-                        for (int kk = 0; kk < 4; ++kk)          // 16 keys per step; channels and ones block
-                            umma_bf16_ts_lo(tmem + hf * C::H_COLS, tmem + hf * C::H_COLS + C::P_COL + kk * 8, b0 + kk * 2, idesc_o, kk ? 1u : acc0);
-                        umma_commit(bar(hf * HALF + PV + (int)t[hf]));
-                        umma_commit(bar(VE + st[hf]));
-                        t[hf] ^= 1u;
-                        if (jt[hf] + 1 == n_tiles[hf]) { no[hf] ^= 1u; first[hf] = false; }
+                    if (!mbar_test_wait(bar(VF + st[hf]), ph[hf])) continue;                              // V^T tile landed
+                    if (jt[hf] < n_tiles[hf]) {
+                        // the first P V of a block overwrites the output columns of the block before
+                        armed[hf] = jt[hf] > 0 || first[hf] || mbar_test_wait(bar(hf * HALF + OE), no[hf] ^ 1u);
                     } else {
+                        idle = 0;
                         mbar_arrive(bar(VE + st[hf]));          // the other half's tile only
+                        ++jt[hf];
+                        if (++st[hf] == STAGES) { st[hf] = 0; ph[hf] ^= 1u; }
                     }
-                    ++jt[hf];
-                    if (++st[hf] == STAGES) { st[hf] = 0; ph[hf] ^= 1u; }
                 }
             }
         }

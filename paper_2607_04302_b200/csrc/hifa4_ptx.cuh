@@ -42,6 +42,20 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity)
         : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
     return ok != 0;
 }
+// Up to four of them in a row (a waiting warp issues one instruction per poll instead of a loop's worth).
+__device__ __forceinline__ bool mbar_try_wait4(uint32_t bar, uint32_t parity)
+{
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "@!p mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "@!p mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "@!p mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+    return ok != 0;
+}
 // Non-blocking poll: returns at once whether or not the phase has completed (try_wait may keep the
 // thread suspended for a while when it has not).
 __device__ __forceinline__ bool mbar_test_wait(uint32_t bar, uint32_t parity)
