@@ -38,10 +38,10 @@ NCU_INSTR_PER_WARP_SCORE = {"attention_fwd_pair_kernel<0, 0>": 12.2, "attention_
                             "attention_fwd_cta2_kernel<0>": 12.7, "attention_fwd_ws64_kernel<128, fp32 P>": 11.3}
 NCU_TRAFFIC_BYTES = {("C2-qwen3-8b-4k", 64): 68.95e6, ("C2-qwen3-8b-4k", 128): 70.42e6, ("C4-gemma2-9b-8k", 64): 233.4e6}
 # Issue slots the method itself needs per score on this machine (per 32 scores one warp instruction each), with P quantized
-# on packed FP16 pairs: exponential 1, scale-subtract FMA 0.5 (packed), FP16 conversion 0.5, row maximum 0.5, scale by the
-# split reciprocal 1, subgroup maxima 0.7, shift selection 1.1, round 0.5, BF16 image 0.5, rescale of the history about 0.7,
-# per-row scalars and tensor-memory traffic about 0.6: 7.6.
-ALGORITHMIC_SLOTS_PER_SCORE = 7.6
+# on packed FP16 pairs: exponential 1, scale-subtract FMA 0.5 (packed), FP16 conversion 0.5, row maximum 0.5, scale 0.5,
+# subgroup maxima 0.6, shift selection 0.8, scale and round 0.5, BF16 image 0.5, rescale of the history about 0.7, per-row
+# scalars and tensor-memory traffic about 0.6: 6.7.
+ALGORITHMIC_SLOTS_PER_SCORE = 6.7
 
 
 def attn_flops(cfg) -> float:

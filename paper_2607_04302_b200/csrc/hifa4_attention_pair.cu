@@ -4,10 +4,11 @@
 // The two blocks ("halves") belong to query heads of one KV head, so every K and V^T tile is loaded once for 256
 // query rows instead of once for 128: with one block per CTA and two CTAs per SM the tiles cross L2 -> SM at 9 TB/s,
 // and leaving those loads out altogether made long launches 13-16 % shorter (the clocks of long launches follow the power
-// they draw).  Against that kernel, sustained: 32 / 8 heads causal N = 2048 52 -> 48 us, N = 4096 168 -> 166, N = 16384 2.31 ->
+// they draw).  Against that kernel, sustained, both with an earlier quantizer of P and earlier waits: 32 / 8 heads causal N = 2048 52 -> 48 us, N = 4096 168 -> 166, N = 16384 2.31 ->
 // 2.29 ms, B = 4 N = 2048 197 -> 187 us, N = 4096 681 -> 655, non-causal 1233 -> 1205; single calls on an idle chip, which do
-// not reach the power cap, are 1 to 4 % slower from N = 8192 up.  hifa4_dispatch.h says when it is taken.  d = 64 stays there (350 against 380 us, 12 / 4 heads, B =
-// 2, N = 8192: its tiles are half as large and its softmax share twice).  Apart from the
+// not reach the power cap, are 1 to 4 % slower from N = 8192 up (since then this kernel alone gained 13 %: N = 4096 152 -> 132 us,
+// N = 8192 539 -> 469).  hifa4_dispatch.h says when it is taken.  d = 64 stays there (350 against 380 us, 12 / 4 heads, B = 2,
+// N = 8192: its tiles are half as large and its softmax share twice).  Apart from the
 // shared tiles the halves run independently of one another, each as the 64-key kernel (hifa4_attention_ws64.cu) runs a
 // CTA.  Warps:
 //   0-15   softmax / quantize: warps 8h..8h+3 own the even key tiles of half h, warps 8h+4..8h+7 the odd ones, one
@@ -24,7 +25,7 @@
 // through 2 KB of shared memory per warp, so that stores cover whole 64-byte row pieces.
 // Template flags: Q-Mean (key sums staged in eight slots by the loader, as in the 64-key kernel); B128: 128-key tiles, each a
 // pair of 64-key ones whose owners exchange their maxima (one more hand-off per tile, one rescale less).  Against the
-// 128-key kernel (hifa4_attention_ws.cu), 32 / 8 heads, causal: N = 4096 213 -> 191 us, N = 8192 722 -> 637.
+// 128-key kernel (hifa4_attention_ws.cu), 32 / 8 heads, causal: N = 4096 213 -> 191 us (158 now), N = 8192 722 -> 637.
 // Every wait is bounded (see hifa4_attention_ws.cu for the failure protocol).
 #include "hifa4_attention.cuh"
 #include "hifa4_dispatch.h"
