@@ -34,9 +34,9 @@ METRIC = "4-bit attention prefill TFLOPS on 1 B200; % of dense 4-bit tensor peak
 UNIT = "TFLOP/s"
 NOMINAL = {"fp4": 9000.0, "fp8": 4500.0, "bf16": 2250.0}      # dense TFLOP/s, context only
 # executed warp instructions per 32 scores and DRAM bytes per launch (ncu), from profiles/attention_pair_and_sm_pairs.md
-NCU_INSTR_PER_WARP_SCORE = {"attention_fwd_pair_kernel<0, 0>": 12.2, "attention_fwd_pair_kernel<0, 1>": 12.0,
-                            "attention_fwd_cta2_kernel<0>": 12.7, "attention_fwd_ws64_kernel<128, fp32 P>": 11.3}
-NCU_TRAFFIC_BYTES = {("C2-qwen3-8b-4k", 64): 68.95e6, ("C2-qwen3-8b-4k", 128): 70.42e6, ("C4-gemma2-9b-8k", 64): 233.4e6}
+NCU_INSTR_PER_WARP_SCORE = {"attention_fwd_pair_kernel<0, 0>": 10.3, "attention_fwd_pair_kernel<0, 1>": 10.3,
+                            "attention_fwd_cta2_kernel<0>": 11.7, "attention_fwd_ws64_kernel<128, fp32 P>": 11.3}
+NCU_TRAFFIC_BYTES = {("C2-qwen3-8b-4k", 64): 68.99e6, ("C2-qwen3-8b-4k", 128): 70.12e6, ("C4-gemma2-9b-8k", 64): 232.8e6}
 # Issue slots the method itself needs per score on this machine (per 32 scores one warp instruction each), with P quantized
 # on packed FP16 pairs: exponential 1, scale-subtract FMA 0.5 (packed), FP16 conversion 0.5, row maximum 0.5, scale 0.5,
 # subgroup maxima 0.6, shift selection 0.8, scale and round 0.5, BF16 image 0.5, rescale of the history about 0.7, per-row
