@@ -384,7 +384,9 @@ int launch_attention(const hifa4_shape& sh, const HeadMap& map, const hifa4_qkv&
     const double sigma = prm.softmax_scale != 0.f ? (double)prm.softmax_scale : 1.0 / sqrt((double)sh.d);
     a.c0 = (float)sigma;
     a.c1 = (float)(sigma * 1.4426950408889634074);
-    a.c1c1 = make_float2(a.c1, a.c1);
+    uint32_t c1_bits;
+    memcpy(&c1_bits, &a.c1, sizeof(c1_bits));
+    a.c1c1 = (uint64_t)c1_bits << 32 | c1_bits;
     a.out = out;
     a.qmean = prm.qmean ? 1 : 0;
     a.q_mu = qkv.q_mu;

@@ -27,7 +27,7 @@ struct AttnArgs {
     int group_heads;              // CTA order: groups of this many (batch, query head) pairs, one group after the other
     int unit_heads, group_units;  // two-block kernel: query heads per unit (G, or 1 under a custom head map), units per group
     float c0, c1;                 // sigma, sigma * log2(e)
-    float2 c1c1;                  // {c1, c1}, the operand of packed instructions as it stands
+    uint64_t c1c1;                // {c1, c1}, the operand of packed instructions as it stands
     int normalizer;               // 1: l accumulates the unquantized P (mismatched), not P-hat
     unsigned long long* hist;     // mass-error histogram [n_bins + 2] or null
     int n_bins;
@@ -188,10 +188,10 @@ template <> struct PQuantConst<false> {
 // Constants from the group maximum A of P.  A = 0 (every key masked) needs no branch: the scale stays finite, every p
 // is 0 and every product below is an exact zero.
 template <bool PF32>
-__device__ __forceinline__ PQuantConst<PF32> p_quant_const(const float2& c1c1, float mL, float A)
+__device__ __forceinline__ PQuantConst<PF32> p_quant_const(uint64_t c1c1, float mL, float A)
 {
     PQuantConst<PF32> k;
-    k.c1c1 = reinterpret_cast<const uint64_t&>(c1c1);
+    k.c1c1 = c1c1;
     k.nml = pack2(-mL, -mL);
     if constexpr (PF32) {
         const int code = e6m2_code_for_max(A);

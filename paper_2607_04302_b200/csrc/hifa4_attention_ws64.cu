@@ -478,7 +478,10 @@ attention_fwd_ws64_kernel(const __grid_constant__ CUtensorMap tmap_q, const __gr
                 if (args.dbg.p_step) ds = args.dbg.p_step + r_idx * (N / 4) + j0 / 4;
             }
             uint32_t w[NU * 4];
-            const auto qc = p_quant_const<PF32>(args.c1c1, mL, A);
+            // FP32 P from Q-hat: the pair is formed here.  Read as it stands it makes ptxas spill 36 / 88 bytes (stored / loaded) in that
+            // instantiation (32 / 8 heads, N = 4096: causal 160.8 against 153.0 us, not causal 289.6 against 278.2); with raw Q it is the
+            // other way round (formed here 40 / 72 bytes, 173 against 163 us).
+            const auto qc = p_quant_const<PF32>(PF32 && !QRAW ? pack2(args.c1, args.c1) : args.c1c1, mL, A);
             exp_quantize_units<NU, 0, NU, DBG, PF32>(p, qc, A == 0.f, w, dc, ds);
             if constexpr (NG > 2) {
                 // the group's P-hat columns are free once P V(jt-NG) has completed; only a rescale waits for P V(jt-1)
