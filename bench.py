@@ -53,17 +53,20 @@ def two_blocks_chosen(cfg, sms: int, qmean: bool = False) -> bool:
     """Whether the library runs this d = 128 workload in the two-block kernel (csrc/hifa4_dispatch.h)."""
     unit, units = (cfg.N + 127) // 128 * (cfg.Hq // cfg.Hkv), cfg.Hkv * cfg.B
     blocks, pairs = unit * units, (unit + 1) // 2 * units
-    if cfg.causal and cfg.N > (128 if cfg.Bc == 128 else 320):
-        return 5 * ((blocks + 1) // 2) >= 8 * sms if cfg.Bc == 128 else 2 * ((blocks + 1) // 2) >= 3 * sms
-    if cfg.causal and cfg.Bc == 64 and cfg.N > 256:
-        return 2 * pairs >= 5 * sms
-    waves = -(-pairs // sms)
+    waves, pairs_per_sm = -(-pairs // sms), ((blocks + 1) // 2) / sms
     if cfg.Bc == 128:
+        if cfg.causal and cfg.N > 128:
+            return pairs_per_sm >= min(0.6 + (cfg.N - 256) / 1000.0, 1.37 if qmean else 1.5)
         tiles = (cfg.N + 127) // 128 * 2
-        return 3 + (1.7 if qmean else 1.9) * waves * tiles <= -(-blocks // sms) * (tiles + 2)
+        return 2.9 + (1.63 if qmean else 1.72) * waves * tiles <= -(-blocks // sms) * (tiles + (2.0 if qmean else 1.5))
+    if cfg.causal and cfg.N > 320:
+        return pairs_per_sm >= min(1.05 + (cfg.N - 512) / 4200.0, 1.42)
     full, rest = divmod(blocks, 2 * sms)
     tiles = (cfg.N + 63) // 64
-    return 3 + waves * tiles <= (full + (0 if rest == 0 else 0.67 if rest <= sms else 1)) * (tiles + 1.5)
+    waves64 = full + (0 if rest == 0 else (0.74 if cfg.causal else 0.44) if rest <= sms else 1)
+    if cfg.causal:
+        return 2.2 + 0.74 * waves * tiles <= waves64 * (tiles + 0.75)
+    return 3.1 + (1.02 if qmean else 0.915) * waves * (tiles + 1.3) <= waves64 * (tiles + 4.0)
 
 
 def attention_kernel(cfg, *, p_f32=False, qmean=False, f8qk=False, sms=148) -> str:

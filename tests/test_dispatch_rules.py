@@ -13,38 +13,61 @@ SMS = 148
 
 # d, N, causal, blocks, two groups of softmax warps, four groups
 GROUPS = [
-    (64, 64, True, 192, 5.87, 8.48), (64, 64, False, 130, 4.00, 4.52), (64, 128, True, 192, 7.85, 10.62), (64, 256, True, 96, 6.64, 6.90),
-    (64, 320, True, 192, 8.53, 11.82), (64, 384, True, 153, 9.22, 10.52), (64, 512, True, 192, 10.24, 12.18), (64, 512, False, 96, 9.26, 8.83),
-    (64, 1024, False, 96, 14.54, 12.97), (64, 1024, False, 160, 22.45, 24.62), (64, 2048, False, 256, 40.08, 41.34),
-    (128, 64, False, 1, 4.55, 4.80), (128, 64, True, 192, 6.73, 9.75), (128, 128, False, 1, 6.24, 6.04), (128, 128, True, 152, 9.39, 11.98),
-    (128, 192, True, 192, 9.52, 12.66), (128, 256, True, 192, 10.69, 13.02), (128, 320, True, 192, 10.56, 14.06), (128, 384, True, 192, 12.28, 14.18),
-    (128, 512, False, 96, 11.17, 10.93), (128, 1024, False, 96, 17.12, 16.62),
+    (64, 64, True, 192, 5.51, 8.19), (64, 64, False, 130, 3.87, 4.25), (64, 128, True, 192, 7.37, 10.00),
+    (64, 256, True, 96, 6.13, 6.46), (64, 320, True, 192, 7.92, 11.18), (64, 384, True, 153, 8.53, 9.93),
+    (64, 512, True, 192, 9.49, 11.53), (64, 512, False, 96, 8.40, 8.19), (64, 1024, False, 96, 13.24, 12.14),
+    (64, 1024, False, 160, 19.81, 22.20), (64, 2048, False, 256, 35.53, 37.94), (128, 64, False, 1, 4.40, 4.71),
+    (128, 64, True, 192, 6.34, 9.38), (128, 128, False, 1, 5.94, 5.94), (128, 128, True, 152, 9.06, 11.59),
+    (128, 192, True, 192, 8.94, 12.16), (128, 256, True, 192, 10.05, 12.51), (128, 320, True, 192, 9.86, 13.41),
+    (128, 384, True, 192, 11.70, 13.64), (128, 512, False, 96, 10.34, 10.25), (128, 1024, False, 96, 15.92, 15.76),
 ]
 
 
 # Bc, N, causal, blocks, pairs launched, 64-key (Bc = 128: 128-key) kernel, two-block kernel
 PAIRS = [
-    (64, 64, False, 160, 160, 6.13, 8.93), (64, 64, False, 224, 224, 6.49, 9.27), (64, 64, False, 294, 168, 6.60, 10.10),
-    (64, 64, True, 448, 448, 11.47, 14.89), (64, 64, True, 1200, 1200, 25.21, 30.06), (64, 64, False, 1200, 600, 23.25, 21.19),
-    (64, 128, False, 156, 104, 9.06, 9.73), (64, 128, False, 294, 168, 9.43, 13.34), (64, 128, False, 1200, 600, 37.61, 31.08),
-    (64, 128, True, 520, 520, 17.43, 20.39), (64, 320, False, 288, 160, 13.66, 19.46), (64, 320, True, 588, 308, 20.45, 24.74),
-    (64, 320, True, 528, 352, 20.19, 22.98), (64, 320, True, 1200, 600, 41.99, 38.32), (64, 384, False, 288, 192, 15.04, 21.61),
-    (64, 384, False, 900, 500, 44.60, 42.57), (64, 384, False, 588, 308, 27.10, 32.05), (64, 384, True, 1200, 800, 53.69, 47.12),
-    (64, 640, False, 520, 312, 36.93, 41.15), (64, 1024, True, 320, 160, 22.15, 26.58), (64, 1024, True, 576, 288, 35.15, 33.24),
-    (64, 1152, False, 288, 160, 29.77, 38.40), (64, 1152, False, 576, 320, 56.07, 64.35), (64, 1152, False, 864, 480, 83.32, 95.13),
-    (64, 4096, False, 1024, 512, 310.0, 322.9), (64, 8192, False, 1024, 512, 585.9, 615.7), (64, 8192, False, 2048, 1024, 1165.3, 1149.3),
-    (64, 4096, True, 1024, 512, 168.0, 165.7),
-    (128, 64, False, 448, 448, 18.46, 20.73), (128, 64, True, 1200, 1200, 36.83, 43.12), (128, 64, False, 608, 304, 22.01, 20.67),
-    (128, 128, False, 294, 168, 12.89, 14.41), (128, 128, False, 602, 344, 25.19, 20.67), (128, 128, True, 448, 224, 21.83, 17.08),
-    (128, 320, False, 288, 192, 19.42, 25.27), (128, 320, False, 588, 308, 33.07, 37.19), (128, 320, False, 600, 400, 41.08, 37.40),
-    (128, 1024, True, 320, 160, 29.10, 32.02), (128, 1024, False, 320, 160, 47.74, 56.95), (128, 1024, True, 576, 288, 43.87, 39.96),
-    (128, 1152, False, 288, 160, 36.27, 47.64), (128, 1152, False, 576, 320, 70.01, 80.49), (128, 2048, False, 256, 128, 56.10, 58.50),
-    (128, 768, False, 396, 198, 39.20, 47.68), (128, 1280, False, 1500, 750, 198.12, 178.88), (128, 2048, False, 736, 368, 132.83, 146.38),
+    (64, 64, False, 160, 160, 5.86, 8.23), (64, 64, False, 224, 224, 6.05, 8.45), (64, 64, False, 294, 168, 6.29, 9.32),
+    (64, 64, True, 448, 448, 10.87, 13.50), (64, 64, True, 1200, 1200, 24.01, 26.20),
+    (64, 64, False, 1200, 600, 22.08, 18.85), (64, 128, False, 156, 104, 8.58, 8.86),
+    (64, 128, False, 294, 168, 8.98, 12.21), (64, 128, False, 1200, 600, 37.11, 29.52),
+    (64, 128, True, 520, 520, 16.99, 18.62), (64, 320, False, 288, 160, 13.06, 17.30),
+    (64, 320, True, 588, 308, 19.75, 22.34), (64, 320, True, 528, 352, 19.62, 19.36),
+    (64, 320, True, 1200, 600, 40.34, 34.18), (64, 384, False, 288, 192, 13.79, 18.50),
+    (64, 384, False, 900, 500, 42.93, 37.83), (64, 384, False, 588, 308, 26.03, 28.37),
+    (64, 384, True, 1200, 800, 52.38, 42.67), (64, 640, False, 520, 312, 33.29, 33.15),
+    (64, 1024, True, 320, 160, 20.87, 23.16), (64, 1024, True, 576, 288, 33.23, 29.72),
+    (64, 1152, False, 288, 160, 26.50, 29.93), (64, 1152, False, 576, 320, 52.32, 54.53),
+    (64, 1152, False, 864, 480, 83.17, 87.40), (64, 4096, False, 1024, 512, 281.4, 296.9),
+    (64, 8192, False, 1024, 512, 525.4, 570.5), (64, 8192, False, 2048, 1024, 1063.9, 1016.4),
+    (64, 4096, True, 1024, 512, 167.5, 157.2), (128, 64, False, 448, 448, 18.14, 19.40),
+    (128, 64, True, 1200, 1200, 35.50, 39.50), (128, 64, False, 608, 304, 21.22, 19.56),
+    (128, 128, False, 294, 168, 12.41, 13.98), (128, 128, False, 602, 344, 24.28, 19.91),
+    (128, 128, True, 448, 224, 21.02, 16.54), (128, 320, False, 288, 192, 18.32, 23.45),
+    (128, 320, False, 588, 308, 31.75, 35.02), (128, 320, False, 600, 400, 38.69, 34.58),
+    (128, 1024, True, 320, 160, 28.15, 30.02), (128, 1024, False, 320, 160, 44.26, 48.44),
+    (128, 1024, True, 576, 288, 42.54, 37.02), (128, 1152, False, 288, 160, 33.98, 41.53),
+    (128, 1152, False, 576, 320, 65.40, 69.86), (128, 2048, False, 256, 128, 51.95, 54.08),
+    (128, 768, False, 396, 198, 37.00, 43.57), (128, 1280, False, 1500, 750, 207.7, 168.9),
+    (128, 2048, False, 736, 368, 128.3, 128.2),
+    # sizes that an earlier form of the rule, fitted to earlier kernels, sent to the slower side
+    (64, 320, False, 2304, 1536, 83.79, 73.79), (64, 1024, False, 224, 112, 28.29, 24.68),
+    (64, 2304, False, 288, 144, 53.22, 46.70), (64, 1152, False, 1512, 768, 153.5, 137.3),
+    (64, 384, True, 384, 192, 18.98, 16.97), (64, 512, True, 384, 192, 19.54, 16.38),
+    (64, 768, True, 420, 210, 25.24, 21.33), (64, 1152, True, 432, 224, 30.79, 26.58),
+    (64, 1664, True, 416, 224, 40.39, 35.43), (128, 320, False, 2304, 1536, 124.6, 105.8),
+    (128, 384, False, 768, 512, 50.16, 43.77), (128, 896, False, 672, 384, 71.48, 62.15),
+    (128, 1152, False, 1440, 800, 162.7, 144.7), (128, 192, True, 256, 128, 14.64, 12.37),
+    (128, 256, True, 320, 160, 18.50, 16.21), (128, 384, True, 360, 192, 22.02, 18.25),
+    (128, 512, True, 448, 224, 26.99, 22.83), (128, 896, True, 448, 224, 32.41, 28.88),
 ]
 PAIRS_QMEAN = [
-    (64, 768, False, 300, 150, 35.62, 43.11), (64, 768, False, 456, 228, 45.43, 44.25), (64, 2048, False, 896, 448, 165.25, 188.78),
-    (128, 768, False, 396, 198, 46.68, 54.34), (128, 768, False, 1044, 522, 114.71, 97.23), (128, 1280, False, 960, 480, 153.08, 143.45),
-    (128, 2048, False, 384, 192, 101.38, 114.06), (128, 2048, False, 608, 304, 166.23, 163.58),
+    (64, 768, False, 300, 150, 31.46, 36.61), (64, 768, False, 456, 228, 40.19, 38.34),
+    (64, 2048, False, 896, 448, 149.7, 161.8), (128, 768, False, 396, 198, 47.04, 47.78),
+    (128, 768, False, 1044, 522, 124.2, 84.50), (128, 1280, False, 960, 480, 163.4, 124.2),
+    (128, 2048, False, 384, 192, 96.13, 94.92), (128, 2048, False, 608, 304, 158.9, 138.7),
+    (64, 384, True, 360, 192, 20.66, 17.20), (64, 512, True, 384, 192, 21.67, 18.87),
+    (64, 1152, True, 432, 216, 33.99, 30.24), (128, 320, False, 1152, 768, 78.44, 66.43),
+    (128, 256, True, 208, 104, 16.42, 12.53), (128, 320, True, 330, 176, 21.69, 17.69),
+    (128, 384, True, 384, 192, 25.06, 21.20), (128, 768, True, 360, 180, 31.96, 28.15),
 ]
 
 
