@@ -155,7 +155,8 @@ typedef struct {
 const char* hifa4_status_string(int status);
 
 /* Self-test of the failure path of the device-side waits (no counterpart in the paper; for deployment
- * checks and for the test-suite).  Launches the Bc = 64, d = 128 attention kernel in an instantiation
+ * checks and for the test-suite).  Launches the Bc = 64, d = 128 attention kernel that a call with these
+ * arguments would take (the one with two query blocks per CTA for large problems) in an instantiation
  * whose softmax warps withhold the arrival that releases the P V product and whose issuer gives up
  * waiting for it after 2^6 polls (at most a fraction of a millisecond) instead of 2^18.  That wait begins
  * only when every TMA load has landed and no MMA is in flight.  When it runs out the kernel records
@@ -163,7 +164,7 @@ const char* hifa4_status_string(int status);
  * entry), raises the CTA's abort flag, every role leaves through the common exit that frees tensor memory, and
  * the call returns normally.
  * `out` is not written.  Arguments as hifa4_attention_fwd (prm: Bc = 64, no variant flags; shape: d = 128);
- * a one-CTA problem (N <= 128, one head) is what the test-suite uses.  Nothing hangs, faults or traps. */
+ * the test-suite uses a one-CTA problem (N <= 128, one head) and some with hundreds of CTAs.  Nothing hangs, faults or traps. */
 int hifa4_selftest_wait_timeout(const hifa4_shape* shape, const hifa4_qkv* qkv, const hifa4_attn_params* prm,
                                 void* out, int* d_status, void* stream);
 

@@ -400,7 +400,8 @@ def attention_fwd_f8qk(qkv: QuantizedQKV, causal: bool, out_dtype=F32, out=None,
 
 
 def selftest_wait_timeout(qkv: QuantizedQKV, causal: bool, d_status, out=None):
-    """Launches the self-test instantiation whose wait for P V runs out (see include/hifa4.h).  d_status: device
+    """Launches the self-test instantiation whose wait for P V runs out, of the kernel that attention_fwd would take (see
+    include/hifa4.h).  d_status: device
     int32 tensor (zero on entry); afterwards it holds HIFA4_ERR_TIMEOUT + 16 * 7.  Returns the (unwritten) out."""
     sh = _shape(qkv.B, qkv.Hq, qkv.Hkv, qkv.N, qkv.d, qkv.in_dtype, qkv.q_to_kv)
     prm = _params(causal, 64, F32)

@@ -428,9 +428,9 @@ int launch_attention(const hifa4_shape& sh, const HeadMap& map, const hifa4_qkv&
     }
     a.normalizer = prm.normalizer ? 1 : 0;
     a.p_f32 = prm.p_dtype == HIFA4_F32 ? 1 : 0;
-    if (selftest) {                               // the instantiation whose wait for P V runs out
+    if (selftest) {                               // the instantiation whose wait for P V runs out, of the kernel that a call would take
         if (a.p_f32 || a.normalizer || a.qmean || stats || dbg || prm.Bc != 64 || sh.d != 128) return HIFA4_ERR_UNSUPPORTED;
-        return launch_attention_ws64_selftest(sh, qkv, a, st);
+        return attention_pair_pays(sh, prm) ? launch_attention_pair_selftest(sh, qkv, a, st) : launch_attention_ws64_selftest(sh, qkv, a, st);
     }
     if (a.p_f32) {                                // variant built for the 64-key warp-specialised kernels only
         if (a.normalizer || stats || prm.Bc != 64 || (sh.d != 128 && sh.d != 256)) return HIFA4_ERR_UNSUPPORTED;

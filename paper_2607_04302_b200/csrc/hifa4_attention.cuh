@@ -447,7 +447,8 @@ int launch_attention_pair(const hifa4_shape& sh, const hifa4_qkv& qkv, const Att
 // The same on pairs of SMs, d = 256 (hifa4_attention_cta2.cu).
 bool attention_cta2_pays(const hifa4_shape& sh, const hifa4_attn_params& prm, int unit_heads);
 int launch_attention_cta2(const hifa4_shape& sh, const hifa4_qkv& qkv, const AttnArgs& args, cudaStream_t st);
-// Self-test instantiation (d = 128): one bounded wait is made to run out (see hifa4_selftest_wait_timeout).
+// Self-test instantiations (d = 128, Bc = 64): one bounded wait is made to run out (see hifa4_selftest_wait_timeout).
+int launch_attention_pair_selftest(const hifa4_shape& sh, const hifa4_qkv& qkv, const AttnArgs& args, cudaStream_t st);
 int launch_attention_ws64_selftest(const hifa4_shape& sh, const hifa4_qkv& qkv, const AttnArgs& args, cudaStream_t st);
 
 }  // namespace hifa4

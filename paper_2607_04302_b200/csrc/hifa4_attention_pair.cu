@@ -144,7 +144,11 @@ static __device__ __forceinline__ int launch_control_answer(uint32_t src)   // b
     return got ? (int)x : -1;
 }
 
-template <bool QM, bool B128>
+// SELFTEST: as in the 64-key kernel, the instantiation whose wait for P V runs out.  The softmax warps withhold the arrivals that
+// release P V; a CTA takes one pair only and two tiles of it at most, and the issuer first waits, with the full limit, until their
+// loads have landed, their S = Q K^T are complete and the launch control has answered: when its 2^6 polls begin, nothing is in
+// flight.  The softmax warps then leave through the abort exits of wait_warp and wait_long, the issuers of S through theirs.
+template <bool QM, bool B128, bool SELFTEST = false>
 __global__ void __launch_bounds__(PairCfg::THREADS, 1)
 attention_fwd_pair_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ CUtensorMap tmap_k,
                           const __grid_constant__ CUtensorMap tmap_v, const __grid_constant__ AttnArgs args)
@@ -239,7 +243,8 @@ attention_fwd_pair_kernel(const __grid_constant__ CUtensorMap tmap_q, const __gr
                     for (int hf = 0; hf < 2; ++hf) {
                         const int r = 2 * p + hf, qi = r / G, q0 = (n_qt - 1 - qi) * 128;
                         const int last_key = args.causal ? min(q0 + 127, N - 1) : N - 1;
-                        const int n = r >= blocks ? 0 : B128 ? 2 * (last_key / 128 + 1) : last_key / BC + 1;
+                        int n = r >= blocks ? 0 : B128 ? 2 * (last_key / 128 + 1) : last_key / BC + 1;
+                        if (SELFTEST) n = min(n, 2);
                         w.n[hf] = n;
                         w.q0[hf] = q0;
                         w.bh_q[hf] = b * args.Hq + h0 + (r - qi * G);
@@ -292,6 +297,7 @@ attention_fwd_pair_kernel(const __grid_constant__ CUtensorMap tmap_q, const __gr
                 }
                 if (!ok) break;
                 if (!wait_pair(bar(CL), (uint32_t)it & 1u, abort_flag)) { fail(17); break; }
+                if (SELFTEST) break;
                 idx = launch_control_answer(smem_base + CL_OFF);
             }
         }
@@ -405,7 +411,7 @@ attention_fwd_pair_kernel(const __grid_constant__ CUtensorMap tmap_q, const __gr
                 tmem_wait_st();
                 tc_fence_before();
                 __syncwarp();
-                arrive0(b_h + 8 * PGO, lane);
+                if (!SELFTEST) arrive0(b_h + 8 * PGO, lane);
             }
             if (!ok) break;
             t0 += n_tiles;
@@ -526,9 +532,17 @@ attention_fwd_pair_kernel(const __grid_constant__ CUtensorMap tmap_q, const __gr
             int it[2] = {0, 0}, jt[2] = {0, 0}, n_max[2] = {0, 0}, n_tiles[2] = {0, 0}, st[2] = {0, 0};
             uint32_t ph[2] = {0, 0}, t[2] = {0, 0}, no[2] = {0, 0};      // parities of the ring round, the tile and the block count
             bool first[2] = {true, true}, done[2] = {false, false}, armed[2] = {false, false};
+            constexpr uint32_t POLLS = SELFTEST ? 1u << 6 : 4 * WAIT_POLLS;
             uint32_t idle = 0;
+            if constexpr (SELFTEST) {
+                bool quiet = wait_pair(bar(WF), 0, abort_flag) && wait_pair(bar(CL), 0, abort_flag);
+                for (int j = 0; quiet && j < work[0].n_max; ++j) quiet = wait_pair(bar(VF + j), 0, abort_flag);
+                for (int hf = 0; hf < 2; ++hf)
+                    for (int j = 0; quiet && j < work[0].n[hf]; ++j) quiet = wait_pair(bar(hf * HALF + SF + j), 0, abort_flag);
+                if (!quiet) fail(2);
+            }
             while (!(done[0] && done[1])) {
-                if (++idle > 4 * WAIT_POLLS || ((idle & 63u) == 63u && ld_flag(abort_flag))) { if (idle > 4 * WAIT_POLLS) fail(7); break; }
+                if (++idle > POLLS || ((idle & 63u) == 63u && ld_flag(abort_flag))) { if (idle > POLLS) fail(7); break; }
 #pragma unroll
                 for (int hf = 0; hf < 2; ++hf) {
                     if (armed[hf]) {
@@ -584,7 +598,7 @@ attention_fwd_pair_kernel(const __grid_constant__ CUtensorMap tmap_q, const __gr
     }
 }
 
-template <bool QM, bool B128>
+template <bool QM, bool B128, bool SELFTEST = false>
 static int launch_pair(const hifa4_shape& sh, const hifa4_qkv& qkv, const AttnArgs& args, cudaStream_t st)
 {
     using C = PairCfg;
@@ -592,7 +606,7 @@ static int launch_pair(const hifa4_shape& sh, const hifa4_qkv& qkv, const AttnAr
     if (!make_bf16_map(&mq, qkv.q_mma, (uint64_t)sh.B * sh.Hq, sh.N, C::D, 128)) return HIFA4_ERR_CUDA;
     if (!make_bf16_map(&mk, qkv.k_mma, (uint64_t)sh.B * sh.Hkv, sh.N, C::D, C::BC)) return HIFA4_ERR_CUDA;
     if (!make_bf16_map(&mv, qkv.v_mma, (uint64_t)sh.B * sh.Hkv, C::D, sh.N, C::D)) return HIFA4_ERR_CUDA;
-    auto kern = attention_fwd_pair_kernel<QM, B128>;
+    auto kern = attention_fwd_pair_kernel<QM, B128, SELFTEST>;
     static SmemOptIn opt_in;
     if (!opt_in.ensure(kern, C::SMEM_BYTES)) return HIFA4_ERR_CUDA;
     const int blocks = (sh.N + 127) / 128 * args.unit_heads;
@@ -609,6 +623,11 @@ bool attention_pair_pays(const hifa4_shape& sh, const hifa4_attn_params& prm)
     const int G = heads_per_unit(sh);
     const long long unit_blocks = (long long)((sh.N + 127) / 128) * G, units = (long long)(sh.Hq / G) * sh.B;
     return two_blocks_faster(prm.Bc, sh.N, prm.causal != 0, prm.qmean != 0, unit_blocks * units, (unit_blocks + 1) / 2 * units, sms);
+}
+
+int launch_attention_pair_selftest(const hifa4_shape& sh, const hifa4_qkv& qkv, const AttnArgs& args, cudaStream_t st)
+{
+    return launch_pair<false, false, true>(sh, qkv, args, st);
 }
 
 int launch_attention_pair(const hifa4_shape& sh, const hifa4_qkv& qkv, const AttnArgs& args, int Bc, cudaStream_t st)

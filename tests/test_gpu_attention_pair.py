@@ -65,3 +65,27 @@ def test_two_block_kernel_with_128_key_tiles(B, Hq, Hkv, N, causal, qmean, head_
         assert torch.equal(hb.attention_fwd(qkv, causal, Bc=128, qmean=qmean, out_dtype=dt, d_status=status), ref)
     assert torch.equal(hb.attention_fwd_raw(q, k, v, None, None, causal, Bc=128, q_to_kv=head_map, qmean=qmean, d_status=status), want)
     assert int(status.item()) == 0
+
+
+@pytest.mark.parametrize("name", ["even-group", "odd-group-ragged-block", "odd-block-count", "one-tile", "two-tiles", "head-map"])
+def test_expired_wait_is_reported_and_leaves_the_device_usable(name):
+    """The self-test instantiation of this kernel (hifa4_selftest_wait_timeout takes the kernel that a call would take): the arrivals
+    that release P V are withheld, the issuer's wait runs out (site 7), the softmax warps' waits for P V see the abort flag, `out`
+    stays untouched and the next call gives the right values."""
+    from paper_2607_04302_b200 import binding as hb
+    B, Hq, Hkv, N, causal, _, head_map = CASES[name]
+    cfg = synth.config("C2", B=B, Hq=Hq, Hkv=Hkv, N=N, causal=causal)
+    q, k, v = synth.make_qkv_device(cfg, DEV)
+    qkv = hb.quantize_qkv(q, k, v, q_to_kv=head_map)
+    status = torch.zeros(1, dtype=torch.int32, device=DEV)
+    want, _ = hb.attention_fwd(qkv, causal, debug_blocks=[(0, 0, 0)], d_status=status)
+    assert int(status.item()) == 0
+    out = torch.full_like(want, 3.0)
+    hb.selftest_wait_timeout(qkv, causal, status, out=out)
+    torch.cuda.synchronize()
+    assert int(status.item()) == 6 + 16 * 7 and bool((out == 3.0).all())
+    hb.attention_fwd(qkv, causal, out=out, d_status=status)             # a set status word: nothing happens
+    assert bool((out == 3.0).all()) and int(status.item()) == 6 + 16 * 7
+    status.zero_()
+    hb.attention_fwd(qkv, causal, out=out, d_status=status)
+    assert torch.equal(out, want) and int(status.item()) == 0
