@@ -152,12 +152,12 @@ __device__ __forceinline__ float p_of_score(float acc, float c1, float mL)
 
 // Arithmetic of the fused form.  P is FP16, so the quantizer runs on packed FP16 pairs from the conversion on and
 // hands over a packed BF16 image: no widening back to FP32, no repacking.  The softmax warps are bound by instruction
-// issue and by the power the SM draws: against a quantizer that multiplied by one reciprocal split into two constants (a product
-// and an FMA per pair, then an addition; shift constants by five operations instead of three) the attention of 32 / 8 heads at
-// d = 128, causal, takes 142 instead of 152 us at N = 4096 and 504 instead of 539 at N = 8192 (B200, back to back, two-block
-// kernel).  In units of S/2:
-//   q = RN(p * c1)                  c1 * c2 = 2/S up to 7e-5, two FP16 factors per mantissa of S, c2 near 1 (one FP16 constant
-//   y = fma(q, c2, 2^(9+k))         errs by 2^-12, which is not enough).  The factors are chosen so that the rounding of q lands on
+// issue and by the power the SM draws, and two factors with one product and one FMA per pair are the fewest instructions found: one
+// reciprocal split into two constants (a product and an FMA per pair, then an addition; shift constants by five operations instead of
+// three) takes 152 instead of 142 us at 32 / 8 heads, d = 128, causal, N = 4096, and 539 instead of 504 at N = 8192 (B200, back to
+// back, two-block kernel before its waits by vote).  In units of S/2:
+//   q = RN(p * c1)                  c1 * c2 = 2/S up to 7e-5, two FP16 factors per mantissa of S, c2 = 2, 1.40, 0.74, 0.74 (one FP16
+//   y = fma(q, c2, 2^(9+k))         constant errs by 2^-12, which is not enough).  The factors are chosen so that the rounding of q lands on
 //                                   the side of a rounding tie on which p lies, and for p on the tie on the side of the even
 //                                   multiple: the FMA rounds p * 2/S to the nearest multiple of the subgroup's step, ties to
 //                                   even, exactly.  The low bits of y are the element code m
@@ -336,7 +336,7 @@ __device__ __forceinline__ void exp_quantize_units(const float (&acc)[NU * 8], c
     }
 }
 
-// Maximum of 64 values in 32 three-input maxima: seven chains of nine, then one chain over their results and the last value.
+// Maximum of 64 values in 31 three-input maxima and one of two: seven chains of nine, then their results and the last value.
 __device__ __forceinline__ float max64(const float (&p)[64])
 {
     float t[8];

@@ -3,12 +3,13 @@
 //
 // The two blocks ("halves") belong to query heads of one KV head, so every K and V^T tile is loaded once for 256
 // query rows instead of once for 128: with one block per CTA and two CTAs per SM the tiles cross L2 -> SM at 9 TB/s,
-// and leaving those loads out altogether made long launches 13-16 % shorter (the clocks of long launches follow the power
-// they draw).  Against that kernel, sustained, both with an earlier quantizer of P and earlier waits: 32 / 8 heads causal N = 2048 52 -> 48 us, N = 4096 168 -> 166, N = 16384 2.31 ->
-// 2.29 ms, B = 4 N = 2048 197 -> 187 us, N = 4096 681 -> 655, non-causal 1233 -> 1205; single calls on an idle chip, which do
-// not reach the power cap, are 1 to 4 % slower from N = 8192 up (since then this kernel alone gained 13 %: N = 4096 152 -> 132 us,
-// N = 8192 539 -> 469).  hifa4_dispatch.h says when it is taken.  d = 64 stays there (350 against 380 us, 12 / 4 heads, B = 2,
-// N = 8192: its tiles are half as large and its softmax share twice).  Apart from the
+// and leaving those loads out altogether made long launches of that kernel 13-16 % shorter (the clocks of long launches follow
+// the power they draw).  Against the 64-key kernel (sustained, us; two-block against 64-key): 32 / 32 heads, causal, N = 4096 157 against
+// 168, N = 8192 whole calls 580 against 606; not causal N = 8192, 2048 blocks 1016 against 1064.  It executes 10.3 instructions per 32
+// scores; of its 132 us at N = 4096 (32 / 8 heads, BF16 output) the quantizer of P with two factors, which all attention kernels
+// share, saved 10 and the waits by vote with the P V issuer's look-ahead, which only this kernel has, another 10.
+// hifa4_dispatch.h says when it is taken.  d = 64 stays with the 64-key kernel (350 against 380 us, 12 / 4 heads, B = 2, N = 8192,
+// both with an earlier quantizer: its tiles are half as large and its softmax share twice).  Apart from the
 // shared tiles the halves run independently of one another, each as the 64-key kernel (hifa4_attention_ws64.cu) runs a
 // CTA.  Warps:
 //   0-15   softmax / quantize: warps 8h..8h+3 own the even key tiles of half h, warps 8h+4..8h+7 the odd ones, one
@@ -25,7 +26,8 @@
 // through 2 KB of shared memory per warp, so that stores cover whole 64-byte row pieces.
 // Template flags: Q-Mean (key sums staged in eight slots by the loader, as in the 64-key kernel); B128: 128-key tiles, each a
 // pair of 64-key ones whose owners exchange their maxima (one more hand-off per tile, one rescale less).  Against the
-// 128-key kernel (hifa4_attention_ws.cu), 32 / 8 heads, causal: N = 4096 213 -> 191 us (158 now), N = 8192 722 -> 637.
+// 128-key kernel (hifa4_attention_ws.cu): 32 / 8 heads, causal, whole calls with an earlier quantizer, N = 4096 191 against 213 us, N =
+// 8192 637 against 722; causal, N = 1024, 576 blocks 37.0 against 42.5.
 // Every wait is bounded (see hifa4_attention_ws.cu for the failure protocol).
 #include "hifa4_attention.cuh"
 #include "hifa4_dispatch.h"
@@ -364,7 +366,8 @@ attention_fwd_pair_kernel(const __grid_constant__ CUtensorMap tmap_q, const __gr
 #pragma unroll
                     for (int i = 0; i < BC; ++i) p[i] = (j0 + i > key_lim) ? -INFINITY : p[i];
                 }
-                // (no instruction: unties the scores from the two blocks of 32 registers that the loads fill, or ptxas spills 48 bytes)
+                // (no instruction: unties the scores from the two blocks of 32 registers that the loads fill; without it ptxas spills 48
+                // bytes in the plain form, with it none there, and with Q-Mean or 128-key tiles still 8 to 12)
 #pragma unroll
                 for (int i = 0; i < BC; ++i) asm volatile("" : "+f"(p[i]));
                 const float mx = max64(p);                         // row maximum = maximum of the tile's single 64-key group
