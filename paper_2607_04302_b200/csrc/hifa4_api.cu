@@ -332,13 +332,14 @@ int hifa4_attention_fwd_raw(const hifa4_shape* shape, const void* q, const void*
     hifa4_qkv bufs;
     size_t used = qkv_layout(shape, prm->qmean, (char*)workspace, &bufs);
     if ((s == nullptr) != (inv_s == nullptr)) return HIFA4_ERR_INVALID_ARG;
-    // K and V here, Q inside the attention kernel: pays once the Q-hat image (written, then read) is large; measured
-    // on B200 at d = 128: -1 to -3 % of the two launches from 64k query rows up, slower below.  The kernel with two query
-    // blocks per CTA takes Q-hat; where it is the faster one, its sizes go through the quantizer.  Whole calls, that way against
-    // raw Q in the 64-key kernel: under sustained load within 2 % (32 / 8 heads, causal: N = 4096 185 and 185 us, 8192 641 and
-    // 646, 32768 8.93 and 8.99 ms, B = 4 N = 1024 78 and 76, N = 2048 223 and 226, N = 4096 724 and 739); single calls with the
-    // chip idle before them, N = 2048 75 and 83, B = 4 N = 4096 709 and 710, N = 8192 638 and 624, 32768 8.27 and 7.93 ms.
-    if (attention_qraw_supported(*shape, *prm) && !attention_pair_pays(*shape, *prm) && (long long)shape->B * shape->Hq * shape->N >= 65536) {
+    // K and V here, Q inside the attention kernel: saves the Q-hat image (written, then read), costs each block its quantization before
+    // the first S.  Whole calls at d = 128 where the two-block kernel, which takes Q-hat, is not the faster one (not causal, a poorly
+    // filled last wave), raw Q against Q-hat, us: sustained from 131072 query rows up -1 to -3 % (B = 8, 8 / 8 heads, N = 2048 187.3
+    // and 189.0; B = 4, 32 / 8, N = 1024 101.8 and 105.0), long rows within 1 %; 100000 to 131071 -1 to -2 % sustained but +1 to +5 % for
+    // single calls with the chip idle before them (B = 2, 32 / 8, N = 1728 139.4 and 141.0, single 166.6 and 162.2); fewer -2 to +3 %
+    // and +1 to +10 % (B = 8, 14 / 2, N = 768 57.8 and 56.0, single 82.5 and 75.0).  Two-block kernel against raw Q in the 64-key kernel,
+    // sustained: 32 / 8 heads, causal, N = 4096 167 and 174, 8192 580 and 603, 32768 8046 and 8356, B = 4 N = 1024 68 and 72.
+    if (attention_qraw_supported(*shape, *prm) && !attention_pair_pays(*shape, *prm) && (long long)shape->B * shape->Hq * shape->N >= 131072) {
         if ((rc = quantize_common(shape, nullptr, k, v, s, inv_s, &bufs, false, stream))) return rc;
         return hifa4_attention_fwd_qraw(shape, q, s, &bufs, prm, out, (char*)workspace + used, d_status, stream);
     }

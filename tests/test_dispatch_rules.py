@@ -118,6 +118,10 @@ def test_the_cases_of_the_gpu_tests_reach_the_kernels_they_name(rules):
         assert takes_pairs(64, B, Hq, Hkv, N, causal, qmean, head_map), name
     for B, Hq, Hkv, N, causal, qmean, head_map in params(pair.test_two_block_kernel_with_128_key_tiles, "B,"):
         assert takes_pairs(128, B, Hq, Hkv, N, causal, qmean, head_map), (B, Hq, N)
+    from tests.test_gpu_attention import RAW_CASES
+    for B, Hq, Hkv, N in RAW_CASES:
+        assert not takes_pairs(64, B, Hq, Hkv, N, False, False, None), (B, Hq, N)
+    assert [B * Hq * N >= 131072 for B, Hq, _, N in RAW_CASES] == [True, False]
     seen = set()
     for B, Hq, Hkv, N, causal, _, _ in params(groups.test_four_groups_are_bit_identical_to_two, "B,"):
         for d in (64, 128):

@@ -359,9 +359,8 @@ def test_in_kernel_query_quantization_is_bit_identical(hb, par, dtype, smooth, c
 
 
 def test_in_kernel_query_quantization_full_size_and_refusals(hb, par):
-    """The headline shape through hifa4_attention_fwd_raw (which quantizes K and V into the workspace and Q inside the
-    attention kernel from 64k query rows up) equals the two-call path; configurations the in-kernel quantizer was
-    not built for are refused without a launch."""
+    """The headline shape through hifa4_attention_fwd_raw and through hifa4_attention_fwd_qraw (Q quantized inside the attention
+    kernel) equals the two-call path; configurations the in-kernel quantizer was not built for are refused without a launch."""
     cfg = synth.config("C2")
     q, k, v = synth.make_qkv_device(cfg, DEV)
     s, inv_s = par.calibrate(cfg, DEV)
@@ -378,6 +377,20 @@ def test_in_kernel_query_quantization_full_size_and_refusals(hb, par):
     q6, k6, v6 = (t.to(DEV) for t in synth.make_qkv(c64))
     with pytest.raises(hb.Hifa4Error):
         hb.attention_fwd_qraw(q6, None, hb.quantize_qkv(None, k6, v6, Hq=1), True)
+
+
+# B, Hq, Hkv, N, not causal: Q quantized inside the attention kernel from 131072 query rows up (the first), and Q-hat below (the
+# second), where the kernel with two query blocks is not the faster one (tests/test_dispatch_rules.py)
+RAW_CASES = [(1, 32, 8, 4096), (8, 14, 2, 768)]
+
+
+@pytest.mark.parametrize("B, Hq, Hkv, N", RAW_CASES)
+def test_raw_call_equals_quantize_and_attention_on_both_ways_for_q(hb, par, B, Hq, Hkv, N):
+    cfg = synth.config("C2", B=B, Hq=Hq, Hkv=Hkv, N=N, causal=False)
+    q, k, v = synth.make_qkv_device(cfg, DEV)
+    s, inv_s = par.calibrate(cfg, DEV)
+    want = hb.attention_fwd(hb.quantize_qkv(q, k, v, s, inv_s), False)
+    assert torch.equal(hb.attention_fwd_raw(q, k, v, s, inv_s, False), want)
 
 
 def test_calls_are_capturable_in_a_cuda_graph_and_replay_bit_identically(hb, par):
